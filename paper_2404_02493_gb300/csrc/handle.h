@@ -184,9 +184,19 @@ int setup_check_fields(const double* k, const double* phi, int n, int ny, double
                        long long* bad_phi, cudaStream_t st);
 double setup_peclet(const double* k64, const double* phi64, const double* sig64, int n, int ny, int pitch, double h,
                     double omega, int bc, double* dscratch, cudaStream_t st);
-int setup_coarse_inverse(const double* k64, const double* phi64, const double* sig64, int n, int ny, int pitch,
-                         double h, double omega, int bc, double shift, int which, int adr_flags, void* inv, int single,
-                         cudaStream_t st);
+// One dense coarsest-level inverse: the Helmholtz (which = 0) or ADR (1)
+// operator of a level of ny rows of n nodes, into inv as complex FP64 or
+// (single) rounded to complex FP32.
+constexpr int MAX_COARSE_NODES = 1024;
+struct CoarseJob {
+    const double *k64, *phi64, *sig64;
+    int n, ny, pitch;
+    double h, omega, shift;
+    int bc, which, adr_flags;
+    void* inv;
+    int single;
+};
+int setup_coarse_inverses(const std::vector<CoarseJob>& jobs, cudaStream_t st);
 
 #define WADR_CHECK(x)                                                                   \
     do {                                                                                \

@@ -587,6 +587,7 @@ static int build(mg_handle* mh, const mg_instance* in, int ninst, cudaStream_t s
     std::vector<double> hs((size_t)S::SIZE * nslots, 0.0);
     double* dscr = (double*)H.alloc(64);
     int di = 0;
+    std::vector<CoarseJob> coarse_jobs;
     for (int b = 0; b < ninst; ++b) {
         InstHost& I = H.inst[b];
         for (int l = 1; l <= I.L; ++l) {
@@ -660,13 +661,14 @@ static int build(mg_handle* mh, const mg_instance* in, int ninst, cudaStream_t s
                 cheb_coeffs(lv.lam_max, lv.alpha, q, s + S::CHEB_C1, s + S::CHEB_C2);
             }
             if (l == I.L) {
-                int r = setup_coarse_inverse(lv.k64, lv.phi64, lv.sig64, lv.n, lv.ny, lv.pitch, lv.h, I.omega, I.bc,
-                                             p.shift, 0, 0, lv.inv_helm, prec == MG_PREC_MIXED, st);
-                if (r) return r;
+                CoarseJob job{lv.k64, lv.phi64, lv.sig64, lv.n, lv.ny, lv.pitch, lv.h, I.omega, p.shift, I.bc,
+                              0, 0, lv.inv_helm, prec == MG_PREC_MIXED};
+                coarse_jobs.push_back(job);
                 if (lv.inv_adr) {
-                    r = setup_coarse_inverse(lv.k64, lv.phi64, lv.sig64, lv.n, lv.ny, lv.pitch, lv.h, I.omega, I.bc,
-                                             p.shift, 1, I.adr_flags, lv.inv_adr, prec == MG_PREC_MIXED, st);
-                    if (r) return r;
+                    job.which = 1;
+                    job.adr_flags = I.adr_flags;
+                    job.inv = lv.inv_adr;
+                    coarse_jobs.push_back(job);
                 }
             }
             ++di;
@@ -694,16 +696,16 @@ static int build(mg_handle* mh, const mg_instance* in, int ninst, cudaStream_t s
                                        I.adr_flags, dscr, st);
                 d.fgs = (float)d.gs;
                 d.coarse = (l < I.L) ? di + 1 : -1;
-                if (l == I.L) {
-                    int r = setup_coarse_inverse(v.k64, v.phi64, v.sig64, v.n, v.ny, v.pitch, v.h, I.omega, I.bc,
-                                                 p.shift, 1, I.adr_flags, v.inv_adr, prec == MG_PREC_MIXED, st);
-                    if (r) return r;
-                }
+                if (l == I.L)
+                    coarse_jobs.push_back(CoarseJob{v.k64, v.phi64, v.sig64, v.n, v.ny, v.pitch, v.h, I.omega, p.shift,
+                                                    I.bc, 1, I.adr_flags, v.inv_adr, prec == MG_PREC_MIXED});
                 H.hdesc.push_back(d);
                 H.base_of[(size_t)di] = base;
                 ++di;
             }
     }
+    // the dense coarsest inverses of every instance, in one go
+    if ((rc = setup_coarse_inverses(coarse_jobs, st)) != MG_OK) return rc;
     // outer descriptors (FP64, level-1 geometry)
     if (p.outer == MG_OUTER_FGMRES) {
         H.fs = (double*)H.alloc(sizeof(double) * FS::SIZE * ninst);
