@@ -108,14 +108,16 @@ __global__ void __launch_bounds__(NT) k_fg_start(const __grid_constant__ KDesc A
         const double2 rv = __ldg(r + p);
         v0[p] = mk<TC>((TC)rv.x * inv, (TC)rv.y * inv);
     }
-    if (c.lb == 0 && threadIdx.x == 0 && threadIdx.y == 0) {
+    if (c.lb == 0) {
         double* f = d.fs;
-        for (int q = FS::H; q < FS::SIZE; ++q) f[q] = 0.0;
-        f[FS::G] = 1.0;
-        f[FS::J] = 0.0;
-        f[FS::JDONE] = 0.0;
-        f[FS::EST] = 1.0;
-        *d.est = (sc > 0) ? 1.0 : 0.0;
+        const int tid = threadIdx.x + threadIdx.y * blockDim.x;
+        for (int q = FS::H + tid; q < FS::SIZE; q += NT) f[q] = q == FS::G ? 1.0 : 0.0;
+        if (tid == 0) {
+            f[FS::J] = 0.0;
+            f[FS::JDONE] = 0.0;
+            f[FS::EST] = 1.0;
+            *d.est = (sc > 0) ? 1.0 : 0.0;
+        }
     }
 }
 
@@ -436,16 +438,96 @@ __device__ __forceinline__ void fg_lag_update(const cplx<TC>* __restrict__ sv, i
     }
 }
 
-// Apply the committed rotations 0..j-1 to col[0..j+1] (rows of column j).
-__device__ __forceinline__ void fg_rotate(const double* f, int j, double2* col) {
-    for (int q = 0; q < j; ++q) {
-        const double2 cs = sload2d(f, FS::CS + 2 * q), sn = sload2d(f, FS::SN + 2 * q);
-        const double2 a = col[q], b = col[q + 1];
-        col[q] = dadd(dmulc(cs, a), dmulc(sn, b));
-        col[q + 1] = dsub(dmul(cs, b), dmul(sn, a));
-    }
+// Sum of a double over the warp, the same value and order in every lane.
+__device__ __forceinline__ double warp_dsum(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+__device__ __forceinline__ double2 shfl_d2(double2 v, int src) {
+    return make_double2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
 }
 
+// The rotations 0..j-1 (lane q holds c_q, s_q) applied to a column whose row
+// q lane q holds (rows 0..j): the rotated row of each lane; lane j's result
+// (the carry) in every lane through `last`.  Only the carry recurrence
+// a <- c_q b_q+1 - s_q a is serial (two dependent FMAs per rotation, ~65 ns);
+// one thread walking the whole column took ~500 ns per rotation.
+__device__ __forceinline__ double2 fg_rotate_warp(int lane, int j, double2 row, double2 cs, double2 sn, double2& last) {
+    const double2 b = make_double2(__shfl_down_sync(0xffffffffu, row.x, 1), __shfl_down_sync(0xffffffffu, row.y, 1));
+    const double2 cb = dmul(cs, b);
+    double2 a = shfl_d2(row, 0), mine = row;
+    for (int q = 0; q < j; ++q) {
+        if (lane == q) mine = a;
+        const double2 t = shfl_d2(cb, q), s = shfl_d2(sn, q);
+        a = make_double2(fma(-s.x, a.x, fma(s.y, a.y, t.x)), fma(-s.x, a.y, fma(-s.y, a.x, t.y)));
+    }
+    last = a;
+    return lane < j ? dadd(dmulc(cs, mine), dmulc(sn, b)) : a;
+}
+
+// Sums over the block of nv per-thread values that put(k) stores at
+// red[k * NT + tid]; warp w sums values w, w + 8, ... (eight per lane, then
+// the warp tree) and lane 0 publishes the block's partial.  True in the block
+// that finishes last within its segment.
+template <typename TC>
+__device__ __forceinline__ bool fg_publish(const LevelDesc& d, const SegCtx& c, const cplx<TC>* red, int nv, int tid,
+                                           int* flag) {
+    __syncthreads();
+    const int lane = tid & 31;
+    for (int k = tid >> 5; k < nv; k += NT / 32) {
+        const cplx<TC>* v = red + k * NT + lane;
+        cplx<TC> s = v[0];
+#pragma unroll
+        for (int i = 1; i < NT / 32; ++i) s = cadd<TC>(s, v[32 * i]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            s.x += __shfl_down_sync(0xffffffffu, s.x, o);
+            s.y += __shfl_down_sync(0xffffffffu, s.y, o);
+        }
+        if (lane == 0) d.fpart[(long long)c.lb * NVL + k] = to_d(s);
+    }
+    __syncthreads();
+    if (tid == 0) {
+        __threadfence();
+        const unsigned prev = atomicAdd(&d.counter[2], 1u);
+        *flag = (prev == (unsigned)(c.nb - 1));
+    }
+    __syncthreads();
+    return *flag != 0;
+}
+// In the last block: the nv totals into tot (shared).  Value k belongs to gw
+// (32 or 64) consecutive threads' column; the NT / gw groups take the blocks
+// in turn and their sums are added in order.
+__device__ __forceinline__ void fg_totals(const LevelDesc& d, int nb, int nv, double2* tot, double2* grp, int tid) {
+    __threadfence();
+    const int gw = nv <= 32 ? 32 : 64, k = tid & (gw - 1), g = tid / gw, ng = NT / gw;
+    double2 s = make_double2(0.0, 0.0);
+    if (k < nv) {
+        const double2* p = d.fpart + k;
+#pragma unroll 8
+        for (int b = g; b < nb; b += ng) s = dadd(s, __ldcg(p + (long long)b * NVL));
+    }
+    grp[tid] = s;
+    __syncthreads();
+    if (tid < nv) {
+        double2 t = grp[tid];
+        for (int q = 1; q < ng; ++q) t = dadd(t, grp[q * gw + tid]);
+        tot[tid] = t;
+    }
+    if (tid == 0) d.counter[2] = 0u;
+    __syncthreads();
+}
+
+// Tail of a pass (the block sums, the last block's totals and the small dense
+// work): with every value summed by shuffle trees over all MAXR slots, one
+// thread storing the partials and one thread walking the Hessenberg column
+// from global memory it took 60 us (pass A) and 43 us (pass B) per iteration
+// whatever the grid; here the sums go through the stage memory (free once the
+// stream has ended), the previous iteration's scalars are loaded before the
+// stream starts, and one warp holds the column, a row per lane
+// (n = 127, event-bracketed: 65 -> 20 us and 48 -> 19 us; n = 4095, j = 12:
+// 447 -> 381 and 457 -> 409 us, 6.5 and 6.7 TB/s).
 template <typename TC, int PASS>
 __global__ void __launch_bounds__(NT, 1) k_fg_lag(const __grid_constant__ KDesc A, const Seg* __restrict__ Sg,
                                                   int nseg, FgGeom g, int vscale) {
@@ -453,24 +535,37 @@ __global__ void __launch_bounds__(NT, 1) k_fg_lag(const __grid_constant__ KDesc 
     TmaCarve cv(fg_raw);
     cplx<TC>* const stg0 = cv.take<cplx<TC>>(g.ns * (MAXR + 1) * g.pw);
     __shared__ LevelDesc d;
-    __shared__ double2 grp[4 * 64];
+    __shared__ double2 grp[NT];
     __shared__ double2 tot[NVL];
-    __shared__ cplx<TC> shT[8 * NVL];
     __shared__ cplx<TC> s1c[MAXR], hc[MAXR];
     __shared__ TC ibeta_sh;
     __shared__ int flag;
     __shared__ alignas(8) uint64_t bars[FG_MAXNS];
     SegCtx c = seg_begin(A, Sg, nseg, d);
     const int tid = threadIdx.x + threadIdx.y * blockDim.x;
-    const int jj = (int)d.fs[FS::J];
+    double* const f = d.fs;
+    const int jj = (int)f[FS::J];
     cplx<TC>* vj = kvec<TC>(d, jj);
     cplx<TC>* w = kvec<TC>(d, jj + 1);
+    // scalars of the earlier iterations, for the small dense work at the end
+    // (warp 0, lane = row): the pending column (PASS 0: j - 1, PASS 1: j), the
+    // committed rotations, gamma and the pending norm
+    const int jc = PASS == 0 ? jj - 1 : jj;
+    double2 hrow = make_double2(0.0, 0.0), cs = hrow, sn = hrow, gam = hrow;
+    double hnp = 0.0;
+    if (tid < MAXR && jc >= 0) {
+        hrow = sload2d(f, FS::H + 2 * (tid * MAXR + jc));
+        cs = sload2d(f, FS::CS + 2 * tid);
+        sn = sload2d(f, FS::SN + 2 * tid);
+        gam = sload2d(f, FS::G + 2 * jc);
+        hnp = f[FS::HN + jj];
+    }
     if (PASS == 1) {
         if (tid < MAXR) {
-            s1c[tid] = tid < jj ? mk<TC>((TC)d.fs[FS::CC + 2 * tid], (TC)d.fs[FS::CC + 2 * tid + 1]) : zero2<TC>();
-            hc[tid] = tid <= jj ? mk<TC>((TC)d.fs[FS::HC + 2 * tid], (TC)d.fs[FS::HC + 2 * tid + 1]) : zero2<TC>();
+            s1c[tid] = tid < jj ? mk<TC>((TC)f[FS::CC + 2 * tid], (TC)f[FS::CC + 2 * tid + 1]) : zero2<TC>();
+            hc[tid] = tid <= jj ? mk<TC>((TC)f[FS::HC + 2 * tid], (TC)f[FS::HC + 2 * tid + 1]) : zero2<TC>();
         }
-        if (tid == 0) ibeta_sh = (TC)(1.0 / d.fs[FS::BETA]);
+        if (tid == 0) ibeta_sh = (TC)(1.0 / f[FS::BETA]);
     }
     __syncthreads();
     cplx<TC> s1[MAXR], s2[MAXR], s3 = zero2<TC>();
@@ -479,7 +574,7 @@ __global__ void __launch_bounds__(NT, 1) k_fg_lag(const __grid_constant__ KDesc 
     TC nv = TC(0), nrm = TC(0);
     const TC ibeta = PASS == 1 ? ibeta_sh : TC(1);
     // vscale: the pending vector V_jj is still W1_{jj-1} (k_fg_prep left out)
-    const double hnv = (vscale && jj > 0) ? d.fs[FS::HN + jj] : 1.0;
+    const double hnv = (vscale && jj > 0) ? f[FS::HN + jj] : 1.0;
     const TC vinv = (TC)(hnv > 0 ? 1.0 / hnv : 0.0);
     const bool ok = fg_stream<TC>(d, c, jj, w, stg0, g, bars,
                                   [&](const cplx<TC>* sv, int PJ, int cnt, long long e0) {
@@ -490,117 +585,91 @@ __global__ void __launch_bounds__(NT, 1) k_fg_lag(const __grid_constant__ KDesc 
         });
     });
     if (!ok) return;
-    // block sums -> per-block partials -> the last block of the segment
-    cplx<TC> red[NVL];
-#pragma unroll
-    for (int q = 0; q < NVL; ++q) red[q] = zero2<TC>();
+    // the thread's values, [S1 (j) | S2 (j) | s3 | ||Vt||^2] or [||W1||^2],
+    // into the stage memory (2 MAXR + 2 values of NT threads fit a stage)
+    const int nval = PASS == 0 ? 2 * jj + 2 : 1;
+    cplx<TC>* const red = stg0;
     if (PASS == 0) {
 #pragma unroll
-        for (int q = 0; q < MAXR; ++q) {
-            red[q] = s1[q];
-            red[MAXR + q] = s2[q];
-        }
-        red[2 * MAXR] = s3;
-        red[2 * MAXR + 1] = mk<TC>(nv, TC(0));
+        for (int q = 0; q < MAXR; ++q)
+            if (q < jj) {
+                red[q * NT + tid] = s1[q];
+                red[(jj + q) * NT + tid] = s2[q];
+            }
+        red[2 * jj * NT + tid] = s3;
+        red[(2 * jj + 1) * NT + tid] = mk<TC>(nv, TC(0));
     } else {
-        red[0] = mk<TC>(nrm, TC(0));
+        red[tid] = mk<TC>(nrm, TC(0));
     }
-    block_sum<cplx<TC>, NVL>(red, shT);
-    if (tid == 0) {
-        for (int q = 0; q < NVL; ++q) d.fpart[(long long)c.lb * NVL + q] = to_d(red[q]);
-        __threadfence();
-        const unsigned prev = atomicAdd(&d.counter[2], 1u);
-        flag = (prev == (unsigned)(c.nb - 1));
-    }
-    __syncthreads();
-    if (!flag) return;
-    __threadfence();
-    {
-        // value k = tid % 64 (< NVL) of block group g = tid / 64 sums blocks g, g+4, ...;
-        // the 4 group sums are added in order
-        const int k = tid & 63, g = tid >> 6;
-        double2 sacc = make_double2(0.0, 0.0);
-        if (k < NVL)
-            for (int b = g; b < c.nb; b += 4) sacc = dadd(sacc, __ldcg(&d.fpart[(long long)b * NVL + k]));
-        grp[g * 64 + k] = sacc;
-        __syncthreads();
-        if (tid < NVL) {
-            double2 t = grp[tid];
-            for (int q = 1; q < 4; ++q) t = dadd(t, grp[q * 64 + tid]);
-            tot[tid] = t;
-        }
-        if (tid == 0) d.counter[2] = 0u;
-        __syncthreads();
-    }
-    if (tid != 0) return;
-    double* f = d.fs;
-    const int j = jj;
+    if (!fg_publish<TC>(d, c, red, nval, tid, &flag)) return;
+    fg_totals(d, c.nb, nval, tot, grp, tid);
+    if (tid >= 32) return;
+    const int j = jj, lane = tid;
+    const double2 zero = make_double2(0.0, 0.0);
     if (PASS == 0) {
-        double2 S1[MAXR], S2[MAXR];
-        double ss = 0.0;
-        for (int q = 0; q < j; ++q) {
-            S1[q] = tot[q];
-            S2[q] = tot[MAXR + q];
-            ss += dabs2(S1[q]);
-        }
-        const double2 s3d = tot[2 * MAXR];
-        const double nvd = tot[2 * MAXR + 1].x;
+        const double2 S1 = lane < j ? tot[lane] : zero, S2 = lane < j ? tot[j + lane] : zero;
+        const double2 s12 = dmulc(S1, S2);
+        const double ss = warp_dsum(dabs2(S1));
+        const double2 ps = make_double2(warp_dsum(s12.x), warp_dsum(s12.y));
         // V_0 comes normalised from the restart; later vectors lose their projections
-        const double b2 = j == 0 ? 1.0 : nvd - ss;
+        const double b2 = j == 0 ? 1.0 : tot[2 * j + 1].x - ss;
         const double beta = b2 > 0.0 ? sqrt(b2) : 1e-300;
         if (j >= 1) {
             // column j-1 final: rows q < j gain ||W1_{j-1}|| S1_q, row j is ||W1_{j-1}|| beta
-            const double hn = f[FS::HN + j];
-            double2 col[MAXR + 1];
-            for (int q = 0; q < j; ++q) col[q] = dadd(sload2d(f, FS::H + 2 * (q * MAXR + (j - 1))), dsc(S1[q], hn));
-            col[j] = make_double2(hn * beta, 0.0);
-            fg_rotate(f, j - 1, col);
-            const double2 a = col[j - 1], b = col[j];
-            const double den = sqrt(dabs2(a) + dabs2(b));
-            double2 cs = make_double2(1, 0), sn = make_double2(0, 0);
+            const double hn = __shfl_sync(0xffffffffu, hnp, 0);
+            const double2 row = dadd(hrow, dsc(S1, hn));
+            double2 a;
+            const double2 rot = fg_rotate_warp(lane, j - 1, row, cs, sn, a);
+            const double b = hn * beta;
+            const double den = sqrt(dabs2(a) + b * b);
+            double2 csj = make_double2(1, 0), snj = zero;
             if (den > 0) {
-                cs = dsc(a, 1.0 / den);
-                sn = dsc(b, 1.0 / den);
+                const double r = 1.0 / den;
+                csj = dsc(a, r);
+                snj = make_double2(b * r, 0.0);
             }
-            sstore2d(f, FS::CS + 2 * (j - 1), cs);
-            sstore2d(f, FS::SN + 2 * (j - 1), sn);
-            col[j - 1] = make_double2(den, 0);
-            for (int q = 0; q < j; ++q) sstore2d(f, FS::H + 2 * (q * MAXR + (j - 1)), col[q]);
-            const double2 gj = sload2d(f, FS::G + 2 * (j - 1));
-            sstore2d(f, FS::G + 2 * j, dsc(dmul(sn, gj), -1.0));
-            sstore2d(f, FS::G + 2 * (j - 1), dmulc(cs, gj));
+            if (lane < j) sstore2d(f, FS::H + 2 * (lane * MAXR + (j - 1)), lane == j - 1 ? make_double2(den, 0) : rot);
+            if (lane == 0) {
+                sstore2d(f, FS::CS + 2 * (j - 1), csj);
+                sstore2d(f, FS::SN + 2 * (j - 1), snj);
+                sstore2d(f, FS::G + 2 * j, dsc(dmul(snj, gam), -1.0));
+                sstore2d(f, FS::G + 2 * (j - 1), dmulc(csj, gam));
+            }
         }
         // column j, rows 0..j (pending until step j+1): h_q = S2_q, h_j = (s3 - S1^H S2) / beta
-        double2 hj = s3d;
-        for (int q = 0; q < j; ++q) hj = dsub(hj, dmulc(S1[q], S2[q]));
-        hj = dsc(hj, 1.0 / beta);
-        for (int q = 0; q < j; ++q) {
-            sstore2d(f, FS::HC + 2 * q, S2[q]);
-            sstore2d(f, FS::CC + 2 * q, S1[q]);
-            sstore2d(f, FS::H + 2 * (q * MAXR + j), S2[q]);
+        if (lane < j) {
+            sstore2d(f, FS::HC + 2 * lane, S2);
+            sstore2d(f, FS::CC + 2 * lane, S1);
+            sstore2d(f, FS::H + 2 * (lane * MAXR + j), S2);
         }
-        sstore2d(f, FS::HC + 2 * j, hj);
-        sstore2d(f, FS::H + 2 * (j * MAXR + j), hj);
-        f[FS::BETA] = beta;
+        if (lane == 0) {
+            const double2 hj = dsc(dsub(tot[2 * j], ps), 1.0 / beta);
+            sstore2d(f, FS::HC + 2 * j, hj);
+            sstore2d(f, FS::H + 2 * (j * MAXR + j), hj);
+            f[FS::BETA] = beta;
+        }
     } else {
         const double hn = sqrt(tot[0].x);
-        f[FS::HN + j + 1] = hn;
-        sstore2d(f, FS::H + 2 * ((j + 1) * MAXR + j), make_double2(hn, 0.0));
         // provisional rotation of the pending column j: the residual estimate
-        double2 col[MAXR + 1];
-        for (int q = 0; q <= j; ++q) col[q] = sload2d(f, FS::H + 2 * (q * MAXR + j));
-        col[j + 1] = make_double2(hn, 0.0);
-        fg_rotate(f, j, col);
-        const double den = sqrt(dabs2(col[j]) + hn * hn);
-        const double est = den > 0 ? hn / den * sqrt(dabs2(sload2d(f, FS::G + 2 * j))) : 0.0;
-        f[FS::EST] = est;
-        f[FS::J] = j + 1;
-        f[FS::JDONE] = j + 1;
-        *d.est = est;
+        double2 a;
+        fg_rotate_warp(lane, j, hrow, cs, sn, a);
+        if (lane == 0) {
+            f[FS::HN + j + 1] = hn;
+            sstore2d(f, FS::H + 2 * ((j + 1) * MAXR + j), make_double2(hn, 0.0));
+            const double den = sqrt(dabs2(a) + hn * hn);
+            const double est = den > 0 ? hn / den * sqrt(dabs2(gam)) : 0.0;
+            f[FS::EST] = est;
+            f[FS::J] = j + 1;
+            f[FS::JDONE] = j + 1;
+            *d.est = est;
+        }
     }
 }
 
-// y = R^{-1} gamma (one thread per instance), then u += ||r|| sum_i y_i Z_i.
+// y = R^{-1} gamma, then u += ||r|| sum_i y_i Z_i.  Every block solves the
+// (tiny) triangular system in one warp, a row per lane with R staged in shared
+// memory and the diagonal inverted up front (one thread reading R from global
+// memory term by term took 150 us at m = 20).
 // LAG (two-pass scheme): the last column is still pending (unrotated); it
 // enters with its provisional rotation.
 template <typename TC, bool LAG>
@@ -608,31 +677,38 @@ __global__ void __launch_bounds__(NT) k_fg_update(const __grid_constant__ KDesc 
                                                   int nseg) {
     __shared__ LevelDesc d;
     __shared__ double2 ysh[MAXR];
+    __shared__ double2 Rsh[MAXR * MAXR];   // [column][row]
     SegCtx c = seg_begin(A, Sg, nseg, d);
     const int tid = threadIdx.x + threadIdx.y * blockDim.x;
-    const int m = (int)d.fs[FS::JDONE];
-    if (tid == 0) {
-        // every block solves the (tiny) triangular system redundantly
-        const double* f = d.fs;
-        double2 rl[MAXR + 1];
-        double2 gl = m > 0 ? sload2d(f, FS::G + 2 * (m - 1)) : make_double2(0, 0);
-        if (LAG && m > 0) {
-            for (int q = 0; q <= m; ++q) rl[q] = sload2d(f, FS::H + 2 * (q * MAXR + (m - 1)));
-            fg_rotate(f, m - 1, rl);
-            const double2 a = rl[m - 1], b = rl[m];
-            const double den = sqrt(dabs2(a) + dabs2(b));
-            const double2 cs = den > 0 ? dsc(a, 1.0 / den) : make_double2(1, 0);
-            rl[m - 1] = make_double2(den, 0);
-            gl = dmulc(cs, gl);
+    const double* f = d.fs;
+    const int m = (int)f[FS::JDONE];
+    for (int e = tid; e < m * m; e += NT) {
+        const int q = e / m, r = e - q * m;
+        if (q <= r) Rsh[r * MAXR + q] = sload2d(f, FS::H + 2 * (q * MAXR + r));
+    }
+    __syncthreads();
+    if (tid < 32 && m > 0) {
+        const int lane = tid;
+        const double2 zero = make_double2(0.0, 0.0);
+        double2 acc = lane < m ? sload2d(f, FS::G + 2 * lane) : zero;
+        if (LAG) {
+            const double2 cs = lane < m ? sload2d(f, FS::CS + 2 * lane) : zero;
+            const double2 sn = lane < m ? sload2d(f, FS::SN + 2 * lane) : zero;
+            const double2 bm = sload2d(f, FS::H + 2 * (m * MAXR + (m - 1)));
+            double2 a;
+            const double2 rot = fg_rotate_warp(lane, m - 1, lane < m ? Rsh[(m - 1) * MAXR + lane] : zero, cs, sn, a);
+            const double den = sqrt(dabs2(a) + dabs2(bm));
+            const double2 cl = den > 0 ? dsc(a, 1.0 / den) : make_double2(1, 0);
+            if (lane < m) Rsh[(m - 1) * MAXR + lane] = lane == m - 1 ? make_double2(den, 0) : rot;
+            if (lane == m - 1) acc = dmulc(cl, acc);
+            __syncwarp();
         }
-        auto Rq = [&](int q, int r) {
-            return (LAG && r == m - 1) ? rl[q] : sload2d(f, FS::H + 2 * (q * MAXR + r));
-        };
+        const double2 rqq = lane < m ? Rsh[lane * MAXR + lane] : zero;
+        const double2 rinv = dabs2(rqq) > 0 ? ddiv(make_double2(1.0, 0.0), rqq) : zero;
         for (int q = m - 1; q >= 0; --q) {
-            double2 acc = (q == m - 1) ? gl : sload2d(f, FS::G + 2 * q);
-            for (int r = q + 1; r < m; ++r) acc = dsub(acc, dmul(Rq(q, r), ysh[r]));
-            const double2 rqq = Rq(q, q);
-            ysh[q] = dabs2(rqq) > 0 ? ddiv(acc, rqq) : make_double2(0, 0);
+            const double2 y = shfl_d2(dmul(acc, rinv), q);
+            if (lane < q) acc = dsub(acc, dmul(Rsh[q * MAXR + lane], y));
+            if (lane == q) ysh[q] = y;
         }
     }
     __syncthreads();
