@@ -12,8 +12,8 @@
 // decreases the values to the same fixed point (Zhao's fast sweeping does it
 // by Gauss-Seidel sweeps in four orderings over the whole grid).
 //
-// GB300 layout: the grid is cut into 32 x 32 tiles; one warp owns a tile in
-// shared memory with a one-node halo and runs the four directional
+// GB300 layout: the grid is cut into 32 x 32 tiles; one warp (a block of its
+// own) owns a tile in shared memory with a one-node halo and runs directional
 // Gauss-Seidel sweeps inside it, one anti-diagonal per step (the 32 lanes
 // update the nodes of a diagonal together; they depend only on the previous
 // diagonal).  A pass runs every tile whose own values or a neighbour tile's
@@ -22,10 +22,24 @@
 // global memory while neighbours may be writing it: any value read is an
 // upper bound of the fixed point, so the monotone iteration is unaffected,
 // and a tile whose neighbour changed runs again in the next pass.
+//
+// What bounds it: the dependent updates along the front (n / 2 diagonals or
+// more from the source to the far corner, each a chain of FP64 operations of
+// ~32 ns and a square root); neither bandwidth nor the number of tiles.  So a
+// visit does only the sweeps that can change something: the nodes that would
+// decrease (at first only the tile's edge nodes can, after a sweep all are
+// looked at, which is a pipelined pass and not a chain) vote for the ordering
+// their information comes from, the ordering with most
+// votes is swept, and so on until no node votes.  Mostly that is one sweep
+// where four orderings, twice, were swept before; the chain of an update is
+// shortened by integer comparisons, one fused multiply-add per sum and a
+// Goldschmidt square root, and nothing is read from global memory inside it.
+// n = 2047, layered medium: 738 -> 155 us per pass, 59.8 -> 12.4 ms per call.
 #include <cuda_runtime.h>
 
 #include <cmath>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -34,116 +48,216 @@
 namespace wadr {
 
 constexpr int ET = 32;          // tile side (nodes)
-constexpr int EW = 4;           // warps (tiles) per block
+constexpr int EBATCH = 8;       // passes between two looks of the host
+constexpr int EMAXS = 32;       // sweeps of one visit; a tile that needs more goes on in the next pass
 constexpr double EINF = 1e300;
 
-// Source initialisation: tau = s(x0) |x - x0| within r_init, inf elsewhere;
-// fixed[p] = 1 on those nodes.  Products and sums rounded separately (no
-// contraction), as the host generator and the oracle evaluate them.
-__global__ void k_eik_init(int n, int ny, double h, const double* __restrict__ s, double x0, double y0,
-                           double r_init, int i0, int j0, double* __restrict__ tau, unsigned char* __restrict__ fixed) {
+// The nodes fixed by the source: within r_init of (x0, y0), inside the index
+// box [i0, i1] x [j0, j1] (a margin of one node around the disc), at
+// s0 |x - x0|, s0 = s at node (is, js).
+struct EikSrc {
+    double x0, y0, r_init;
+    int i0, i1, j0, j1;
+    int is, js;
+};
+
+// distance of node (i, j) from the source, products and sums rounded
+// separately (no contraction), as the host generator and the oracle evaluate
+// them
+__device__ __forceinline__ double src_dist(const EikSrc& c, double h, int i, int j) {
+    const double dx = __dsub_rn(__dmul_rn((double)(i + 1), h), c.x0);
+    const double dy = __dsub_rn(__dmul_rn((double)(j + 1), h), c.y0);
+    return sqrt(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)));
+}
+__device__ __forceinline__ bool in_box(const EikSrc& c, int i, int j) {
+    return i >= c.i0 && i <= c.i1 && j >= c.j0 && j <= c.j1;
+}
+
+// tau = s(x0) |x - x0| on the fixed nodes, inf elsewhere (a plain fill: the
+// distance is formed inside the box only; with a square root per node the
+// FP64 pipes took 154 us at n = 2047)
+__global__ void k_eik_init(int n, int ny, double h, const double* __restrict__ s, EikSrc c, double* __restrict__ tau) {
     const long long N = (long long)n * ny;
-    const double s0 = s[(long long)j0 * n + i0];
     for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < N; p += (long long)gridDim.x * blockDim.x) {
         const int i = (int)(p % n), j = (int)(p / n);
-        const double dx = __dsub_rn(__dmul_rn((double)(i + 1), h), x0);
-        const double dy = __dsub_rn(__dmul_rn((double)(j + 1), h), y0);
-        const double r = sqrt(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)));
-        const bool fx = r <= r_init;
-        fixed[p] = fx ? 1 : 0;
-        tau[p] = fx ? __dmul_rn(s0, r) : EINF;
+        double v = EINF;
+        if (in_box(c, i, j)) {
+            const double r = src_dist(c, h, i, j);
+            if (r <= c.r_init) v = __dmul_rn(s[(long long)c.js * n + c.is], r);
+        }
+        tau[p] = v;
     }
 }
 
-// Godunov update from the smaller neighbour in x (a) and in y (b), f = s h.
-__device__ __forceinline__ double godunov_upd(double a, double b, double f) {
-    const double d = __dsub_rn(a, b);
-    if (!(fabs(d) < f)) return __dadd_rn(fmin(a, b), f);   // one-sided (also an infinite neighbour)
-    const double rad = __dsub_rn(__dmul_rn(__dmul_rn(2.0, f), f), __dmul_rn(d, d));
-    return __dmul_rn(0.5, __dadd_rn(__dadd_rn(a, b), sqrt(rad)));
+// Square root of a normal x well inside the exponent range: Goldschmidt's
+// coupled iteration for sqrt(x) and 1/(2 sqrt(x)) from an approximate
+// reciprocal square root, and one residual correction (five dependent
+// operations after the seed; the seed's ~20 bits square twice).
+__device__ __forceinline__ double sqrt_gs(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    double g = x * y, h = 0.5 * y;
+    const double r = fma(-g, h, 0.5);
+    g = fma(g, r, g);
+    h = fma(h, r, h);
+    return fma(fma(-g, g, x), h, g);
+}
+
+// Order of two values.  FAST: both are >= 0 (or +inf, NaN last), where
+// doubles order like their bits and an integer comparison takes a few
+// instructions; else the FP64 comparison (~32 ns).
+template <bool FAST> __device__ __forceinline__ bool dlt(double a, double b) {
+    return FAST ? __double_as_longlong(a) < __double_as_longlong(b) : a < b;
+}
+template <bool FAST> __device__ __forceinline__ double dmin2(double a, double b) { return dlt<FAST>(b, a) ? b : a; }
+
+// Godunov update from the smaller neighbour in x (a) and in y (b), f = s h:
+// one-sided where |a - b| >= f (also with an infinite neighbour).  FAST:
+// values >= 0 and f inside the range of sqrt_gs; without branches, so that
+// independent updates overlap.
+template <bool FAST> __device__ __forceinline__ double godunov_upd(double a, double b, double f) {
+    const double d = a - b;
+    const double one = dmin2<FAST>(a, b) + f;
+    const double rad = fma(-d, d, (2.0 * f) * f);
+    const double two = fma(0.5, FAST ? sqrt_gs(rad) : sqrt(rad), 0.5 * (a + b));
+    return dlt<FAST>(fabs(d), f) ? two : one;
 }
 
 // One pass over the active tiles (see the file comment).  act_in[t] != 0:
-// tile t changed in the previous pass; act_out[t] is set when it changes in
-// this one and *nchanged counts such tiles.
-__global__ void __launch_bounds__(32 * EW) k_eik_pass(int n, int ny, double h, const double* __restrict__ s,
-                                                      const unsigned char* __restrict__ fixed, double* tau,
-                                                      const unsigned char* __restrict__ act_in,
-                                                      unsigned char* __restrict__ act_out, unsigned* nchanged,
-                                                      double tol, int reps) {
-    __shared__ double Ts[EW][ET + 2][ET + 2];
-    const int lane = threadIdx.x, w = threadIdx.y;
+// tile t changed in the previous pass (2: all its nodes are to be looked at);
+// act_out[t] is set when it changes in this one and *nchanged counts such
+// tiles; act_clr is the next pass's act_out.
+__global__ void __launch_bounds__(32) k_eik_pass(int n, int ny, double h, const double* __restrict__ s, EikSrc src,
+                                                 double* tau, const unsigned char* __restrict__ act_in,
+                                                 unsigned char* __restrict__ act_out,
+                                                 unsigned char* __restrict__ act_clr, unsigned* nchanged, double tol) {
+    // odd distances between the nodes of a diagonal (in 8-byte banks): no conflicts
+    __shared__ double T[ET + 2][ET + 2];
+    __shared__ double Fs[ET][ET];
+    const int lane = threadIdx.x;
     const int ntx = (n + ET - 1) / ET, nty = (ny + ET - 1) / ET;
-    const int t = blockIdx.x * EW + w;
-    if (t >= ntx * nty) return;
-    const int tx = t % ntx, ty = t / ntx;
-    bool active = act_in[t] != 0;
-    if (!active) {
-        active = (tx > 0 && act_in[t - 1]) || (tx < ntx - 1 && act_in[t + 1]) || (ty > 0 && act_in[t - ntx]) ||
-                 (ty < nty - 1 && act_in[t + ntx]);
-    }
-    if (!active) return;                      // warp-uniform
-    double (*T)[ET + 2] = Ts[w];
-    const int gx0 = tx * ET, gy0 = ty * ET;
-    auto G = [&](int gi, int gj) -> double {
-        return (gi >= 0 && gi < n && gj >= 0 && gj < ny) ? __ldcg(&tau[(long long)gj * n + gi]) : EINF;
-    };
-    // interior and halo rows (lane = column), halo columns (lane = row)
-    for (int r = -1; r <= ET; ++r) T[r + 1][lane + 1] = G(gx0 + lane, gy0 + r);
-    T[lane + 1][0] = G(gx0 - 1, gy0 + lane);
-    T[lane + 1][ET + 1] = G(gx0 + ET, gy0 + lane);
-    if (lane == 0) {
-        T[0][0] = EINF;
-        T[0][ET + 1] = EINF;
-        T[ET + 1][0] = EINF;
-        T[ET + 1][ET + 1] = EINF;
-    }
-    __syncwarp();
-    bool changed = false;
-    for (int rep = 0; rep < reps; ++rep) {
-        bool chg_rep = false;
-        for (int dir = 0; dir < 4; ++dir) {
-            const bool fwx = (dir & 1) == 0, fwy = (dir & 2) == 0;
-            for (int u = 0; u < 2 * ET - 1; ++u) {
-                const int ii = lane, jj = u - lane;
-                if (jj >= 0 && jj < ET) {
-                    const int i = fwx ? ii : ET - 1 - ii, j = fwy ? jj : ET - 1 - jj;
-                    const int gi = gx0 + i, gj = gy0 + j;
-                    if (gi < n && gj < ny) {
-                        const long long p = (long long)gj * n + gi;
-                        if (!fixed[p]) {
-                            const double a = fmin(T[j + 1][i], T[j + 1][i + 2]);
-                            const double b = fmin(T[j][i + 1], T[j + 2][i + 1]);
-                            if (a < EINF || b < EINF) {
-                                const double cur = T[j + 1][i + 1];
-                                const double v = godunov_upd(a, b, __dmul_rn(__ldg(&s[p]), h));
-                                if (v < cur) {
-                                    if (cur >= EINF || __dsub_rn(cur, v) > tol) chg_rep = true;
-                                    T[j + 1][i + 1] = v;
-                                }
-                            }
-                        }
-                    }
-                }
-                __syncwarp();
+    for (int t = blockIdx.x; t < ntx * nty; t += gridDim.x) {
+        const int tx = t % ntx, ty = t / ntx;
+        const int self = act_in[t];
+        const bool active = self || (tx > 0 && act_in[t - 1]) || (tx < ntx - 1 && act_in[t + 1]) ||
+                            (ty > 0 && act_in[t - ntx]) || (ty < nty - 1 && act_in[t + ntx]);
+        if (lane == 0) act_clr[t] = 0;
+        if (!active) continue;                      // warp-uniform
+        const int gx0 = tx * ET, gy0 = ty * ET;
+        auto G = [&](int gi, int gj) -> double {
+            return (gi >= 0 && gi < n && gj >= 0 && gj < ny) ? __ldcg(&tau[(long long)gj * n + gi]) : EINF;
+        };
+        // interior and halo rows (lane = column), halo columns (lane = row);
+        // upd: the column's nodes that are in the grid and not fixed
+        unsigned upd = 0;
+#pragma unroll 8
+        for (int r = -1; r <= ET; ++r) T[r + 1][lane + 1] = G(gx0 + lane, gy0 + r);
+        T[lane + 1][0] = G(gx0 - 1, gy0 + lane);
+        T[lane + 1][ET + 1] = G(gx0 + ET, gy0 + lane);
+        const bool near = gx0 <= src.i1 && gx0 + ET > src.i0 && gy0 <= src.j1 && gy0 + ET > src.j0;
+#pragma unroll 8
+        for (int r = 0; r < ET; ++r) {
+            const int gi = gx0 + lane, gj = gy0 + r;
+            const bool in = gi < n && gj < ny;
+            Fs[r][lane] = in ? __dmul_rn(__ldg(&s[(long long)gj * n + gi]), h) : 0.0;
+            if (in) upd |= 1u << r;
+        }
+        if (near)
+            for (int r = 0; r < ET; ++r) {
+                const int gi = gx0 + lane, gj = gy0 + r;
+                if (in_box(src, gi, gj) && src_dist(src, h, gi, gj) <= src.r_init) upd &= ~(1u << r);
             }
+        const unsigned updr = __shfl_sync(0xffffffffu, upd, ET - 1 - lane);   // of column 31 - lane
+        __syncwarp();
+        bool fast = true;
+#pragma unroll 8
+        for (int r = 0; r < ET; ++r)
+            fast = fast && T[r + 1][lane + 1] >= 0.0 && (!((upd >> r) & 1) || (Fs[r][lane] > 1e-140 && Fs[r][lane] < 1e140));
+        fast = fast && T[0][lane + 1] >= 0.0 && T[ET + 1][lane + 1] >= 0.0 && T[lane + 1][0] >= 0.0 &&
+               T[lane + 1][ET + 1] >= 0.0;
+        fast = __all_sync(0xffffffffu, fast);
+        unsigned left;
+        auto visit = [&](auto fc) -> bool {
+            constexpr bool FAST = decltype(fc)::value;
+            bool big = false;
+            // vote of node (i, j), if it would decrease: one byte counter per
+            // ordering (bit 0: information from the east, bit 1: from the
+            // north).  A decrease that rounding alone can make (two ulp) does
+            // not vote unless tol is smaller still; one above tol counts as
+            // a change of the tile.
+            auto look = [&](int i, int j, bool ok) -> unsigned {
+                const double w = T[j + 1][i], e = T[j + 1][i + 2], so = T[j][i + 1], no = T[j + 2][i + 1];
+                const bool fe = dlt<FAST>(e, w), fn = dlt<FAST>(no, so);
+                const double a = fe ? e : w, b = fn ? no : so;
+                const double cur = T[j + 1][i + 1], v = godunov_upd<FAST>(a, b, Fs[j][i]);
+                const double dec = cur - v;
+                ok = ok && dlt<FAST>(dmin2<FAST>(a, b), EINF) && dlt<FAST>(v, cur);
+                const bool over = ok && (cur >= EINF || dec > tol);
+                big = big || over;
+                return over || (ok && dec > 4.5e-16 * cur) ? 1u << (8 * ((fe ? 1 : 0) + (fn ? 2 : 0))) : 0u;
+            };
+            auto look_all = [&]() -> unsigned {
+                unsigned v = 0;
+#pragma unroll 8
+                for (int r = 0; r < ET; ++r) v += look(lane, r, (upd >> r) & 1);
+                return v;
+            };
+            unsigned votes;
+            if (self == 2) {
+                votes = look_all();
+            } else {
+                // the interior was at rest for the halo of its last visit
+                const unsigned c0 = __shfl_sync(0xffffffffu, upd, 0), c1 = __shfl_sync(0xffffffffu, upd, ET - 1);
+                votes = look(lane, 0, upd & 1) + look(lane, ET - 1, upd >> (ET - 1)) + look(0, lane, (c0 >> lane) & 1) +
+                        look(ET - 1, lane, (c1 >> lane) & 1);
+            }
+            bool swept = false;
+            int n_left = EMAXS;
+            while (true) {
+                // ordering with most votes over the warp (counts <= 32 per lane)
+                unsigned lo = (votes & 0xffu) | ((votes & 0xff00u) << 8);
+                unsigned hi = ((votes >> 16) & 0xffu) | ((votes >> 24) << 16);
+                lo = __reduce_add_sync(0xffffffffu, lo);
+                hi = __reduce_add_sync(0xffffffffu, hi);
+                left = lo | hi;
+                if (left == 0 || n_left == 0) break;
+                const unsigned c[4] = {lo & 0xffffu, lo >> 16, hi & 0xffffu, hi >> 16};
+                int dir = 0;
+                unsigned most = c[0];
+#pragma unroll
+                for (int q = 1; q < 4; ++q)
+                    if (c[q] > most) { most = c[q]; dir = q; }
+                const bool fwx = (dir & 1) == 0, fwy = (dir & 2) == 0;
+                const unsigned um = fwx ? upd : updr;
+                const int i = fwx ? lane : ET - 1 - lane;
+                for (int u = 0; u < 2 * ET - 1; ++u) {
+                    const int jj = u - lane, j = fwy ? jj : ET - 1 - jj;
+                    if ((unsigned)jj < (unsigned)ET && ((um >> j) & 1)) {
+                        const double a = dmin2<FAST>(T[j + 1][i], T[j + 1][i + 2]);
+                        const double b = dmin2<FAST>(T[j][i + 1], T[j + 2][i + 1]);
+                        const double v = godunov_upd<FAST>(a, b, Fs[j][i]);
+                        if (dlt<FAST>(dmin2<FAST>(a, b), EINF) && dlt<FAST>(v, T[j + 1][i + 1])) T[j + 1][i + 1] = v;
+                    }
+                    __syncwarp();
+                }
+                swept = true;
+                --n_left;
+                votes = look_all();
+            }
+            big = __any_sync(0xffffffffu, big);
+            // below-tol decreases are written but do not wake the neighbours
+            if (swept && lane == 0 && (big || left)) {
+                act_out[t] = left ? 2 : 1;
+                atomicAdd(nchanged, 1u);
+            }
+            return swept;
+        };
+        const bool swept = fast ? visit(std::true_type{}) : visit(std::false_type{});
+        if (swept) {
+            for (int r = 0; r < ET; ++r)
+                if ((upd >> r) & 1) __stcg(&tau[(long long)(gy0 + r) * n + gx0 + lane], T[r + 1][lane + 1]);
         }
-        chg_rep = __any_sync(0xffffffffu, chg_rep);
-        changed = changed || chg_rep;
-        if (!chg_rep) break;
-    }
-    // write the interior back (also values that decreased by less than tol)
-    for (int r = 0; r < ET; ++r) {
-        const int gi = gx0 + lane, gj = gy0 + r;
-        if (gi < n && gj < ny) {
-            const long long p = (long long)gj * n + gi;
-            const double v = T[r + 1][lane + 1];
-            if (v < __ldcg(&tau[p])) __stcg(&tau[p], v);
-        }
-    }
-    if (changed && lane == 0) {
-        act_out[t] = 1;
-        atomicAdd(nchanged, 1u);
+        __syncwarp();
     }
 }
 
@@ -199,43 +313,64 @@ extern "C" int mg_eikonal_rect(int n, int ny, const double* s, double x0, double
         ds = q;
     }
     double* dt = is_dev(tau) ? tau : (double*)dalloc(N * 8);
-    unsigned char* fixed = (unsigned char*)dalloc(N);
-    unsigned char* act = (unsigned char*)dalloc(2 * (size_t)ntiles);
-    unsigned* cnt = (unsigned*)dalloc(sizeof(unsigned));
-    unsigned* hcnt = nullptr;
-    if (!dt || !fixed || !act || !cnt || cudaMallocHost(&hcnt, sizeof(unsigned)) != cudaSuccess) {
+    // three activity tables (read, written, cleared for the pass after) and
+    // the changed-tile counts of a batch of passes
+    unsigned char* act = (unsigned char*)dalloc(3 * (size_t)ntiles + 256 + EBATCH * sizeof(unsigned));
+    if (!dt || !act) {
         release();
         set_error("mg_eikonal: out of device memory");
         return MG_ENOMEM;
     }
-    k_eik_init<<<1216, 256, 0, st>>>(n, ny, h, ds, x0, y0, r_init, i0, j0, dt, fixed);
-    cudaMemsetAsync(act, 1, (size_t)ntiles, st);            // every tile runs in the first pass
-    const dim3 blk(32, EW);
-    const unsigned nblk = (unsigned)((ntiles + EW - 1) / EW);
+    unsigned* cnt = (unsigned*)(((uintptr_t)(act + 3 * (size_t)ntiles) + 255) / 256 * 256);
+    EikSrc src;
+    src.x0 = x0;
+    src.y0 = y0;
+    src.r_init = r_init;
+    src.is = i0;
+    src.js = j0;
+    {
+        // index box of the fixed disc, one node wider on every side
+        auto lo = [&](double c) { return (int)std::max(-1.0, std::min((c - r_init) / h - 3.0, 65536.0)); };
+        auto hi = [&](double c) { return (int)std::max(-1.0, std::min((c + r_init) / h + 2.0, 65536.0)); };
+        src.i0 = lo(x0);
+        src.i1 = hi(x0);
+        src.j0 = lo(y0);
+        src.j1 = hi(y0);
+    }
+    k_eik_init<<<1216, 256, 0, st>>>(n, ny, h, ds, src, dt);
+    cudaMemsetAsync(act, 2, (size_t)ntiles, st);            // every tile is looked at in the first pass
+    cudaMemsetAsync(act + ntiles, 0, 2 * (size_t)ntiles, st);
+    const unsigned nblk = (unsigned)std::min(ntiles, 16384);
     int pass = 0, rc = MG_ENOTCONV;
-    for (; pass < max_passes; ++pass) {
-        unsigned char* a_in = act + (size_t)(pass & 1) * ntiles;
-        unsigned char* a_out = act + (size_t)((pass + 1) & 1) * ntiles;
-        cudaMemsetAsync(a_out, 0, (size_t)ntiles, st);
-        cudaMemsetAsync(cnt, 0, sizeof(unsigned), st);
-        k_eik_pass<<<nblk, blk, 0, st>>>(n, ny, h, ds, fixed, dt, a_in, a_out, cnt, tol, 2);
-        cudaMemcpyAsync(hcnt, cnt, sizeof(unsigned), cudaMemcpyDeviceToHost, st);
+    unsigned hcnt[EBATCH];
+    while (pass < max_passes && rc != MG_OK) {
+        // a few passes per look of the host: after the pass that changed
+        // nothing the rest of a batch finds no active tile
+        const int nb = std::min(EBATCH, max_passes - pass);
+        cudaMemsetAsync(cnt, 0, EBATCH * sizeof(unsigned), st);
+        for (int q = 0; q < nb; ++q) {
+            unsigned char* a_in = act + (size_t)((pass + q) % 3) * ntiles;
+            unsigned char* a_out = act + (size_t)((pass + q + 1) % 3) * ntiles;
+            unsigned char* a_clr = act + (size_t)((pass + q + 2) % 3) * ntiles;
+            k_eik_pass<<<nblk, 32, 0, st>>>(n, ny, h, ds, src, dt, a_in, a_out, a_clr, cnt + q, tol);
+        }
+        cudaMemcpyAsync(hcnt, cnt, sizeof(unsigned) * nb, cudaMemcpyDeviceToHost, st);
         cudaError_t e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) {
-            cudaFreeHost(hcnt);
             release();
             set_error(std::string("mg_eikonal: ") + cudaGetErrorString(e));
             return MG_ECUDA;
         }
-        if (*hcnt == 0) {
-            rc = MG_OK;
+        for (int q = 0; q < nb; ++q) {
             ++pass;
-            break;
+            if (hcnt[q] == 0) {
+                rc = MG_OK;
+                break;
+            }
         }
     }
     if (dt != tau) cudaMemcpyAsync(tau, dt, N * 8, cudaMemcpyDeviceToHost, st);
     cudaError_t e = cudaStreamSynchronize(st);
-    cudaFreeHost(hcnt);
     release();
     if (e != cudaSuccess) {
         set_error(std::string("mg_eikonal: ") + cudaGetErrorString(e));
