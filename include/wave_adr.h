@@ -109,21 +109,19 @@ typedef struct mg_params {
                                setup and keep the fastest (default); 0: default tile shapes */
     int tile_candidate;     /* -1 (default); 0..MG_TILE_CANDIDATES-1: use that candidate for every ADR
                                GMRES kernel (overrides autotune; for testing each shape) */
-    int tail_nmax;          /* ADR levels l >= 3 with n_l <= tail_nmax and everything below them form the
-                               coarse tail of an instance, run without per-level launches (see tail_cluster);
-                               0 = off; -1 (default): 31 for a handle with one instance and the shared-
-                               memory tail, else 0 (measured fastest on this GPU).  The same bound, when
+    int tail_nmax;          /* ADR levels l >= 3 with max(n_l, ny_l) <= tail_nmax and everything below them form
+                               the coarse tail of an instance, run as one cluster launch (see tail_cluster); where
+                               the level of the ADR corrections itself is within the bound, all M corrections are
+                               one launch; 0 = off; -1 (default): for a handle with one instance 127 (mixed) or
+                               63 (FP64), else 0 (measured fastest on this GPU).  The same bound, when
                                set, selects the wave-cycle levels l >= 4 that run as a shared-memory tail
                                (Chebyshev smoothing and transfers in one block per instance); -1: n_l <= 63 */
     int pdl;                /* 1: kernels are launched with programmatic dependent launch (a kernel's
                                descriptor prologue overlaps its predecessor); 0 (default): plain launches
                                (measured 0.1 ms per n=4095 cycle faster on this GPU) */
-    int tail_cluster;       /* must be 0: the coarse tail is the shared-memory tail -- one block per instance
-                               runs the pre-smoothing chain down to the coarsest level, the FP64 coarsest solve
-                               follows, one block per instance runs the post-smoothing chain up (3 launches per
-                               ADR cycle; a level joins the tail only if its vectors fit in one block's shared
-                               memory).  Other values return MG_EINVAL (a cluster-per-instance tail was measured
-                               slower on this GPU and is not built) */
+    int tail_cluster;       /* must be 0 (other values return MG_EINVAL): the coarse ADR tail is one thread-block
+                               cluster per instance, its levels' rows dealt to the blocks' shared memory; a level
+                               joins the tail only if the chain from it down fits there */
     int ray;                /* 0 (default): the M ADR corrections use the input phase phi (Wave-ADR);
                                1: Wave-Ray (the ray equations of Section 3.2): correction m = 1..M uses the
                                plane-wave phase phi_m = cos(theta_m) x + sin(theta_m) y, theta_m =

@@ -21,7 +21,7 @@
 #include "cheb_stream.cuh"
 #include "cheb_multi.cuh"
 #include "restrict_stream.cuh"
-#include "tail_smem.cuh"
+#include "tail_cluster.cuh"
 #include "tail_wave.cuh"
 #include "setup_kernels.cuh"
 
@@ -584,7 +584,7 @@ struct Engine : EngineBase {
         for (int l = 2; l <= H.Lmax; ++l) {
             std::vector<int> rest;
             for (size_t b = 0; b < H.inst.size(); ++b)
-                if (adr_per_level(H, (int)b, l)) rest.push_back((int)b);
+                if (adr_per_level(H, (int)b, l) && !adr_whole(H, (int)b)) rest.push_back((int)b);
             if (rest.empty()) continue;   // not launched per level (coarse tail) or no such level
             const std::vector<int> ds = descs(H, l, rest);
             TileChoice tc;
@@ -636,61 +636,101 @@ struct Engine : EngineBase {
         }, t.pts);
     }
 
-    // Shared-memory tail (tail_smem.cuh): the largest dynamic shared memory
-    // its kernels may use (opt-in limit minus their static shared memory),
-    // set on both kernels once.
-    static long long ts_smem_limit() {
-        static long long lim = -1;
-        if (lim >= 0) return lim;
-        int dev = 0, optin = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        cudaFuncAttributes a1 = {}, a2 = {};
-        cudaFuncGetAttributes(&a1, k_adr_down<T>);
-        cudaFuncGetAttributes(&a2, k_adr_up<T>);
-        lim = (long long)optin - (long long)std::max(a1.sharedSizeBytes, a2.sharedSizeBytes) - 256;
-        if (lim < 0) lim = 0;
-        cudaFuncSetAttribute(k_adr_down<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim);
-        cudaFuncSetAttribute(k_adr_up<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim);
-        cudaGetLastError();
+    // Cluster form of the coarse ADR levels (tail_cluster.cuh): blocks per
+    // cluster, 16 where the GPU can place such a cluster with the most shared
+    // memory a block may ask for, else 8, else 0 (per-level launches).
+    template <int CS> static int ct_try(long long limit) {
+        auto kern = k_adr_cluster<T, CS>;
+        if (CS > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+            return 0;
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit) != cudaSuccess) return 0;
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute at[1];
+        ct_config(cfg, at, CS, 1, limit, nullptr);
+        int nc = 0;
+        return cudaOccupancyMaxActiveClusters(&nc, kern, &cfg) == cudaSuccess && nc > 0 ? CS : 0;
+    }
+    static void ct_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, int cs, unsigned clusters, long long smem,
+                          cudaStream_t st) {
+        cfg.gridDim = dim3((unsigned)cs * clusters);
+        cfg.blockDim = dim3(CT_THREADS);
+        cfg.dynamicSmemBytes = (size_t)smem;
+        cfg.stream = st;
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)cs;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+    }
+    static long long ct_smem_limit() {
+        static const long long lim = [] {
+            int dev = 0, optin = 0;
+            cudaGetDevice(&dev);
+            cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+            cudaFuncAttributes a = {}, b = {};
+            cudaFuncGetAttributes(&a, k_adr_cluster<T, 16>);
+            cudaFuncGetAttributes(&b, k_adr_cluster<T, 8>);
+            return std::max(0LL, (long long)optin - (long long)std::max(a.sharedSizeBytes, b.sharedSizeBytes));
+        }();
         return lim;
     }
-    // The shared-memory tail holds the vectors of its first level n x n.
-    static bool ts_fits(int n, int ny) {
-        return n <= TS_MAXN && ts_up_smem<T>(n, ny) <= ts_smem_limit() && ts_down_smem<T>(n, ny) <= ts_smem_limit();
+    static int ct_cluster() {
+        static const int cs = [] {
+            int c = ct_try<16>(ct_smem_limit());
+            if (!c) c = ct_try<8>(ct_smem_limit());
+            cudaGetLastError();
+            return c;
+        }();
+        return cs;
+    }
+    // Levels l .. L of instance b fit one cluster (whole: with the iterate of
+    // the ADR corrections).
+    static bool ct_fits(Handle& H, int b, int l, bool whole) {
+        const InstHost& I = H.inst[b];
+        const int nl = I.L - l + 1, cs = ct_cluster();
+        return cs > 0 && nl >= 2 && nl <= CT_MAXL &&
+               ct_smem<T>(I.lv[l - 1].n, I.lv[l - 1].ny, nl, cs, whole) <= ct_smem_limit();
     }
 
-    // Down / coarsest / up launches of the shared-memory tail for the
-    // instances in `tail` (their level l is the first tail level).
-    void launch_tail_smem(Handle& H, int l, const std::vector<int>& tail, cudaStream_t st) {
+    // One cluster per instance of `tail`: the ADR V-cycle from level l (corr
+    // = 0, SAB to SAX), or `corr` whole ADR corrections on level l.
+    void launch_adr_cluster(Handle& H, int l, const std::vector<int>& tail, int corr, cudaStream_t st) {
         const std::vector<int> ds = adescs(H, l, tail);
-        const std::string key = "tsm" + desc_key(ds);
+        const std::string key = "ct" + desc_key(ds);
         auto it = H.tail_first.find(key);
-        int* dfirst = nullptr;
+        int* dchain = nullptr;
         if (it == H.tail_first.end()) {
-            dfirst = (int*)H.alloc(sizeof(int) * ds.size());
-            cudaMemcpy(dfirst, ds.data(), sizeof(int) * ds.size(), cudaMemcpyHostToDevice);
-            H.tail_first[key] = dfirst;
+            std::vector<int> ch(ds.size() * CT_MAXL, -1);
+            for (size_t q = 0; q < ds.size(); ++q)
+                for (int k = 0, d = ds[q]; d >= 0 && k < CT_MAXL; ++k, d = H.hdesc[(size_t)d].coarse)
+                    ch[q * CT_MAXL + k] = d;
+            dchain = (int*)H.alloc(sizeof(int) * ch.size());
+            cudaMemcpy(dchain, ch.data(), sizeof(int) * ch.size(), cudaMemcpyHostToDevice);
+            H.tail_first[key] = dchain;
         } else {
-            dfirst = it->second;
+            dchain = it->second;
         }
-        long long sd = 0, su = 0, pts = 0;
+        const int cs = ct_cluster();
+        long long sm = 0, pts = 0, mat = 0, top = 0;
         for (int b : tail) {
-            const int n = H.inst[b].lv[l - 1].n, ny = H.inst[b].lv[l - 1].ny;
-            sd = std::max(sd, ts_down_smem<T>(n, ny));
-            su = std::max(su, ts_up_smem<T>(n, ny));
-            for (int q = l; q < H.inst[b].L; ++q) pts += (long long)H.inst[b].lv[q - 1].n * H.inst[b].lv[q - 1].ny;
+            const InstHost& I = H.inst[b];
+            const int n = I.lv[l - 1].n, ny = I.lv[l - 1].ny;
+            sm = std::max(sm, ct_smem<T>(n, ny, I.L - l + 1, cs, corr > 0));
+            top += (long long)n * ny;
+            for (int q = l; q < I.L; ++q) pts += (long long)I.lv[q - 1].n * I.lv[q - 1].ny;
+            const long long N = (long long)I.lv[I.L - 1].n * I.lv[I.L - 1].ny;
+            mat += N * N;
         }
-        ts_smem_limit();
-        const unsigned nb = (unsigned)tail.size();
-        // per tail-level point, as the multi-launch kernels count them: down = gram pass and pre-smoothing
-        // update, up = prolongation, gram pass and post-smoothing update
-        go(H, st, KK_ADR_TAIL, ((3 * C + Q) + (4 * C + Q + C / 4)) * (double)pts, [&] {
-            k_adr_down<T><<<nb, TS_THREADS, (size_t)sd, st>>>((const LevelDesc*)H.ddesc, (const int*)dfirst);
-        }, pts);
-        coarse_solve(H, tail, 1, st);   // every depth in one launch
-        go(H, st, KK_ADR_TAIL, ((4 * C + Q + C) + (3 * C + Q) + 5 * C) * (double)pts, [&] {
-            k_adr_up<T><<<nb, TS_THREADS, (size_t)su, st>>>((const LevelDesc*)H.ddesc, (const int*)dfirst);
+        // bytes as the per-level kernels count them
+        const double vc = (2 * (3 * C + Q) + (4 * C + Q + C / 4) + (4 * C + Q + C) + 5 * C) * (double)pts + C * (double)mat;
+        go(H, st, KK_ADR_TAIL, std::max(corr, 1) * vc + corr * (6 * C + R) * (double)top, [&] {
+            cudaLaunchConfig_t cfg = {};
+            cudaLaunchAttribute at[1];
+            ct_config(cfg, at, cs, (unsigned)tail.size(), sm, st);
+            const LevelDesc* D = H.ddesc;
+            const int* ch = dchain;
+            if (cs == 16) cudaLaunchKernelEx(&cfg, k_adr_cluster<T, 16>, D, ch, corr);
+            else cudaLaunchKernelEx(&cfg, k_adr_cluster<T, 8>, D, ch, corr);
         }, pts);
     }
 
@@ -761,10 +801,18 @@ struct Engine : EngineBase {
     }
     // Level l (not the coarsest) of instance b starts or lies in the coarse
     // tail: l >= 3 (below the ADR-correction level), max(n_l, ny_l) <=
-    // tail_nmax and its vectors fit in one block's shared memory.
+    // tail_nmax and the levels from l down fit in one cluster.
     static bool in_tail(Handle& H, int b, int l) {
         const int n = H.inst[b].lv[l - 1].n, ny = H.inst[b].lv[l - 1].ny;
-        return l >= 3 && l > H.inst[b].la && std::max(n, ny) <= H.p.tail_nmax && ts_fits(n, ny);
+        return l >= 3 && l > H.inst[b].la && std::max(n, ny) <= H.p.tail_nmax && ct_fits(H, b, l, false);
+    }
+    // The ADR corrections of instance b run whole in one cluster launch: the
+    // correction level itself is within the tail's bound and fits (Wave-Ray
+    // changes the operators from one correction to the next).
+    static bool adr_whole(Handle& H, int b) {
+        const InstHost& I = H.inst[b];
+        return I.la > 0 && !H.p.ray && std::max(I.lv[I.la - 1].n, I.lv[I.la - 1].ny) <= H.p.tail_nmax &&
+               ct_fits(H, b, I.la, true);
     }
     // ADR V-cycle on levels l..L (Section 3.2.2), right-hand side in SAB of
     // level l, result in SAX (or, at level 2 with `modulate`, added as
@@ -787,7 +835,7 @@ struct Engine : EngineBase {
             coarse_solve(H, due, 1, st);
             due.clear();
         }
-        if (!tail.empty()) launch_tail_smem(H, l, tail, st);
+        if (!tail.empty()) launch_adr_cluster(H, l, tail, 0, st);
         if (rest.empty()) return;
         const std::vector<int> ds = adescs(H, l, rest);
         const TileChoice tc = tiles_of(H, ds);
@@ -811,7 +859,11 @@ struct Engine : EngineBase {
     // Algorithm 1's ADR correction steps on the ADR level la (M times; level
     // 2 with the roles by index).
     // Wave-Ray (H.p.ray): correction m uses the ADR levels of plane wave m.
-    void adr_corrections(Handle& H, const std::vector<int>& I, int la, int M, cudaStream_t st) {
+    void adr_corrections(Handle& H, const std::vector<int>& all, int la, int M, cudaStream_t st) {
+        std::vector<int> whole, I;
+        for (int b : all) (adr_whole(H, b) ? whole : I).push_back(b);
+        if (!whole.empty() && M > 0) launch_adr_cluster(H, la, whole, M, st);
+        if (I.empty()) return;
         for (int m = 0; m < M; ++m) {
             H.cur_var = H.p.ray ? m : 0;
             const SegTable& t = H.seg(adescs(H, la, I), false, kPts);

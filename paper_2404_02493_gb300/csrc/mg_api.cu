@@ -985,13 +985,14 @@ int mg_setup(mg_handle** out, const mg_instance* inst, int ninst, const mg_param
     mg_handle* mh = new mg_handle();
     mh->H.p = *p;
     mh->H.alloc_limit = p->workspace_limit;
-    // automatic coarse tail: the shared-memory tail of the levels with n <= 31
-    // pays off for a single instance (one block per instance runs those
-    // levels); with many instances the per-level launches spread the work
-    // over more SMs
+    // automatic coarse tail (one cluster per instance, tail_cluster.cuh) for a
+    // handle with one instance: levels with n <= 127 in FP32, where a launch
+    // costs more than its work, n <= 63 in FP64, whose arithmetic wants all
+    // SMs above that; with many instances the per-level launches spread the
+    // work over more SMs
     // the wave-cycle tail (tail_wave.cuh) follows an explicit tail_nmax; automatic: levels with n <= 63
     mh->H.wave_tail_nmax = mh->H.p.tail_nmax >= 0 ? mh->H.p.tail_nmax : 63;
-    if (mh->H.p.tail_nmax < 0) mh->H.p.tail_nmax = ninst == 1 ? 31 : 0;
+    if (mh->H.p.tail_nmax < 0) mh->H.p.tail_nmax = ninst == 1 ? (p->precision == MG_PREC_FP64 ? 63 : 127) : 0;
     // the two tails follow the index roles: with a role list every level has
     // its own launches
     if (roles_set(*p)) {

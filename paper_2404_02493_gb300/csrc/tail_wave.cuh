@@ -21,10 +21,11 @@
 // not read it).  Only block barriers are used; every thread runs the same
 // level loop.
 #pragma once
-#include "tail_smem.cuh"
+#include "kernels.cuh"
 
 namespace wadr {
 
+constexpr int TS_MAXL = 8;    // levels of a chain, the coarsest included
 constexpr int WT_THREADS = 1024;
 constexpr int WT_MAXN = 64;   // nodes map to threads as 64 columns x 16 rows
 
@@ -40,6 +41,37 @@ constexpr int WT_MAXN = 64;   // nodes map to threads as 64 columns x 16 rows
 // and g / x of the odd levels ((n/2)(ny/2))
 template <typename T> __host__ __device__ constexpr long long wt_smem(int n, int ny) {
     return (long long)sizeof(cplx<T>) * (5LL * n * ny + (long long)(n / 2) * (ny / 2));
+}
+
+// The level chain of this block's instance from first[blockIdx.x] down to
+// the coarsest level, descriptors copied to shared memory; returns the
+// number of levels (>= 2: at least one tail level and the coarsest).
+__device__ __forceinline__ int ts_chain(const LevelDesc* __restrict__ D, const int* __restrict__ first, LevelDesc* Lv,
+                                        int* didx, int* nlev) {
+    if (threadIdx.x == 0) {
+        int di = first[blockIdx.x];
+        int k = 0;
+        while (di >= 0 && k < TS_MAXL) {
+            didx[k++] = di;
+            di = D[di].coarse;
+        }
+        *nlev = k;
+    }
+    __syncthreads();
+    constexpr int W = (int)(sizeof(LevelDesc) / sizeof(unsigned long long));
+    static_assert(sizeof(LevelDesc) % sizeof(unsigned long long) == 0, "descriptor size");
+    const int nl = *nlev;
+    for (int e = threadIdx.x; e < nl * W; e += blockDim.x) {
+        const int k = e / W, w = e - k * W;
+        reinterpret_cast<unsigned long long*>(&Lv[k])[w] = reinterpret_cast<const unsigned long long*>(D + didx[k])[w];
+    }
+    __syncthreads();
+    return nl;
+}
+
+template <typename T>
+__device__ __forceinline__ cplx<T> ts_coarse_at(const cplx<T>* E, int nc, int ncy, int I, int J) {
+    return ((unsigned)I < (unsigned)nc && (unsigned)J < (unsigned)ncy) ? E[J * nc + I] : zero2<T>();
 }
 
 // DG = h^2 diag(A) of level d (eq. A1's diagonal with the boundary terms)
