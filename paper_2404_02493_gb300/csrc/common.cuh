@@ -110,6 +110,7 @@ struct LevelDesc {
     double* fs;             // outer: FGMRES scalars
     double2* fpart;         // outer: FGMRES reduction partials [MAXB][NVF]
     double* est;            // outer: |gamma_{j+1}| of this instance (contiguous over instances)
+    long long uoff;         // level 1: offset of this instance in dense user arrays (elements)
     const void* tm;         // tensor maps of the tile kernels (MapId order, 128 B each)
     unsigned* err;          // handle error word (device-side wait expiry)
 };

@@ -110,7 +110,8 @@ struct Handle {
     long long alloc_limit = 0;      // mg_params.workspace_limit (0: none)
     long long total_elems = 0;      // sum of n ny over instances
     // graphs
-    cudaGraphExec_t g_cycle0 = nullptr;     // cycle from u = 0 (level-1 SG -> SD)
+    cudaGraphExec_t g_cycle = nullptr;      // mg_cycle's cycle (level-1 SX2, SG -> SD)
+    int cycle_calls = 0;                    // device-array calls of mg_cycle (the second captures g_cycle)
     cudaGraphExec_t g_irstep = nullptr;     // scale + cycle + update + residual
     cudaStream_t g_stream = nullptr;
     int launches_cycle = 0;                 // kernels of the last emitted cycle
@@ -159,6 +160,9 @@ struct EngineBase {
     virtual void fg_start(Handle& H, cudaStream_t st) = 0;
     virtual void fg_iter(Handle& H, cudaStream_t st) = 0;
     virtual void fg_finish(Handle& H, cudaStream_t st) = 0;
+    // dense user arrays (device memory) -> level-1 SX2, SG; level-1 SD -> a dense user array
+    virtual void user_in(Handle& H, const void* u, const void* g, cudaStream_t st) = 0;
+    virtual void user_out(Handle& H, void* u, cudaStream_t st) = 0;
     // level operations (single instance) used by the parity tests
     virtual int level_op(Handle& H, int inst, int level, int what, int a0, int a1, cudaStream_t st) = 0;
     // halo-tile autotuner of the ADR launches (fills Handle::tiles)

@@ -1039,4 +1039,37 @@ __global__ void __launch_bounds__(NT) k_zero(const __grid_constant__ KDesc A, co
         slot<T>(d, sa)[(long long)j * d.pitch + i] = zero2<T>();
     }
 }
+
+// Dense user arrays of all instances <-> the level-1 slots of a cycle, one
+// launch for every instance: u and g into SX2 and SG, the result SD out (two
+// row-pitched copies and a slot copy per instance and call before).
+template <typename T>
+__global__ void __launch_bounds__(NT) k_user_in(const __grid_constant__ KDesc A, const Seg* __restrict__ Sg, int nseg,
+                                                const cplx<T>* __restrict__ u, const cplx<T>* __restrict__ g) {
+    __shared__ LevelDesc d;
+    SegCtx c = seg_begin(A, Sg, nseg, d);
+    const int ntx = (d.n + BX - 1) / BX, nty = (d.ny + BY - 1) / BY;
+    cplx<T>* const us = slot<T>(d, SX2);
+    cplx<T>* const gs = slot<T>(d, SG);
+    for (int t = c.lb; t < ntx * nty; t += c.nb) {
+        const int i = (t % ntx) * BX + threadIdx.x, j = (t / ntx) * BY + threadIdx.y;
+        if (i >= d.n || j >= d.ny) continue;
+        const long long p = (long long)j * d.pitch + i, q = d.uoff + (long long)j * d.n + i;
+        us[p] = u[q];
+        gs[p] = g[q];
+    }
+}
+template <typename T>
+__global__ void __launch_bounds__(NT) k_user_out(const __grid_constant__ KDesc A, const Seg* __restrict__ Sg, int nseg,
+                                                 cplx<T>* __restrict__ u) {
+    __shared__ LevelDesc d;
+    SegCtx c = seg_begin(A, Sg, nseg, d);
+    const int ntx = (d.n + BX - 1) / BX, nty = (d.ny + BY - 1) / BY;
+    const cplx<T>* const us = slot<T>(d, SD);
+    for (int t = c.lb; t < ntx * nty; t += c.nb) {
+        const int i = (t % ntx) * BX + threadIdx.x, j = (t / ntx) * BY + threadIdx.y;
+        if (i >= d.n || j >= d.ny) continue;
+        u[d.uoff + (long long)j * d.n + i] = us[(long long)j * d.pitch + i];
+    }
+}
 }  // namespace wadr

@@ -626,6 +626,7 @@ static int build(mg_handle* mh, const mg_instance* in, int ninst, cudaStream_t s
                 lv.peclet = setup_peclet(lv.k64, lv.phi64, lv.sig64, lv.n, lv.ny, lv.pitch, lv.h, I.omega, I.bc, dscr, st);
             d.fgs = (float)d.gs;
             d.bc = I.bc;
+            d.uoff = l == 1 ? I.off : 0;
             d.inst = b;
             d.level = l;
             d.coarse = (l < I.L) ? di + 1 : -1;
@@ -795,11 +796,15 @@ static int build(mg_handle* mh, const mg_instance* in, int ninst, cudaStream_t s
 }
 
 // Capture `emit` into a graph on the handle's stream (after one plain run
-// on the zeroed workspace that builds every segment table).
+// on the zeroed workspace that builds every segment table, unless the tables
+// exist already).
 template <class F>
-static int capture(Handle& H, cudaGraphExec_t* out, F emit) {
-    emit(H.g_stream);
-    cudaError_t e = cudaStreamSynchronize(H.g_stream);
+static int capture(Handle& H, cudaGraphExec_t* out, F emit, bool built = false) {
+    cudaError_t e = cudaSuccess;
+    if (!built) {
+        emit(H.g_stream);
+        e = cudaStreamSynchronize(H.g_stream);
+    }
     if (e != cudaSuccess) { set_error(cudaGetErrorString(e)); return MG_ECUDA; }
     cudaGraph_t g;
     e = cudaStreamBeginCapture(H.g_stream, cudaStreamCaptureModeThreadLocal);
@@ -816,7 +821,7 @@ static int capture(Handle& H, cudaGraphExec_t* out, F emit) {
 static void free_all(Handle& H) {
     for (cudaEvent_t e : H.ev_pool) cudaEventDestroy(e);
     H.ev_pool.clear();
-    if (H.g_cycle0) cudaGraphExecDestroy(H.g_cycle0);
+    if (H.g_cycle) cudaGraphExecDestroy(H.g_cycle);
     if (H.g_irstep) cudaGraphExecDestroy(H.g_irstep);
     if (H.g_fgiter) cudaGraphExecDestroy(H.g_fgiter);
     if (H.g_stream) cudaStreamDestroy(H.g_stream);
@@ -1171,11 +1176,57 @@ static bool is_host_ptr(const void* p) {
     return !dev;
 }
 
+// p is device (or managed) memory of the current device, aligned for the
+// cycle's complex type: kernels may read and write it where it lies.
+static bool kernel_ptr(const void* p, size_t es) {
+    cudaPointerAttributes a;
+    int dev = -1;
+    const bool ok = cudaPointerGetAttributes(&a, p) == cudaSuccess && cudaGetDevice(&dev) == cudaSuccess &&
+                    (a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == dev));
+    cudaGetLastError();
+    return ok && (uintptr_t)p % es == 0;
+}
+
 int mg_cycle(mg_handle* h, void* u, const void* g, int ncycles, mg_stream stream) {
     if (!h || !u || !g || ncycles < 0) { set_error("mg_cycle: bad argument"); return MG_EINVAL; }
     Handle& H = h->H;
     cudaStream_t st = (cudaStream_t)stream;
     const size_t es = esz(H.prec);
+    auto next_cycle = [&](int c) -> int {   // SD -> SX2 between cycles
+        if (c + 1 < ncycles)
+            for (auto& I : H.inst) {
+                LevelHost& l1 = I.lv[0];
+                WADR_CHECK(cudaMemcpyAsync(slot_ptr(H, l1, SX2), slot_ptr(H, l1, SD), l1.slot_stride * es,
+                                           cudaMemcpyDeviceToDevice, st));
+            }
+        return MG_OK;
+    };
+    if (ncycles > 0 && kernel_ptr(u, es) && kernel_ptr(g, es)) {
+        // device arrays.  The first call emits the cycle kernel by kernel (it
+        // builds the launch tables), the second captures it into a graph,
+        // which every call from then on replays: a cycle is 30 to 250 small
+        // launches, and the host took ~6.5 us to emit each of them (n = 127,
+        // M = 2: 225 us per call, host-bound).  A stream that is being
+        // captured itself takes the plain launches.
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        WADR_CHECK(cudaStreamIsCapturing(st, &cap));
+        const bool plain = !H.p.use_graph || cap != cudaStreamCaptureStatusNone;
+        if (!plain && !H.g_cycle && H.cycle_calls > 0) {
+            const int rc = capture(H, &H.g_cycle, [&](cudaStream_t s) { h->eng->cycle(H, false, s); }, true);
+            if (rc) return rc;
+        }
+        h->eng->user_in(H, u, g, st);
+        for (int c = 0; c < ncycles; ++c) {
+            if (!plain && H.g_cycle) WADR_CHECK(cudaGraphLaunch(H.g_cycle, st));
+            else h->eng->cycle(H, false, st);
+            const int rc = next_cycle(c);
+            if (rc) return rc;
+        }
+        h->eng->user_out(H, u, st);
+        WADR_CHECK(cudaGetLastError());
+        H.cycle_calls = 1;
+        return MG_OK;
+    }
     for (auto& I : H.inst) {
         LevelHost& l1 = I.lv[0];
         WADR_CHECK(copy_in(g, I.off, es, slot_ptr(H, l1, SG), l1.n, l1.ny, l1.pitch, st));
@@ -1183,15 +1234,12 @@ int mg_cycle(mg_handle* h, void* u, const void* g, int ncycles, mg_stream stream
     }
     for (int c = 0; c < ncycles; ++c) {
         h->eng->cycle(H, false, st);
-        for (auto& I : H.inst) {
-            LevelHost& l1 = I.lv[0];
-            WADR_CHECK(cudaMemcpyAsync(slot_ptr(H, l1, SX2), slot_ptr(H, l1, SD), l1.slot_stride * es,
-                                       cudaMemcpyDeviceToDevice, st));
-        }
+        const int rc = next_cycle(c);
+        if (rc) return rc;
     }
     for (auto& I : H.inst) {
         LevelHost& l1 = I.lv[0];
-        WADR_CHECK(copy_out(u, I.off, es, slot_ptr(H, l1, SX2), l1.n, l1.ny, l1.pitch, st));
+        WADR_CHECK(copy_out(u, I.off, es, slot_ptr(H, l1, ncycles > 0 ? SD : SX2), l1.n, l1.ny, l1.pitch, st));
     }
     WADR_CHECK(cudaGetLastError());
     if (is_host_ptr(u)) return check_device_error(H, st);   // synchronises: host result complete on return
