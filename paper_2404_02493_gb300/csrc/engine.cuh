@@ -592,6 +592,9 @@ struct Engine : EngineBase {
                 float best = 1e30f;
                 int arg = -1;
                 for (int c = 0; c < GS_NCAND; ++c) {
+                    // (in FP64 a strip march, one warp's chain of rows on a pipe
+                    // of two lanes, takes 4 to 10 times a tile's time)
+                    if (!kStream && w == 0 && gs_gram_streaming(c)) continue;
                     auto run = [&] {
                         if (w == 0) gs_gram(H, ds, c, SAB, st);
                         else gs_pre(H, ds, c, st);

@@ -59,6 +59,11 @@ template <typename T> struct GsEps;
 template <> struct GsEps<float> { static constexpr float tau = 32.0f * 1.1920929e-7f; };
 template <> struct GsEps<double> { static constexpr double tau = 32.0 * 2.220446049250313e-16; };
 
+// 1 / sqrt(x): in FP64 one call (a square root and a division are ~560 ns of
+// dependent FP64 operations here)
+__device__ __forceinline__ float inv_sqrt(float x) { return 1.0f / sqrtf(x); }
+__device__ __forceinline__ double inv_sqrt(double x) { return rsqrt(x); }
+
 // Normal equations of the s-step GMRES(3) in the last block (thread 0).
 // G[0] = (|K0|^2, |K1|^2), G[1] = (|K2|^2, |K3|^2), G[2..4] = <K0, K1..K3>,
 // G[5] = <K1,K2>, G[6] = <K1,K3>, G[7] = <K2,K3>  (<a,b> = sum conj(a) b).
@@ -71,7 +76,7 @@ __device__ inline void gs_solve(const cplx<T> (&G)[8], T* sc) {
     int m = 0;
     T dsc[3] = {T(0), T(0), T(0)};
     if (G[0].x > T(0))
-        while (m < 3 && dg[m] > T(0)) { dsc[m] = T(1) / sqrt(dg[m]); ++m; }
+        while (m < 3 && dg[m] > T(0)) { dsc[m] = inv_sqrt(dg[m]); ++m; }
     cplx<T> bb[3], c[3];
     for (int i = 0; i < 3; ++i) {
         bb[i] = cscale<T>(mk<T>(G[2 + i].x, -G[2 + i].y), dsc[i]);   // <K_{i+1}, K0>
@@ -80,30 +85,30 @@ __device__ inline void gs_solve(const cplx<T> (&G)[8], T* sc) {
     const cplx<T> r01 = cscale<T>(G[5], dsc[0] * dsc[1]);
     const cplx<T> r02 = cscale<T>(G[6], dsc[0] * dsc[2]);
     const cplx<T> a12 = cscale<T>(G[7], dsc[1] * dsc[2]);
-    T r11 = T(1), r22 = T(1);
+    T i11 = T(1), i22 = T(1);   // inverse pivots
     cplx<T> r12 = zero2<T>();
     if (m >= 2) {
         const T p1 = T(1) - cabs2<T>(r01);
-        if (p1 > GsEps<T>::tau) r11 = sqrt(p1);
+        if (p1 > GsEps<T>::tau) i11 = inv_sqrt(p1);
         else m = 1;
     }
     if (m >= 3) {
-        r12 = cscale<T>(csub<T>(a12, cmulc<T>(r01, r02)), T(1) / r11);
+        r12 = cscale<T>(csub<T>(a12, cmulc<T>(r01, r02)), i11);
         const T p2 = T(1) - cabs2<T>(r02) - cabs2<T>(r12);
-        if (p2 > GsEps<T>::tau) r22 = sqrt(p2);
+        if (p2 > GsEps<T>::tau) i22 = inv_sqrt(p2);
         else m = 2;
     }
     // R^H z = bb, then R c = z, on the leading m columns
     cplx<T> z[3];
     z[0] = bb[0];
-    z[1] = cscale<T>(csub<T>(bb[1], cmulc<T>(r01, z[0])), T(1) / r11);
-    z[2] = cscale<T>(csub<T>(csub<T>(bb[2], cmulc<T>(r02, z[0])), cmulc<T>(r12, z[1])), T(1) / r22);
+    z[1] = cscale<T>(csub<T>(bb[1], cmulc<T>(r01, z[0])), i11);
+    z[2] = cscale<T>(csub<T>(csub<T>(bb[2], cmulc<T>(r02, z[0])), cmulc<T>(r12, z[1])), i22);
     if (m == 3) {
-        c[2] = cscale<T>(z[2], T(1) / r22);
-        c[1] = cscale<T>(csub<T>(z[1], cmul<T>(r12, c[2])), T(1) / r11);
+        c[2] = cscale<T>(z[2], i22);
+        c[1] = cscale<T>(csub<T>(z[1], cmul<T>(r12, c[2])), i11);
         c[0] = csub<T>(csub<T>(z[0], cmul<T>(r01, c[1])), cmul<T>(r02, c[2]));
     } else if (m == 2) {
-        c[1] = cscale<T>(z[1], T(1) / r11);
+        c[1] = cscale<T>(z[1], i11);
         c[0] = csub<T>(z[0], cmul<T>(r01, c[1]));
     } else if (m == 1) {
         c[0] = z[0];
@@ -202,17 +207,98 @@ __device__ __forceinline__ void gram_acc(GramAcc<T>& g, cplx<T> k0, cplx<T> k1, 
     gacc_cross<T>(g.crs[5], k2, k3);
 }
 
-// reduction of the Gram entries of a launch and the small solve
+// The warp's sums of 16 values of every lane, value lane / 2 in each lane:
+// halves of the values are exchanged as the lane bits go (16 shuffles instead
+// of a tree per value).
+template <typename T> __device__ __forceinline__ T warp_sum16(T (&v)[16], int lane) {
+#pragma unroll
+    for (int o = 16, m = 8; o > 1; o >>= 1, m >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < m; ++i) {
+            const T send = up ? v[i] : v[i + m], keep = up ? v[i + m] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+// Sum over q < cnt rows of 16 values at sh, value lane / 2 in each lane
+// (one warp; each lane takes every second row).
+template <typename T> __device__ __forceinline__ T rows_sum16(const T* sh, int cnt, int lane) {
+    const int id = lane >> 1;
+    T t = T(0);
+    for (int q = lane & 1; q < cnt; q += 2) t += sh[q * 16 + id];
+    return t + __shfl_xor_sync(0xffffffffu, t, 1);
+}
+// the 16 sums of the lanes as the entries of gs_solve
+template <typename T> __device__ __forceinline__ void gram_entries(T t, cplx<T> (&G)[8]) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+        G[k] = mk<T>(__shfl_sync(0xffffffffu, t, 4 * k), __shfl_sync(0xffffffffu, t, 4 * k + 2));
+}
+
+// Reduction of the Gram entries of a launch and the small solve; sh: 16
+// values per 16 threads.  This chain ends every sweep, so on small levels it
+// is most of the pass: with a shuffle tree per value, one thread adding the
+// warps, storing the partials and adding the blocks, a 63 x 63 level took 7.3
+// us in FP32 and 61 us in FP64 (where a warp's addition holds the pipe for 16
+// cycles and a dependent one takes 32 ns).  Now 16 shuffles per warp, a lane
+// per value from there on, every sum split over two lanes or more (FP64 cycle at n = 511 3.44 -> 2.42 ms with the
+// selected upwind stencil, FP32 cycle at n = 1024 450 -> 416 us).
 template <typename T>
-__device__ __forceinline__ void gram_finish(const LevelDesc& d, const SegCtx& c, const GramAcc<T>& g, cplx<T>* sh,
-                                            int* flag) {
-    cplx<T> ac[8];
-    g.to_layout(ac);
-    block_sum<cplx<T>, 8>(ac, sh);
-    if (publish_partials<cplx<T>, 8>(partp<T>(d), MAXDOT, d.counter, c.lb, c.nb, ac, flag)) {
-        cplx<T> tot[8];
-        finish_partials<cplx<T>, 8>(partp<T>(d), MAXDOT, d.counter, c.nb, tot, sh);
-        if (threadIdx.x == 0 && threadIdx.y == 0) gs_solve<T>(tot, scalp<T>(d));
+__device__ __forceinline__ void gram_finish(const LevelDesc& d, const SegCtx& c, const GramAcc<T>& g, T* sh, int* flag) {
+    const int tid = threadIdx.x + threadIdx.y * blockDim.x, nt = blockDim.x * blockDim.y;
+    const int lane = tid & 31, w = tid >> 5;
+    {
+        cplx<T> ac[8];
+        g.to_layout(ac);
+        T v[16];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            v[2 * k] = ac[k].x;
+            v[2 * k + 1] = ac[k].y;
+        }
+        const T ws = warp_sum16<T>(v, lane);
+        if (!(lane & 1)) sh[w * 16 + (lane >> 1)] = ws;
+    }
+    __syncthreads();
+    T* const part = reinterpret_cast<T*>(d.part);
+    if (w == 0) {
+        T t = rows_sum16<T>(sh, nt >> 5, lane);
+        if (c.nb == 1) {
+            cplx<T> G[8];
+            gram_entries<T>(t, G);
+            if (lane == 0) gs_solve<T>(G, scalp<T>(d));
+        } else {
+            if (!(lane & 1)) part[(long long)c.lb * (2 * MAXDOT) + (lane >> 1)] = t;
+            __syncwarp();
+            if (lane == 0) {
+                __threadfence();
+                *flag = atomicAdd(d.counter, 1u) == (unsigned)(c.nb - 1);
+            }
+        }
+    }
+    if (c.nb == 1) return;
+    __syncthreads();
+    if (!*flag) return;
+    __threadfence();
+    {
+        // value tid % 16 of the blocks tid / 16, tid / 16 + nt / 16, ...
+        const int id = tid & 15, ng = nt >> 4;
+        T s = T(0);
+#pragma unroll 4
+        for (int b = tid >> 4; b < c.nb; b += ng) s += __ldcg(part + (long long)b * (2 * MAXDOT) + id);
+        sh[tid] = s;
+    }
+    __syncthreads();
+    if (w == 0) {
+        const T t = rows_sum16<T>(sh, nt >> 4, lane);
+        cplx<T> G[8];
+        gram_entries<T>(t, G);
+        if (lane == 0) {
+            gs_solve<T>(G, scalp<T>(d));
+            *d.counter = 0u;
+        }
     }
 }
 
@@ -232,7 +318,7 @@ __global__ void __launch_bounds__(NT) k_gs_gram_tile(const __grid_constant__ KDe
     cplx<T>* S1 = S0b + 2 * W0 * H0;
     cplx<T>* S2 = S1 + W1 * H1;
     __shared__ LevelDesc d;
-    __shared__ cplx<T> sh[8 * 8];
+    __shared__ T sh[NT];
     __shared__ int flag;
     SegCtx c = seg_begin(A, Sg, nseg, d);
     const int tid = threadIdx.x + threadIdx.y * blockDim.x;
@@ -301,7 +387,7 @@ __global__ void __launch_bounds__(32 * GS_WPB, sizeof(T) == 4 ? 4 : 1) k_gs_gram
     cplx<T>* Kr = reinterpret_cast<cplx<T>*>(reinterpret_cast<quad<T>*>(gs_smem) + GS_WPB * SW_DEP * SW_COLS) +
                   warp * SW_DEP * SW_COLS;
     __shared__ LevelDesc d;
-    __shared__ cplx<T> sh[8 * 8];
+    __shared__ T sh[32 * GS_WPB];
     __shared__ int flag;
     SegCtx c = seg_begin(A, Sg, nseg, d);
     const int n = d.n, ny = d.ny, pitch = d.pitch;

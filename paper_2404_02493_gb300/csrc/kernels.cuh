@@ -115,6 +115,26 @@ __device__ __forceinline__ cplx<T> adr_pt(const quad<T>& q, T ih2, T wh, cplx<T>
     return r;
 }
 
+// FP64: of each upwind pair one coefficient is zero, so the neighbour that
+// counts is selected (integer pipes) and its coefficient is 2 |p|: 18 FP64
+// operations instead of 26, on a pipe of two lanes per SM and clock.  The same
+// values (2 |p| w + 0 e = 2 |p| w; the factor 2 is exact).
+template <>
+__device__ __forceinline__ double2 adr_pt<double>(const quad<double>& q, double ih2, double wh, double2 c, double2 w,
+                                                  double2 e, double2 s, double2 nn) {
+    const double ax = fabs(q.x), ay = fabs(q.y), wh2 = 2.0 * wh;
+    const bool fx = __double_as_longlong(q.x) >= 0, fy = __double_as_longlong(q.y) >= 0;
+    const double2 ux = fx ? w : e, uy = fy ? s : nn;
+    const double avx = fma(ay, uy.x, ax * ux.x), avy = fma(ay, uy.y, ax * ux.y);
+    const double lx = (w.x + e.x) + (s.x + nn.x), ly = (w.y + e.y) + (s.y + nn.y);
+    double2 r;
+    r.x = fma(-q.w, c.y, q.z * c.x);
+    r.y = fma(q.w, c.x, q.z * c.y);
+    r.x = fma(-wh2, avy, fma(-ih2, lx, r.x));
+    r.y = fma(wh2, avx, fma(-ih2, ly, r.y));
+    return r;
+}
+
 // FP32: the same stencil in packed FP32x2 instructions (sm_100+), each
 // component rounded as the scalar operation.
 template <>

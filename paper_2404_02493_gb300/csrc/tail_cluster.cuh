@@ -73,22 +73,6 @@ template <typename T> struct CtLevel {
     T ih2, wh, s;
 };
 
-// The warp's sums of 16 values of every lane, value lane / 2 in each lane:
-// halves of the values are exchanged as the lane bits go (16 shuffles instead
-// of a tree per value).
-template <typename T> __device__ __forceinline__ T warp_sum16(T (&v)[16], int lane) {
-#pragma unroll
-    for (int o = 16, m = 8; o > 1; o >>= 1, m >>= 1) {
-        const bool up = lane & o;
-#pragma unroll
-        for (int i = 0; i < m; ++i) {
-            const T send = up ? v[i] : v[i + m], keep = up ? v[i + m] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-        }
-    }
-    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
-}
-
 template <typename T, int CS>
 __global__ void __launch_bounds__(CT_THREADS, 1) k_adr_cluster(const LevelDesc* __restrict__ D,
                                                                const int* __restrict__ chain, int corr) {
@@ -214,24 +198,14 @@ __global__ void __launch_bounds__(CT_THREADS, 1) k_adr_cluster(const LevelDesc* 
         __syncthreads();
         if (w == 0) {
             const int id = lane >> 1, h = lane & 1;
-            T t = shw[(h * (CT_WARPS / 2)) * 16 + id];
-#pragma unroll
-            for (int q = 1; q < CT_WARPS / 2; ++q) t += shw[(h * (CT_WARPS / 2) + q) * 16 + id];
-            t += __shfl_xor_sync(0xffffffffu, t, 1);
+            const T t = rows_sum16<T>(shw, CT_WARPS, lane);
 #pragma unroll
             for (int p = 0; p < CS; p += 2) *cl.map_shared_rank(&part[par][rank][id], p + h) = t;
         }
         cl.sync();
         if (w == 0) {
-            const int id = lane >> 1, h = lane & 1;
-            T t = part[par][h * (CS / 2)][id];
-#pragma unroll
-            for (int q = 1; q < CS / 2; ++q) t += part[par][h * (CS / 2) + q][id];
-            t += __shfl_xor_sync(0xffffffffu, t, 1);
             cplx<T> G[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-                G[k] = mk<T>(__shfl_sync(0xffffffffu, t, 4 * k), __shfl_sync(0xffffffffu, t, 4 * k + 2));
+            gram_entries<T>(rows_sum16<T>(&part[par][0][0], CS, lane), G);
             if (lane == 0) gs_solve<T>(G, scl);
         }
         par ^= 1;
