@@ -198,6 +198,35 @@ __device__ __forceinline__ cplx<T> helm_diag_h2(const LevelDesc& d, int i, int j
     return mk<T>(re, im);
 }
 
+// helm_diag_h2 less the 4 of the Laplacian, formed without it: -h^2 k^2 - m
+// ... keeps its own relative precision.
+template <typename T>
+__device__ __forceinline__ cplx<T> helm_diag4(const LevelDesc& d, int i, int j, T k, T sig) {
+    const T h = LC<T>::h(d), kh = k * h;
+    T re = -(kh * kh), im = T(0);
+    if (d.bc == BC_ABC1) {
+        const int m = (i == 0) + (i == d.n - 1) + (j == 0) + (j == d.ny - 1);
+        re -= (T)m;
+        im -= (T)m * kh;
+    } else if (d.bc == BC_SPONGE) {
+        im -= h * h * sig;
+    }
+    if (d.has_shift) im -= LC<T>::shift(d) * kh * kh;
+    return mk<T>(re, im);
+}
+// A z at a node from its diagonal dg4 (helm_diag4), value c and neighbours
+// (zero outside the grid), the Laplacian as a sum of differences.  A wave of
+// several nodes per wavelength makes (4 z - sum of neighbours) a small
+// difference of large terms: summed term by term in FP32 the product is off by
+// ~4 eps / (k h)^2, which dominated the error of the mixed solver's iterates
+// (5.7e-6 of their norm at k h = 0.39); differences of neighbouring values are
+// exact or nearly so.
+template <typename T>
+__device__ __forceinline__ cplx<T> helm_diff(cplx<T> dg4, cplx<T> c, cplx<T> w, cplx<T> e, cplx<T> s, cplx<T> n, T ih2) {
+    const cplx<T> t = cadd<T>(cadd<T>(csub<T>(c, w), csub<T>(c, e)), cadd<T>(csub<T>(c, s), csub<T>(c, n)));
+    return cscale<T>(cfma<T>(dg4, c, t), ih2);
+}
+
 template <typename T> __device__ __forceinline__ T load_k(const LevelDesc& d, int i, int j) {
     return __ldg(reinterpret_cast<const T*>(d.kf) + (long long)j * d.pitch + i);
 }
@@ -206,6 +235,20 @@ template <typename T> __device__ __forceinline__ T load_sig(const LevelDesc& d, 
 }
 template <typename T> __device__ __forceinline__ cplx<T> helm_diag_at(const LevelDesc& d, int i, int j) {
     return helm_diag_h2<T>(d, i, j, load_k<T>(d, i, j), load_sig<T>(d, i, j));
+}
+
+// FP64 residual g - A u at an interior node p of a grid of row pitch `pitch`
+// where the diagonal is real (no sponge, no shift): 14 FP64 operations with
+// its |r|^2, where the general form with its boundary terms takes ~28.  The
+// FP64 pipes (two lanes per SM and clock) bound every FP64 residual, not its
+// 56 bytes per node.
+__device__ __forceinline__ double2 helm_residual_in(const double2* __restrict__ u, const double2* __restrict__ g,
+                                                    long long p, int pitch, double k, double h, double ih2) {
+    const double kh = k * h, re = fma(-kh, kh, 4.0);
+    const double2 uc = __ldg(u + p), w = __ldg(u + p - 1), e = __ldg(u + p + 1), s = __ldg(u + p - pitch),
+                  n = __ldg(u + p + pitch), gv = __ldg(g + p);
+    const double sx = (w.x + e.x) + (s.x + n.x), sy = (w.y + e.y) + (s.y + n.y);
+    return make_double2(fma(-ih2, fma(re, uc.x, -sx), gv.x), fma(-ih2, fma(re, uc.y, -sy), gv.y));
 }
 
 // --------------------------------------------------- deterministic reductions

@@ -165,11 +165,11 @@ __global__ void __launch_bounds__(NT) k_fg_matvec(const __grid_constant__ KDesc 
         const int i = (t % ntx) * BX + threadIdx.x, j = (t / ntx) * BY + threadIdx.y;
         if (i >= d.n || j >= d.ny) continue;
         const long long p = (long long)j * d.pitch + i;
-        const cplx<TC> zc = __ldg(z + p);
-        const cplx<TC> s = nbr_sum<TC>(z, d.n, d.ny, d.pitch, i, j, p);
-        const cplx<TC> dg = helm_diag_h2<TC>(d, i, j, __ldg(kf + p), sg ? __ldg(sg + p) : TC(0));
+        const cplx<TC> zc = __ldg(z + p), zero = zero2<TC>();
+        const cplx<TC> zw = i > 0 ? __ldg(z + p - 1) : zero, ze = i < d.n - 1 ? __ldg(z + p + 1) : zero;
+        const cplx<TC> zs = j > 0 ? __ldg(z + p - d.pitch) : zero, zn = j < d.ny - 1 ? __ldg(z + p + d.pitch) : zero;
         zj[p] = zc;
-        w[p] = cscale<TC>(csub<TC>(cmul<TC>(dg, zc), s), ih2);
+        w[p] = helm_diff<TC>(helm_diag4<TC>(d, i, j, __ldg(kf + p), sg ? __ldg(sg + p) : TC(0)), zc, zw, ze, zs, zn, ih2);
     }
 }
 

@@ -956,15 +956,23 @@ __global__ void __launch_bounds__(NT) k_outer_residual(const __grid_constant__ K
     double2* r = slot<double>(d, SD);
     double2 acc[2] = {{0, 0}, {0, 0}};
     double* sc = scalp<double>(d);
+    const bool real = d.bc != BC_SPONGE && !d.has_shift;   // inside the grid the diagonal is real
+    const double* kf = reinterpret_cast<const double*>(d.kf);
     for (int t = c.lb; t < ntx * nty; t += c.nb) {
         const int i = (t % ntx) * BX + threadIdx.x, j = (t / ntx) * BY + threadIdx.y;
         if (i >= d.n || j >= d.ny) continue;
         const long long p = (long long)j * d.pitch + i;
-        double2 gv = __ldg(g + p);
-        double2 v = dsub(gv, helm_apply_pt<double, false>(d, u, i, j));
+        double2 v;
+        if (real && i > 0 && i < d.n - 1 && j > 0 && j < d.ny - 1)
+            v = helm_residual_in(u, g, p, d.pitch, __ldg(kf + p), d.h, d.inv_h2);
+        else
+            v = dsub(__ldg(g + p), helm_apply_pt<double, false>(d, u, i, j));
         r[p] = v;
-        acc[0].x += dabs2(v);
-        if (with_gnorm) acc[1].x += dabs2(gv);
+        acc[0].x = fma(v.y, v.y, fma(v.x, v.x, acc[0].x));
+        if (with_gnorm) {
+            const double2 gv = __ldg(g + p);
+            acc[1].x = fma(gv.y, gv.y, fma(gv.x, gv.x, acc[1].x));
+        }
     }
     block_sum<double2, 2>(acc, sh);
     if (publish_partials<double2, 2>(partp<double>(d), MAXDOT, d.counter, c.lb, c.nb, acc, &flag)) {

@@ -46,6 +46,12 @@ __global__ void __launch_bounds__(NT) k_residual_norm_na(int n, int ny, double h
         const int i = (t % ntx) * BX + threadIdx.x, j = (t / ntx) * BY + threadIdx.y;
         if (i >= n || j >= ny) continue;
         const long long p = (long long)j * n + i;
+        if (bc != BC_SPONGE && i > 0 && i < n - 1 && j > 0 && j < ny - 1) {
+            const double2 rv = helm_residual_in(u, g, p, n, k[p], h, ih2);
+            r[p] = rv;
+            acc[0].x = fma(rv.y, rv.y, fma(rv.x, rv.x, acc[0].x));
+            continue;
+        }
         const double kk = k[p], kh = kk * h;
         double re = 4.0 - kh * kh, im = 0.0;
         const int miss = (i == 0) + (i == n - 1) + (j == 0) + (j == ny - 1);

@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(32 * RS_WPB) k_prolong_jac_stream(const __grid
         }
         P2<T> ua2 = p2zero<T>(), ua1 = p2zero<T>();   // u at j-2, j-1
         P2<T> ob3 = p2zero<T>(), ob2 = p2zero<T>();   // FG: z at j-3, j-2
-        P2<T> dgp = p2zero<T>();                      // FG: diagonal at j-2
+        P2<T> dgp = p2zero<T>();                      // FG: diagonal less 4 at j-2
         for (int j = j0; j <= j1; ++j) {
             if (j + PS_AH <= j1) issue(j + PS_AH);
             cp_async_commit();
@@ -284,14 +284,16 @@ __global__ void __launch_bounds__(32 * RS_WPB) k_prolong_jac_stream(const __grid
                     const bool ro1 = (unsigned)r1 < (unsigned)ny;
                     o1 = p2sel<T>(o1, ro1 && cin0, ro1 && cin1);
                     const int r2 = j - 2;
-                    const P2<T> w = helm_row<T, false>(dgp, ob2, ob3, o1, ih2);
+                    const cplx<T> zw = shfl_up1<T>(ob2.v1), ze = shfl_dn1<T>(ob2.v0);
+                    const P2<T> w{helm_diff<T>(dgp.v0, ob2.v0, zw, ob2.v1, ob3.v0, o1.v0, ih2),
+                                  helm_diff<T>(dgp.v1, ob2.v1, ob2.v0, ze, ob3.v1, o1.v1, ih2)};
                     if (own && r2 >= y0 && r2 < y1) {
                         const long long p = (long long)r2 * pitch + col;
                         if (cin0) wv[p] = w.v0;
                         if (cin1) wv[p + 1] = w.v1;
                     }
                     ob3 = ob2; ob2 = o1;
-                    dgp = dg;
+                    dgp = P2<T>{helm_diag4<T>(d, col, r1, k0, s0), helm_diag4<T>(d, col + 1, r1, k1, s1)};
                 }
             }
             ua2 = ua1; ua1 = u0;
