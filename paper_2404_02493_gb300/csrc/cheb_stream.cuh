@@ -233,14 +233,8 @@ __global__ void __launch_bounds__(32 * cs_wpb<HS>()) k_cheb_stream(const __grid_
             if constexpr (NS == 1) {
                 if (own && r2 >= y0 && r2 < y1) {
                     const long long p = (long long)r2 * pitch + col;
-                    if (cin0) {
-                        xout[p] = xm1.v0;
-                        if (wd) dout[p] = dm.v0;
-                    }
-                    if (cin1) {
-                        xout[p + 1] = xm1.v1;
-                        if (wd) dout[p + 1] = dm.v1;
-                    }
+                    store_pair<T>(xout, p, xm1, cin0, cin1);
+                    if (wd) store_pair<T>(dout, p, dm, cin0, cin1);
                 }
             } else {
                 const P2<T> xn = E ? p2sel<T>(xm1, ro2 && cin0, ro2 && cin1) : xm1;
@@ -258,16 +252,10 @@ __global__ void __launch_bounds__(32 * cs_wpb<HS>()) k_cheb_stream(const __grid_
                 const P2<T> s2 = helm_row<T, true>(dg4, tb4, tb5, t2, ih2);
                 if (own && r4 >= y0 && r4 < y1) {
                     const long long p = (long long)r4 * pitch + col;
-                    const cplx<T> e0 = cadd<T>(cscale<T>(s2.v0, c2b), cscale<T>(db4.v0, c1b));
-                    const cplx<T> e1 = cadd<T>(cscale<T>(s2.v1, c2b), cscale<T>(db4.v1, c1b));
-                    if (cin0) {
-                        xout[p] = cadd<T>(xb4.v0, e0);
-                        if (wd) dout[p] = e0;
-                    }
-                    if (cin1) {
-                        xout[p + 1] = cadd<T>(xb4.v1, e1);
-                        if (wd) dout[p + 1] = e1;
-                    }
+                    const P2<T> e{cadd<T>(cscale<T>(s2.v0, c2b), cscale<T>(db4.v0, c1b)),
+                                  cadd<T>(cscale<T>(s2.v1, c2b), cscale<T>(db4.v1, c1b))};
+                    store_pair<T>(xout, p, P2<T>{cadd<T>(xb4.v0, e.v0), cadd<T>(xb4.v1, e.v1)}, cin0, cin1);
+                    if (wd) store_pair<T>(dout, p, e, cin0, cin1);
                 }
                 tb5 = t2;
                 xb4 = xn;

@@ -695,24 +695,25 @@ struct Engine : EngineBase {
                ct_smem<T>(I.lv[l - 1].n, I.lv[l - 1].ny, nl, cs, whole) <= ct_smem_limit();
     }
 
+    // Device table of the level chains from the descriptors ds down (maxl
+    // indices per chain, -1 after the coarsest), built once per launch shape.
+    static const int* chain_table(Handle& H, const char* kind, const std::vector<int>& ds, int maxl) {
+        const std::string key = kind + desc_key(ds);
+        auto it = H.tail_first.find(key);
+        if (it != H.tail_first.end()) return it->second;
+        std::vector<int> ch(ds.size() * (size_t)maxl, -1);
+        for (size_t q = 0; q < ds.size(); ++q)
+            for (int k = 0, d = ds[q]; d >= 0 && k < maxl; ++k, d = H.hdesc[(size_t)d].coarse) ch[q * maxl + k] = d;
+        int* dev = (int*)H.alloc(sizeof(int) * ch.size());
+        cudaMemcpy(dev, ch.data(), sizeof(int) * ch.size(), cudaMemcpyHostToDevice);
+        return H.tail_first[key] = dev;
+    }
+
     // One cluster per instance of `tail`: the ADR V-cycle from level l (corr
     // = 0, SAB to SAX), or `corr` whole ADR corrections on level l.
     void launch_adr_cluster(Handle& H, int l, const std::vector<int>& tail, int corr, cudaStream_t st) {
         const std::vector<int> ds = adescs(H, l, tail);
-        const std::string key = "ct" + desc_key(ds);
-        auto it = H.tail_first.find(key);
-        int* dchain = nullptr;
-        if (it == H.tail_first.end()) {
-            std::vector<int> ch(ds.size() * CT_MAXL, -1);
-            for (size_t q = 0; q < ds.size(); ++q)
-                for (int k = 0, d = ds[q]; d >= 0 && k < CT_MAXL; ++k, d = H.hdesc[(size_t)d].coarse)
-                    ch[q * CT_MAXL + k] = d;
-            dchain = (int*)H.alloc(sizeof(int) * ch.size());
-            cudaMemcpy(dchain, ch.data(), sizeof(int) * ch.size(), cudaMemcpyHostToDevice);
-            H.tail_first[key] = dchain;
-        } else {
-            dchain = it->second;
-        }
+        const int* const dchain = chain_table(H, "ct", ds, CT_MAXL);
         const int cs = ct_cluster();
         long long sm = 0, pts = 0, mat = 0, top = 0;
         for (int b : tail) {
@@ -731,9 +732,8 @@ struct Engine : EngineBase {
             cudaLaunchAttribute at[1];
             ct_config(cfg, at, cs, (unsigned)tail.size(), sm, st);
             const LevelDesc* D = H.ddesc;
-            const int* ch = dchain;
-            if (cs == 16) cudaLaunchKernelEx(&cfg, k_adr_cluster<T, 16>, D, ch, corr);
-            else cudaLaunchKernelEx(&cfg, k_adr_cluster<T, 8>, D, ch, corr);
+            if (cs == 16) cudaLaunchKernelEx(&cfg, k_adr_cluster<T, 16>, D, dchain, corr);
+            else cudaLaunchKernelEx(&cfg, k_adr_cluster<T, 8>, D, dchain, corr);
         }, pts);
     }
 
@@ -759,23 +759,14 @@ struct Engine : EngineBase {
     // wave tail: n_l within the bound and its vectors fit one block.
     static bool in_wave_tail(Handle& H, int b, int l) {
         const int n = H.inst[b].lv[l - 1].n, ny = H.inst[b].lv[l - 1].ny;
-        return l >= 4 && H.inst[b].L > l && std::max(n, ny) <= H.wave_tail_nmax && n <= WT_MAXN &&
-               wt_smem<T>(n, ny) <= wt_smem_limit();
+        return l >= 4 && H.inst[b].L > l && H.inst[b].L - l < TS_MAXL && std::max(n, ny) <= H.wave_tail_nmax &&
+               n <= WT_MAXN && ny <= wt_maxny<T>() && wt_smem<T>(n, ny) <= wt_smem_limit();
     }
     // Down / coarsest / up launches of the wave tail for the instances in
     // `tail` (their level l is the first tail level).
     void launch_wave_tail(Handle& H, int l, const std::vector<int>& tail, cudaStream_t st) {
         const std::vector<int> ds = descs(H, l, tail);
-        const std::string key = "wt" + desc_key(ds);
-        auto it = H.tail_first.find(key);
-        int* dfirst = nullptr;
-        if (it == H.tail_first.end()) {
-            dfirst = (int*)H.alloc(sizeof(int) * ds.size());
-            cudaMemcpy(dfirst, ds.data(), sizeof(int) * ds.size(), cudaMemcpyHostToDevice);
-            H.tail_first[key] = dfirst;
-        } else {
-            dfirst = it->second;
-        }
+        const int* const dchain = chain_table(H, "wt", ds, TS_MAXL);
         long long sm = 0, pts = 0;
         for (int b : tail) {
             sm = std::max(sm, wt_smem<T>(H.inst[b].lv[l - 1].n, H.inst[b].lv[l - 1].ny));
@@ -789,11 +780,11 @@ struct Engine : EngineBase {
         const double cheb_zero = (C + R + C) + (q - 2) * (5 * C + R) + (4 * C + R);
         const double cheb_x = (2 * C + R + C) + (q - 2) * (5 * C + R) + (4 * C + R);
         go(H, st, KK_WAVE_TAIL, (cheb_zero + 2 * C + R + C / 4) * (double)pts, [&] {
-            k_wave_down<T><<<nb, WT_THREADS, (size_t)sm, st>>>((const LevelDesc*)H.ddesc, (const int*)dfirst, q);
+            k_wave_down<T><<<nb, WT_THREADS, (size_t)sm, st>>>((const LevelDesc*)H.ddesc, dchain, q);
         }, pts);
         coarse_solve(H, tail, 0, st);   // every depth in one launch
         go(H, st, KK_WAVE_TAIL, (2 * C + C / 4 + cheb_x) * (double)pts, [&] {
-            k_wave_up<T><<<nb, WT_THREADS, (size_t)sm, st>>>((const LevelDesc*)H.ddesc, (const int*)dfirst, q);
+            k_wave_up<T><<<nb, WT_THREADS, (size_t)sm, st>>>((const LevelDesc*)H.ddesc, dchain, q);
         }, pts);
     }
 

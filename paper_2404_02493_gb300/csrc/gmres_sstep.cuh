@@ -448,14 +448,10 @@ __global__ void __launch_bounds__(32 * GS_WPB, sizeof(T) == 4 ? 4 : 1) k_gs_gram
             const P2<T> k3 = sl_row<T>(q0, q1, c1w, c0w, k2, ih2, wh, s, r3 && cin0, r3 && cin1);
             if (own) {
                 if (j - 1 >= gg.y0 && j - 1 < gg.y1) {
-                    const long long p = (long long)(j - 1) * pitch + col;
-                    if (cin0) k1o[p] = k1.v0;
-                    if (cin1) k1o[p + 1] = k1.v1;
+                    store_pair<T>(k1o, (long long)(j - 1) * pitch + col, k1, cin0, cin1);
                 }
                 if (j - 2 >= gg.y0 && j - 2 < gg.y1) {
-                    const long long p = (long long)(j - 2) * pitch + col;
-                    if (cin0) k2o[p] = k2.v0;
-                    if (cin1) k2o[p + 1] = k2.v1;
+                    store_pair<T>(k2o, (long long)(j - 2) * pitch + col, k2, cin0, cin1);
                 }
                 if (r3) {
                     // K0 at j - 3 (issued: j - 3 >= y0 > j0)
@@ -618,17 +614,19 @@ __global__ void __launch_bounds__(NT) k_gs_post(const __grid_constant__ KDesc A,
         const int r = e / npr, q = e - r * npr;
         const long long p = (long long)r * pitch + 2 * q;
         const bool two = 2 * q + 1 < n;
-        const int m = two ? 2 : 1;
-#pragma unroll
-        for (int v = 0; v < 2; ++v) {
-            if (v < m) {
-                cplx<T> x = xzero ? zero2<T>() : __ldg(xo + p + v);
-                x = cfma<T>(c0, __ldg(k0 + p + v), x);
-                x = cfma<T>(c1, __ldg(k1 + p + v), x);
-                x = cfma<T>(c2, __ldg(k2 + p + v), x);
-                if (modulate) u[p + v] = cfma<T>(__ldg(mod + p + v), x, u[p + v]);
-                else xout[p + v] = x;
-            }
+        // (a row's padding follows its last node: the second value of an odd
+        // row's last pair is read there and not written)
+        P2<T> x = xzero ? p2zero<T>() : load_pair<T>(xo, p);
+        const P2<T> a0 = load_pair<T>(k0, p), a1 = load_pair<T>(k1, p), a2 = load_pair<T>(k2, p);
+        x.v0 = cfma<T>(c2, a2.v0, cfma<T>(c1, a1.v0, cfma<T>(c0, a0.v0, x.v0)));
+        x.v1 = cfma<T>(c2, a2.v1, cfma<T>(c1, a1.v1, cfma<T>(c0, a0.v1, x.v1)));
+        if (modulate) {
+            const P2<T> m = load_pair<T>(mod, p), w = load_pair<T>(u, p);
+            x.v0 = cfma<T>(m.v0, x.v0, w.v0);
+            x.v1 = cfma<T>(m.v1, x.v1, w.v1);
+            store_pair<T>(u, p, x, true, two);
+        } else {
+            store_pair<T>(xout, p, x, true, two);
         }
     }
 }

@@ -851,7 +851,9 @@ __global__ void __launch_bounds__(NT) k_prolong(const __grid_constant__ KDesc A,
 
 // ----------------------------------------------------------- modulation
 // b = exp(-i w phi) (g - A u)  at level 2 (eq. Rytov: r_hat = r e^{-i w phi}
-// in the exp(+i w phi) convention); result in slot SAB.
+// in the exp(+i w phi) convention); result in slot SAB.  The Laplacian as a
+// sum of differences (helm_diff): the corrections amplify what rounding leaves
+// in this residual.
 template <typename T>
 __global__ void __launch_bounds__(NT) k_resdemod(const __grid_constant__ KDesc A, const Seg* __restrict__ Sg,
                                                  int nseg, int /*unused*/) {
@@ -866,7 +868,11 @@ __global__ void __launch_bounds__(NT) k_resdemod(const __grid_constant__ KDesc A
         const int i = (t % ntx) * BX + threadIdx.x, j = (t / ntx) * BY + threadIdx.y;
         if (i >= d.n || j >= d.ny) continue;
         const long long p = (long long)j * d.pitch + i;
-        cplx<T> r = csub<T>(__ldg(g + p), helm_apply_pt<T, false>(d, u, i, j));
+        const cplx<T> zero = zero2<T>(), uc = __ldg(u + p);
+        const cplx<T> uw = i > 0 ? __ldg(u + p - 1) : zero, ue = i < d.n - 1 ? __ldg(u + p + 1) : zero;
+        const cplx<T> us = j > 0 ? __ldg(u + p - d.pitch) : zero, un = j < d.ny - 1 ? __ldg(u + p + d.pitch) : zero;
+        const cplx<T> dg = helm_diag4<T>(d, i, j, load_k<T>(d, i, j), load_sig<T>(d, i, j));
+        const cplx<T> r = csub<T>(__ldg(g + p), helm_diff<T>(dg, uc, uw, ue, us, un, LC<T>::ih2(d)));
         b[p] = cmulc<T>(__ldg(mod + p), r);
     }
 }

@@ -103,9 +103,7 @@ __global__ void __launch_bounds__(32 * RS_WPB) k_restrict_jac0_stream(const __gr
                               (g0.v1.y * dg0.v1.x - g0.v1.x * dg0.v1.y) * a1);
             }
             if (own && j >= fy0 && j < fy1) {
-                const long long p = (long long)j * pitch + col;
-                if (cin0) xs[p] = u0.v0;
-                if (cin1) xs[p + 1] = u0.v1;
+                store_pair<T>(xs, (long long)j * pitch + col, u0, cin0, cin1);
             }
             // r = g - A u1 at row j - 1
             P2<T> rr;
@@ -275,9 +273,7 @@ __global__ void __launch_bounds__(32 * RS_WPB) k_prolong_jac_stream(const __grid
                                                   (rr.v1.y * dg.v1.x - rr.v1.x * dg.v1.y) * a));
                 }
                 if (wr1) {
-                    const long long p = (long long)r1 * pitch + col;
-                    if (cin0) os[p] = o1.v0;
-                    if (cin1) os[p + 1] = o1.v1;
+                    store_pair<T>(os, (long long)r1 * pitch + col, o1, cin0, cin1);
                 }
                 if constexpr (FG) {
                     // W = A z at row j - 2 (z zero outside the grid)
@@ -288,9 +284,7 @@ __global__ void __launch_bounds__(32 * RS_WPB) k_prolong_jac_stream(const __grid
                     const P2<T> w{helm_diff<T>(dgp.v0, ob2.v0, zw, ob2.v1, ob3.v0, o1.v0, ih2),
                                   helm_diff<T>(dgp.v1, ob2.v1, ob2.v0, ze, ob3.v1, o1.v1, ih2)};
                     if (own && r2 >= y0 && r2 < y1) {
-                        const long long p = (long long)r2 * pitch + col;
-                        if (cin0) wv[p] = w.v0;
-                        if (cin1) wv[p + 1] = w.v1;
+                        store_pair<T>(wv, (long long)r2 * pitch + col, w, cin0, cin1);
                     }
                     ob3 = ob2; ob2 = o1;
                     dgp = P2<T>{helm_diag4<T>(d, col, r1, k0, s0), helm_diag4<T>(d, col + 1, r1, k1, s1)};

@@ -56,6 +56,31 @@ struct P2 {
 };
 template <typename T> __device__ __forceinline__ P2<T> p2zero() { return P2<T>{zero2<T>(), zero2<T>()}; }
 
+// Store the lane's pair at element p (even: a 16-byte boundary in FP32) of a
+// row, c0 / c1: its columns are in the grid (c1 implies c0).  One 16-byte
+// store per lane: two 8-byte stores at a stride of 16 bytes wrote every
+// 32-byte sector twice, half at a time.
+template <typename T>
+__device__ __forceinline__ void store_pair(cplx<T>* __restrict__ a, long long p, const P2<T>& v, bool c0, bool c1) {
+    if constexpr (std::is_same<T, float>::value) {
+        if (c1) *reinterpret_cast<float4*>(a + p) = make_float4(v.v0.x, v.v0.y, v.v1.x, v.v1.y);
+        else if (c0) a[p] = v.v0;
+    } else {
+        if (c0) a[p] = v.v0;
+        if (c1) a[p + 1] = v.v1;
+    }
+}
+
+template <typename T>
+__device__ __forceinline__ P2<T> load_pair(const cplx<T>* a, long long p) {
+    if constexpr (std::is_same<T, float>::value) {
+        const float4 v = *reinterpret_cast<const float4*>(a + p);
+        return P2<T>{make_float2(v.x, v.y), make_float2(v.z, v.w)};
+    } else {
+        return P2<T>{a[p], a[p + 1]};
+    }
+}
+
 // Copy row r of an array of ny rows of n (pitch) into ring slot r & (DEP-1)
 // of this lane's two columns; zero outside the grid.
 template <typename E>

@@ -228,9 +228,9 @@ __global__ void __launch_bounds__(CT_THREADS, 1) k_adr_cluster(const LevelDesc* 
             over(l, 0, 0,
                  [&](int o, int row, int c) {
                      const long long p = (long long)row * d0.pitch + c;
-                     const cplx<T> dg = helm_diag_at<T>(d0, c, row);
-                     const cplx<T> sn = cadd<T>(cadd<T>(U[o - 1], U[o + 1]), cadd<T>(U[o - W], U[o + W]));
-                     const cplx<T> r = csub<T>(__ldg(g + p), cscale<T>(csub<T>(cmul<T>(dg, U[o]), sn), l.ih2));
+                     const cplx<T> dg = helm_diag4<T>(d0, c, row, load_k<T>(d0, c, row), load_sig<T>(d0, c, row));
+                     const cplx<T> r = csub<T>(__ldg(g + p), helm_diff<T>(dg, U[o], U[o - 1], U[o + 1], U[o - W],
+                                                                          U[o + W], l.ih2));
                      l.B[o] = cmulc<T>(__ldg(mod + p), r);
                  },
                  none);

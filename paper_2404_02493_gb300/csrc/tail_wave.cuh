@@ -15,11 +15,21 @@
 //                (e the result of level l+1), q Chebyshev steps from x', the
 //                result to the level's SU slot
 //
+// What bounds it: 20 dependent stencil passes per level in one block, each its
+// SM's shared-memory traffic and a barrier.  A thread owns WT_RPT rows of a
+// column: x, d, g and the diagonal of its nodes stay in registers, north and
+// south neighbours inside its rows too, and the two shared vectors (x, the
+// residual t) have a zero border, so a pass loads 2.5 values per node and
+// stores one.  With every operand in shared memory, a test per neighbour, the
+// step coefficients read from global memory inside the chain and the level
+// chain followed pointer by pointer the two launches took 29 and 26 us for
+// levels of 63 and 31; now 21 and 19 us (of which ~5 are the launch and the first loads).
+//
 // Slots and per-node arithmetic are those of the multi-launch path
 // (k_cheb_step, k_restrict<MODE_HELM>, k_prolong<PMODE_ADD>); the Chebyshev
-// direction lives in shared memory only (the first step of a smoothing does
-// not read it).  Only block barriers are used; every thread runs the same
-// level loop.
+// direction lives in registers only (the first step of a smoothing does not
+// read it).  Only block barriers are used; every thread runs the same level
+// loop.
 #pragma once
 #include "kernels.cuh"
 
@@ -27,167 +37,159 @@ namespace wadr {
 
 constexpr int TS_MAXL = 8;    // levels of a chain, the coarsest included
 constexpr int WT_THREADS = 1024;
-constexpr int WT_MAXN = 64;   // nodes map to threads as 64 columns x 16 rows
+constexpr int WT_MAXN = 64;   // columns; nodes map to threads as 64 columns x 16 groups of rows
+// rows per thread (64 registers a thread at 1024 threads)
+template <typename T> __host__ __device__ constexpr int wt_rpt() { return sizeof(T) == 4 ? 4 : 2; }
+template <typename T> __host__ __device__ constexpr int wt_maxny() { return WT_THREADS / WT_MAXN * wt_rpt<T>(); }
 
-// for (j, i) over a level of ny rows of n nodes (n <= WT_MAXN), this
-// thread's nodes
-#define WT_FOR_NODES(n, ny, i, j)                                                  \
-    for (int j = (int)(threadIdx.x >> 6), i = (int)(threadIdx.x & 63); j < (ny); \
-         j += WT_THREADS / WT_MAXN)                                                \
-        if (i < (n))
-
-// dynamic shared memory for a first level of n x ny nodes: x, the Chebyshev
-// direction, the residual t, the diagonal of A, g of the even levels (n ny)
-// and g / x of the odd levels ((n/2)(ny/2))
+// dynamic shared memory for a first level of n x ny nodes: x and t with a
+// zero border, and the next level's vector (right-hand side going down,
+// solution with a zero border coming up)
 template <typename T> __host__ __device__ constexpr long long wt_smem(int n, int ny) {
-    return (long long)sizeof(cplx<T>) * (5LL * n * ny + (long long)(n / 2) * (ny / 2));
+    return (long long)sizeof(cplx<T>) * (2LL * (n + 2) * (ny + 2) + (long long)(n / 2 + 2) * (ny / 2 + 2));
 }
 
-// The level chain of this block's instance from first[blockIdx.x] down to
-// the coarsest level, descriptors copied to shared memory; returns the
-// number of levels (>= 2: at least one tail level and the coarsest).
-__device__ __forceinline__ int ts_chain(const LevelDesc* __restrict__ D, const int* __restrict__ first, LevelDesc* Lv,
-                                        int* didx, int* nlev) {
-    if (threadIdx.x == 0) {
-        int di = first[blockIdx.x];
-        int k = 0;
-        while (di >= 0 && k < TS_MAXL) {
-            didx[k++] = di;
-            di = D[di].coarse;
-        }
-        *nlev = k;
-    }
+// The level chain of this block's instance (TS_MAXL descriptor indices, -1
+// after the coarsest), its descriptors and Chebyshev coefficients in shared
+// memory; returns the number of levels.
+template <typename T>
+__device__ __forceinline__ int wt_chain(const LevelDesc* __restrict__ D, const int* __restrict__ chain, LevelDesc* Lv,
+                                        int* didx, T (*cc)[2][16]) {
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    if (tid < TS_MAXL) didx[tid] = chain[blockIdx.x * TS_MAXL + tid];
     __syncthreads();
-    constexpr int W = (int)(sizeof(LevelDesc) / sizeof(unsigned long long));
-    static_assert(sizeof(LevelDesc) % sizeof(unsigned long long) == 0, "descriptor size");
-    const int nl = *nlev;
-    for (int e = threadIdx.x; e < nl * W; e += blockDim.x) {
-        const int k = e / W, w = e - k * W;
-        reinterpret_cast<unsigned long long*>(&Lv[k])[w] = reinterpret_cast<const unsigned long long*>(D + didx[k])[w];
+    int nl = 0;
+    while (nl < TS_MAXL && didx[nl] >= 0) ++nl;
+    for (int k = w; k < nl; k += WT_THREADS / 32) copy_desc(Lv[k], D + didx[k], lane);
+    __syncthreads();
+    for (int e = tid; e < nl * 32; e += WT_THREADS) {
+        const int k = e >> 5, c = (e >> 4) & 1, m = e & 15;
+        cc[k][c][m] = scalp<T>(Lv[k])[(c ? S::CHEB_C2 : S::CHEB_C1) + m];
     }
     __syncthreads();
     return nl;
 }
 
-template <typename T>
-__device__ __forceinline__ cplx<T> ts_coarse_at(const cplx<T>* E, int nc, int ncy, int I, int J) {
-    return ((unsigned)I < (unsigned)nc && (unsigned)J < (unsigned)ncy) ? E[J * nc + I] : zero2<T>();
-}
+// One thread's nodes of a level: rows j0 .. j0 + RPT - 1 of column i.
+template <typename T> struct WtNodes {
+    static constexpr int RPT = wt_rpt<T>();
+    cplx<T> x[RPT], g[RPT], dg[RPT];
+    int i, j0, W;
+    bool in[RPT];
+    __device__ __forceinline__ void place(const LevelDesc& d) {
+        i = threadIdx.x & (WT_MAXN - 1);
+        j0 = (threadIdx.x / WT_MAXN) * RPT;
+        W = d.n + 2;
+#pragma unroll
+        for (int r = 0; r < RPT; ++r) {
+            in[r] = i < d.n && j0 + r < d.ny;
+            x[r] = g[r] = dg[r] = zero2<T>();
+        }
+    }
+    __device__ __forceinline__ int at(int r) const { return (j0 + r + 1) * W + i + 1; }
+    // sum of the four neighbours of row r: own rows in v, the others in V
+    __device__ __forceinline__ cplx<T> nsum(const cplx<T> (&v)[RPT], const cplx<T>* V, int r) const {
+        const int p = at(r);
+        const cplx<T> s = r > 0 ? v[r > 0 ? r - 1 : 0] : V[p - W];
+        const cplx<T> n = r < RPT - 1 ? v[r < RPT - 1 ? r + 1 : 0] : V[p + W];
+        return cadd<T>(cadd<T>(V[p - 1], V[p + 1]), cadd<T>(s, n));
+    }
+    // t = g - A x, to the shared vector Tt
+    __device__ __forceinline__ void residual(cplx<T> (&t)[RPT], const cplx<T>* X, cplx<T>* Tt, T ih2, bool xz) const {
+#pragma unroll
+        for (int r = 0; r < RPT; ++r) {
+            t[r] = g[r];
+            if (!xz && in[r]) t[r] = csub<T>(g[r], cscale<T>(csub<T>(cmul<T>(dg[r], x[r]), nsum(x, X, r)), ih2));
+            if (in[r]) Tt[at(r)] = t[r];
+        }
+    }
+};
 
-// DG = h^2 diag(A) of level d (eq. A1's diagonal with the boundary terms)
+// q Chebyshev steps on a level: s = A^H t, t = g - A x; d = c2[m] s + c1[m] d
+// (c1[0] = 0); x += d.  x of the nodes in registers and (unless xzero) in X.
 template <typename T>
-__device__ __forceinline__ void wt_diag(const LevelDesc& d, cplx<T>* DG) {
-    const int n = d.n, ny = d.ny;
-    WT_FOR_NODES(n, ny, i, j) DG[j * n + i] = helm_diag_h2<T>(d, i, j, load_k<T>(d, i, j), load_sig<T>(d, i, j));
-}
-
-// the four in-grid neighbours of node q of the dense vector S (ny rows of n;
-// zero outside)
-template <typename T>
-__device__ __forceinline__ cplx<T> wt_nsum(const cplx<T>* S, int n, int ny, int i, int j, int q) {
-    const cplx<T> z = zero2<T>();
-    return cadd<T>(cadd<T>(i > 0 ? S[q - 1] : z, i < n - 1 ? S[q + 1] : z),
-                   cadd<T>(j > 0 ? S[q - n] : z, j < ny - 1 ? S[q + n] : z));
-}
-
-// q Chebyshev steps on level d: X (x; zero on entry when xzero), G (g), Dv
-// (direction), Tt (residual), DG (h^2 diag A).  Step m: t = g - A x,
-// s = A^H t, d = c2[m] s + c1[m] d (c1[0] = 0), x += d.
-template <typename T>
-__device__ void wt_cheb(const LevelDesc& d, int q, bool xzero, cplx<T>* X, const cplx<T>* G, cplx<T>* Dv, cplx<T>* Tt,
-                        const cplx<T>* DG) {
-    const int n = d.n, ny = d.ny;
-    const T ih2 = LC<T>::ih2(d);
-    const T* scl = scalp<T>(d);
+__device__ __forceinline__ void wt_cheb(WtNodes<T>& N, int q, bool xzero, cplx<T>* X, cplx<T>* Tt, T ih2,
+                                        const T (*c)[16]) {
+    constexpr int RPT = WtNodes<T>::RPT;
+    cplx<T> d[RPT], t[RPT];
+#pragma unroll
+    for (int r = 0; r < RPT; ++r) d[r] = zero2<T>();
     for (int m = 0; m < q; ++m) {
-        const bool xz = xzero && m == 0;
-        WT_FOR_NODES(n, ny, i, j) {
-            const int p = j * n + i;
-            cplx<T> tv = G[p];
-            if (!xz) {
-                const cplx<T> sn = wt_nsum<T>(X, n, ny, i, j, p);
-                tv = csub<T>(tv, cscale<T>(csub<T>(cmul<T>(DG[p], X[p]), sn), ih2));
-            }
-            Tt[p] = tv;
-        }
+        N.residual(t, X, Tt, ih2, xzero && m == 0);
         __syncthreads();
-        const T c1 = scl[S::CHEB_C1 + m], c2 = scl[S::CHEB_C2 + m];
-        WT_FOR_NODES(n, ny, i, j) {
-            const int p = j * n + i;
-            const cplx<T> sn = wt_nsum<T>(Tt, n, ny, i, j, p);
-            cplx<T> dg = DG[p];
-            dg.y = -dg.y;
-            const cplx<T> sv = cscale<T>(csub<T>(cmul<T>(dg, Tt[p]), sn), ih2);
-            cplx<T> dn = cscale<T>(sv, c2);
-            if (c1 != T(0)) dn = cadd<T>(dn, cscale<T>(Dv[p], c1));
-            const cplx<T> xv = xz ? zero2<T>() : X[p];
-            X[p] = cadd<T>(xv, dn);
-            Dv[p] = dn;
-        }
+        const T c1 = c[0][m], c2 = c[1][m];
+#pragma unroll
+        for (int r = 0; r < RPT; ++r)
+            if (N.in[r]) {
+                cplx<T> dg = N.dg[r];
+                dg.y = -dg.y;
+                const cplx<T> sv = cscale<T>(csub<T>(cmul<T>(dg, t[r]), N.nsum(t, Tt, r)), ih2);
+                cplx<T> dn = cscale<T>(sv, c2);
+                if (c1 != T(0)) dn = cadd<T>(dn, cscale<T>(d[r], c1));
+                d[r] = dn;
+                N.x[r] = cadd<T>(N.x[r], dn);
+                X[N.at(r)] = N.x[r];
+            }
         __syncthreads();
     }
+}
+
+// zero the borders (and everything else) of the two shared vectors of a level
+template <typename T> __device__ __forceinline__ void wt_zero(cplx<T>* X, cplx<T>* Tt, const LevelDesc& d) {
+    const int e = (d.n + 2) * (d.ny + 2);
+    for (int q = threadIdx.x; q < e; q += WT_THREADS) X[q] = Tt[q] = zero2<T>();
 }
 
 // ------------------------------------------------------------ down
 template <typename T>
 __global__ void __launch_bounds__(WT_THREADS, 1) k_wave_down(const LevelDesc* __restrict__ D,
-                                                             const int* __restrict__ first, int q) {
+                                                             const int* __restrict__ chain, int q) {
     extern __shared__ __align__(16) unsigned char wt_smem_raw[];
     __shared__ LevelDesc Lv[TS_MAXL];
     __shared__ int didx[TS_MAXL];
-    __shared__ int nlev;
-    const int nl = ts_chain(D, first, Lv, didx, &nlev);
-    const int n0 = Lv[0].n, ny0 = Lv[0].ny, N0 = n0 * ny0;
-    cplx<T>* X = reinterpret_cast<cplx<T>*>(wt_smem_raw);
-    cplx<T>* Dv = X + N0;
-    cplx<T>* Tt = Dv + N0;
-    cplx<T>* DG = Tt + N0;
-    cplx<T>* GA = DG + N0;      // g of levels l0, l0+2, ...
-    cplx<T>* GB = GA + N0;      // g of levels l0+1, l0+3, ... ((n0/2)(ny0/2) values)
-    {
-        const LevelDesc& d = Lv[0];
-        const cplx<T>* g = slot<T>(d, SG);
-        WT_FOR_NODES(n0, ny0, i, j) GA[j * n0 + i] = g[(long long)j * d.pitch + i];
-    }
+    __shared__ T cc[TS_MAXL][2][16];
+    const int nl = wt_chain<T>(D, chain, Lv, didx, cc);
+    const int E0 = (Lv[0].n + 2) * (Lv[0].ny + 2);
+    cplx<T>* const X = reinterpret_cast<cplx<T>*>(wt_smem_raw);
+    cplx<T>* const Tt = X + E0;
+    cplx<T>* const Gn = Tt + E0;       // the next level's right-hand side
+    constexpr int RPT = WtNodes<T>::RPT;
     for (int k = 0; k + 1 < nl; ++k) {
         const LevelDesc& d = Lv[k];
         const LevelDesc& dc = Lv[k + 1];
-        const int n = d.n, ny = d.ny;
-        const cplx<T>* G = (k & 1) ? GB : GA;
-        cplx<T>* Gn = (k & 1) ? GA : GB;
-        wt_diag<T>(d, DG);
-        __syncthreads();
-        wt_cheb<T>(d, q, true, X, G, Dv, Tt, DG);
-        // x to SU; r = g - A x over Tt
-        {
-            const T ih2 = LC<T>::ih2(d);
-            cplx<T>* xs = slot<T>(d, SU);
-            WT_FOR_NODES(n, ny, i, j) {
-                const int p = j * n + i;
-                xs[(long long)j * d.pitch + i] = X[p];
-                const cplx<T> sn = wt_nsum<T>(X, n, ny, i, j, p);
-                Tt[p] = csub<T>(G[p], cscale<T>(csub<T>(cmul<T>(DG[p], X[p]), sn), ih2));
+        const T ih2 = LC<T>::ih2(d);
+        WtNodes<T> N;
+        N.place(d);
+        const cplx<T>* gg = slot<T>(d, SG);
+#pragma unroll
+        for (int r = 0; r < RPT; ++r)
+            if (N.in[r]) {
+                N.g[r] = k == 0 ? gg[(long long)(N.j0 + r) * d.pitch + N.i] : Gn[(N.j0 + r) * d.n + N.i];
+                N.dg[r] = helm_diag_at<T>(d, N.i, N.j0 + r);
             }
-        }
+        wt_zero<T>(X, Tt, d);
         __syncthreads();
-        {
-            // full weighting (1/16)[1 2 1; 2 4 2; 1 2 1] of r; coarse node I on fine node 2I+1
-            const int nc = dc.n, ncy = dc.ny;
-            cplx<T>* gc = slot<T>(dc, SG);
-            const cplx<T> z = zero2<T>();
-            WT_FOR_NODES(nc, ncy, I, J) {
-                const int fi = 2 * I + 1, fj = 2 * J + 1, b = fj * n + fi;
-                const bool e_in = fi + 1 < n, n_in = fj + 1 < ny;
-                const cplx<T> s4 = Tt[b];
-                const cplx<T> s2 = cadd<T>(cadd<T>(Tt[b - 1], e_in ? Tt[b + 1] : z),
-                                           cadd<T>(Tt[b - n], n_in ? Tt[b + n] : z));
-                const cplx<T> s1 = cadd<T>(cadd<T>(Tt[b - n - 1], e_in ? Tt[b - n + 1] : z),
-                                           cadd<T>(n_in ? Tt[b + n - 1] : z, (e_in && n_in) ? Tt[b + n + 1] : z));
-                const cplx<T> v = cscale<T>(cadd<T>(cadd<T>(cscale<T>(s4, T(4)), cscale<T>(s2, T(2))), s1), T(0.0625));
+        wt_cheb<T>(N, q, true, X, Tt, ih2, cc[k]);
+        // x to SU; r = g - A x
+        cplx<T>* xs = slot<T>(d, SU);
+        cplx<T> t[RPT];
+#pragma unroll
+        for (int r = 0; r < RPT; ++r)
+            if (N.in[r]) xs[(long long)(N.j0 + r) * d.pitch + N.i] = N.x[r];
+        N.residual(t, X, Tt, ih2, false);
+        __syncthreads();
+        // full weighting (1/16)[1 2 1; 2 4 2; 1 2 1] of r; coarse node I on fine node 2I+1
+        const int nc = dc.n, ncy = dc.ny, W = N.W;
+        cplx<T>* gc = slot<T>(dc, SG);
+        for (int J = threadIdx.x / WT_MAXN, I = N.i; J < ncy; J += WT_THREADS / WT_MAXN)
+            if (I < nc) {
+                const cplx<T>* b = Tt + (2 * J + 2) * W + 2 * I + 2;
+                const cplx<T> s2 = cadd<T>(cadd<T>(b[-1], b[1]), cadd<T>(b[-W], b[W]));
+                const cplx<T> s1 = cadd<T>(cadd<T>(b[-W - 1], b[-W + 1]), cadd<T>(b[W - 1], b[W + 1]));
+                const cplx<T> v = cscale<T>(cadd<T>(cadd<T>(cscale<T>(b[0], T(4)), cscale<T>(s2, T(2))), s1), T(0.0625));
                 Gn[J * nc + I] = v;
                 gc[(long long)J * dc.pitch + I] = v;
             }
-        }
         __syncthreads();
     }
 }
@@ -195,61 +197,68 @@ __global__ void __launch_bounds__(WT_THREADS, 1) k_wave_down(const LevelDesc* __
 // ------------------------------------------------------------ up
 template <typename T>
 __global__ void __launch_bounds__(WT_THREADS, 1) k_wave_up(const LevelDesc* __restrict__ D,
-                                                           const int* __restrict__ first, int q) {
+                                                           const int* __restrict__ chain, int q) {
     extern __shared__ __align__(16) unsigned char wt_smem_raw[];
     __shared__ LevelDesc Lv[TS_MAXL];
     __shared__ int didx[TS_MAXL];
-    __shared__ int nlev;
-    const int nl = ts_chain(D, first, Lv, didx, &nlev);
-    const int n0 = Lv[0].n, ny0 = Lv[0].ny, N0 = n0 * ny0;
-    cplx<T>* XA = reinterpret_cast<cplx<T>*>(wt_smem_raw);   // x of levels l0, l0+2, ...
-    cplx<T>* Dv = XA + N0;
-    cplx<T>* Tt = Dv + N0;
-    cplx<T>* DG = Tt + N0;
-    cplx<T>* G = DG + N0;
-    cplx<T>* XB = G + N0;                                     // x of levels l0+1, l0+3, ... ((n0/2)(ny0/2) values)
-    {
-        // the coarsest solution into the buffer of level nl-1
-        const LevelDesc& dL = Lv[nl - 1];
-        const int nL = dL.n, nyL = dL.ny;
-        cplx<T>* XL = ((nl - 1) & 1) ? XB : XA;
-        const cplx<T>* xg = slot<T>(dL, SU);
-        WT_FOR_NODES(nL, nyL, i, j) XL[j * nL + i] = xg[(long long)j * dL.pitch + i];
-    }
+    __shared__ T cc[TS_MAXL][2][16];
+    const int nl = wt_chain<T>(D, chain, Lv, didx, cc);
+    const int E0 = (Lv[0].n + 2) * (Lv[0].ny + 2);
+    cplx<T>* const X = reinterpret_cast<cplx<T>*>(wt_smem_raw);
+    cplx<T>* const Tt = X + E0;
+    cplx<T>* const E = Tt + E0;        // solution of the next coarser level, zero border
+    constexpr int RPT = WtNodes<T>::RPT;
+    for (int e = threadIdx.x; e < (Lv[0].n / 2 + 2) * (Lv[0].ny / 2 + 2); e += WT_THREADS) E[e] = zero2<T>();
     __syncthreads();
+    {
+        const LevelDesc& dL = Lv[nl - 1];
+        const cplx<T>* xg = slot<T>(dL, SU);
+        for (int J = threadIdx.x / WT_MAXN, I = threadIdx.x & (WT_MAXN - 1); J < dL.ny; J += WT_THREADS / WT_MAXN)
+            if (I < dL.n) E[(J + 1) * (dL.n + 2) + I + 1] = xg[(long long)J * dL.pitch + I];
+    }
     for (int k = nl - 2; k >= 0; --k) {
         const LevelDesc& d = Lv[k];
-        const int n = d.n, ny = d.ny, nc = Lv[k + 1].n, ncy = Lv[k + 1].ny;
-        cplx<T>* X = (k & 1) ? XB : XA;
-        const cplx<T>* E = (k & 1) ? XA : XB;             // x of level k+1
-        wt_diag<T>(d, DG);
-        {
-            // x' = x + P e (bilinear; coarse node I on fine node 2I+1); g of the level
-            const cplx<T>* xg = slot<T>(d, SU);
-            const cplx<T>* gg = slot<T>(d, SG);
-            WT_FOR_NODES(n, ny, i, j) {
-                const int ia = (i - 1) >> 1, ja = (j - 1) >> 1;
+        const int Wc = Lv[k + 1].n + 2;
+        const T ih2 = LC<T>::ih2(d);
+        WtNodes<T> N;
+        N.place(d);
+        const cplx<T>* xg = slot<T>(d, SU);
+        const cplx<T>* gg = slot<T>(d, SG);
+#pragma unroll
+        for (int r = 0; r < RPT; ++r)
+            if (N.in[r]) {
+                const long long p = (long long)(N.j0 + r) * d.pitch + N.i;
+                N.x[r] = xg[p];
+                N.g[r] = gg[p];
+                N.dg[r] = helm_diag_at<T>(d, N.i, N.j0 + r);
+            }
+        wt_zero<T>(X, Tt, d);
+        __syncthreads();
+        // x' = x + P e (bilinear; coarse node I on fine node 2I+1)
+#pragma unroll
+        for (int r = 0; r < RPT; ++r)
+            if (N.in[r]) {
+                const int i = N.i, j = N.j0 + r, ia = (i - 1) >> 1, ja = (j - 1) >> 1;
                 const T wa0 = (i & 1) ? T(1) : T(0.5), wa1 = T(1) - wa0;
                 const T wb0 = (j & 1) ? T(1) : T(0.5), wb1 = T(1) - wb0;
-                cplx<T> v = cscale<T>(cadd<T>(cscale<T>(ts_coarse_at<T>(E, nc, ncy, ia, ja), wa0),
-                                              cscale<T>(ts_coarse_at<T>(E, nc, ncy, ia + 1, ja), wa1)), wb0);
-                v = cadd<T>(v, cscale<T>(cadd<T>(cscale<T>(ts_coarse_at<T>(E, nc, ncy, ia, ja + 1), wa0),
-                                                 cscale<T>(ts_coarse_at<T>(E, nc, ncy, ia + 1, ja + 1), wa1)), wb1));
-                const long long pg = (long long)j * d.pitch + i;
-                X[j * n + i] = cadd<T>(xg[pg], v);
-                G[j * n + i] = gg[pg];
+                const cplx<T>* e = E + (ja + 1) * Wc + ia + 1;
+                cplx<T> v = cscale<T>(cadd<T>(cscale<T>(e[0], wa0), cscale<T>(e[1], wa1)), wb0);
+                v = cadd<T>(v, cscale<T>(cadd<T>(cscale<T>(e[Wc], wa0), cscale<T>(e[Wc + 1], wa1)), wb1));
+                N.x[r] = cadd<T>(N.x[r], v);
+                X[N.at(r)] = N.x[r];
             }
-        }
         __syncthreads();
-        wt_cheb<T>(d, q, false, X, G, Dv, Tt, DG);
-        {
-            cplx<T>* xs = slot<T>(d, SU);
-            WT_FOR_NODES(n, ny, i, j) xs[(long long)j * d.pitch + i] = X[j * n + i];
+        wt_cheb<T>(N, q, false, X, Tt, ih2, cc[k]);
+        cplx<T>* xs = slot<T>(d, SU);
+#pragma unroll
+        for (int r = 0; r < RPT; ++r)
+            if (N.in[r]) xs[(long long)(N.j0 + r) * d.pitch + N.i] = N.x[r];
+        if (k > 0) {
+            const int e = (d.n + 2) * (d.ny + 2);
+            for (int p = threadIdx.x; p < e; p += WT_THREADS) E[p] = X[p];   // borders zero as in X
+            __syncthreads();
         }
-        __syncthreads();
     }
 }
-
-#undef WT_FOR_NODES
 
 }  // namespace wadr
