@@ -68,9 +68,10 @@ __global__ void ka_lincomb(int n, int ny, int pitch, double2* out, int acc, cons
 }
 
 // y = base + s op(x), base = b if given, else y (acc) or 0; op: 0 A, 1 A^H,
-// 2 L, 4 L^H.  With z given, also z += x (pointwise).
+// 2 L, 4 L^H.  With z given, also z += x (pointwise); with y2 given, also
+// y2 = s2 y.
 __global__ void ka_apply(LevelDesc d, int op, const double2* x, double2* y, double2 s, int acc, const double2* b,
-                         double2* z) {
+                         double2* z, double2* y2, double s2) {
     int i, j;
     if (!ij_of((long long)blockIdx.x * ANT + threadIdx.x, d.n, d.ny, i, j)) return;
     const long long p = (long long)j * d.pitch + i;
@@ -80,8 +81,23 @@ __global__ void ka_apply(LevelDesc d, int op, const double2* x, double2* y, doub
     else if (op == 2) r = adr_apply_pt<double>(d, x, i, j);
     else r = adr_apply_t_pt<double, true>(d, x, i, j);
     r = dmul(s, r);
-    y[p] = b ? dadd(b[p], r) : (acc ? dadd(y[p], r) : r);
+    r = b ? dadd(b[p], r) : (acc ? dadd(y[p], r) : r);
+    y[p] = r;
+    if (y2) y2[p] = dsc(r, s2);
     if (z) z[p] = dadd(z[p], x[p]);
+}
+
+// One Chebyshev step from t = g - A x: d = c2 A^H t (+ c1 d unless first),
+// xn = x + d (x null: zero).
+__global__ void ka_cheb_update(LevelDesc d, const double2* t, double2* dv, double c1, double c2, int first,
+                               const double2* x, double2* xn) {
+    int i, j;
+    if (!ij_of((long long)blockIdx.x * ANT + threadIdx.x, d.n, d.ny, i, j)) return;
+    const long long p = (long long)j * d.pitch + i;
+    double2 v = dsc(helm_apply_pt<double, true>(d, t, i, j), c2);
+    if (!first) v = dadd(v, dsc(dv[p], c1));
+    dv[p] = v;
+    xn[p] = x ? dadd(x[p], v) : v;
 }
 
 // y (+)= s D^{-1} x  or  s D^{-H} x  (D = Helmholtz diagonal)
@@ -113,9 +129,10 @@ __global__ void ka_restrict(int nf, int nyf, int pf, int nc, int nyc, int pc, co
     y[q] = acc ? dadd(y[q], v) : v;
 }
 
-// y_fine (+)= s P e_coarse  (bilinear)
+// y_fine = base + s P e_coarse  (bilinear; base null: zero).  With z given,
+// also z += y.
 __global__ void ka_prolong(int nf, int nyf, int pf, int nc, int nyc, int pc, const double2* e, double2* y, double s,
-                           int acc) {
+                           const double2* base, double2* z) {
     int i, j;
     if (!ij_of((long long)blockIdx.x * ANT + threadIdx.x, nf, nyf, i, j)) return;
     int ia[2], ja[2];
@@ -130,98 +147,9 @@ __global__ void ka_prolong(int nf, int nyf, int pf, int nc, int nyc, int pc, con
                 v = dadd(v, dsc(e[(long long)ja[q] * pc + ia[r]], wa[r] * wb[q]));
     v = dsc(v, s);
     const long long p = (long long)j * pf + i;
-    y[p] = acc ? dadd(y[p], v) : v;
-}
-
-// up to ADOTS (x, y) vector pairs of a dot-product launch, passed by value;
-// with z[k] set the pair's left vector is x[k] - z[k]
-constexpr int ADOTS = 9;
-struct DotPtrs {
-    const double2* x[ADOTS];
-    const double2* y[ADOTS];
-    const double2* z[ADOTS];
-};
-
-// up to ADOTS dot products sum conj(x_k) y_k into out[k].  FP64 issues at a
-// small fraction of the FP32 rate on this GPU, so the reductions are laid out
-// to spend few FP64 instructions: each thread accumulates many elements (the
-// host launches a few blocks per SM), a warp then transposes its 2 ADOTS
-// partial sums through shared memory and lane l adds up column l (31 adds
-// instead of a 5-level shuffle tree per value), the warps' sums are added in
-// warp order, and the last block to finish (counter) adds the blocks'
-// partials in 8 interleaved groups, then the groups in order.  The order is
-// fixed, so the result is reproducible.
-constexpr int ADV = 2 * ADOTS;   // doubles per thread
-__global__ void __launch_bounds__(ANT) ka_dots(int n, int ny, int pitch, int npair, DotPtrs P, double* part,
-                                               unsigned* count, double2* out) {
-    __shared__ double tr[ANT / 32][32][ADV + 1];
-    __shared__ double ws[ANT / 32][ADV];
-    __shared__ bool last;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    double2 acc[ADOTS];
-#pragma unroll
-    for (int k = 0; k < ADOTS; ++k) acc[k] = make_double2(0, 0);
-    const unsigned N = (unsigned)n * (unsigned)ny, un = (unsigned)n;
-    for (unsigned q = blockIdx.x * ANT + tid; q < N; q += gridDim.x * ANT) {
-        const unsigned j = q / un, i = q - j * un;
-        const long long p = (long long)j * pitch + i;
-#pragma unroll
-        for (int k = 0; k < ADOTS; ++k)
-            if (k < npair) {
-                // a norm pair (x = y) accumulates |x|^2 only, any other pair
-                // Re and Im of conj(x) y, as FMA chains
-                const double2 xv = P.z[k] ? dsub(P.x[k][p], P.z[k][p]) : P.x[k][p];
-                if (P.x[k] == P.y[k] && !P.z[k]) {
-                    acc[k].x = fma(xv.x, xv.x, acc[k].x);
-                    acc[k].x = fma(xv.y, xv.y, acc[k].x);
-                } else {
-                    const double2 yv = P.y[k][p];
-                    acc[k].x = fma(xv.x, yv.x, acc[k].x);
-                    acc[k].x = fma(xv.y, yv.y, acc[k].x);
-                    acc[k].y = fma(xv.x, yv.y, acc[k].y);
-                    acc[k].y = fma(-xv.y, yv.x, acc[k].y);
-                }
-            }
-    }
-#pragma unroll
-    for (int k = 0; k < ADOTS; ++k) {
-        tr[wid][lane][2 * k] = acc[k].x;
-        tr[wid][lane][2 * k + 1] = acc[k].y;
-    }
-    __syncwarp();
-    if (lane < 2 * npair) {
-        double sm = tr[wid][0][lane];
-        for (int r = 1; r < 32; ++r) sm += tr[wid][r][lane];
-        ws[wid][lane] = sm;
-    }
-    __syncthreads();
-    if (tid < 2 * npair) {
-        double sm = ws[0][tid];
-#pragma unroll
-        for (int w = 1; w < ANT / 32; ++w) sm += ws[w][tid];
-        part[(long long)blockIdx.x * ADV + tid] = sm;
-        __threadfence();   // every writer publishes its partial before the count
-    }
-    __syncthreads();
-    if (tid == 0) last = atomicAdd(count, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    // value v = tid % ADV of group g = tid / ADV sums blocks g, g + 8, ...
-    const int v = tid % ADV, g = tid / ADV;
-    if (g < 8 && v < 2 * npair) {
-        double sm = 0.0;
-        for (int b = g; b < (int)gridDim.x; b += 8) sm += __ldcg(&part[(long long)b * ADV + v]);
-        tr[0][g][v] = sm;
-    }
-    __syncthreads();
-    if (tid < 2 * npair) {
-        double sm = tr[0][0][tid];
-#pragma unroll
-        for (int q = 1; q < 8; ++q) sm += tr[0][q][tid];
-        reinterpret_cast<double*>(out)[tid] = sm;
-    }
-    if (tid == 0) *count = 0;
+    if (base) v = dadd(base[p], v);
+    y[p] = v;
+    if (z) z[p] = dadd(z[p], v);
 }
 
 // complex 3 x 3 solve, Gaussian elimination with partial pivoting (largest
@@ -272,14 +200,14 @@ __device__ inline void solve3_dev(const double2 (&G)[3][3], const double2* z, do
 __device__ __forceinline__ double2 dconj(double2 a) { return make_double2(a.x, -a.y); }
 
 // GMRES(3) least squares from the dots d1 = (<w0,w0>, <w0,w1>, <w0,w2>,
-// <w1,w1>, <w1,w2>, <w2,w2>, <w0,r0>, <w1,r0>) and d2 = <w2,r0>: the tape's
+// <w1,w1>, <w1,w2>, <w2,w2>, <w0,r0>, <w1,r0>, <w2,r0>): the tape's
 // scalars t = (c[3], G[9] row-major, z[3], zero flag); c = 0 when r0 = 0.
-__global__ void ka_gm_solve(const double2* d1, const double2* d2, double2* t) {
+__device__ inline void gm_solve(const double2* d1, double2* t) {
     double2 G[3][3];
     G[0][0] = d1[0]; G[0][1] = d1[1]; G[0][2] = d1[2];
     G[1][1] = d1[3]; G[1][2] = d1[4]; G[2][2] = d1[5];
     G[1][0] = dconj(G[0][1]); G[2][0] = dconj(G[0][2]); G[2][1] = dconj(G[1][2]);
-    const double2 z[3] = {d1[6], d1[7], d2[0]};
+    const double2 z[3] = {d1[6], d1[7], d1[8]};
     const bool zero = !(sqrt(dabs2(G[0][0])) > 0);
     double2 c[3] = {make_double2(0, 0), make_double2(0, 0), make_double2(0, 0)};
     if (!zero) solve3_dev(G, z, c);
@@ -297,7 +225,7 @@ __global__ void ka_gm_solve(const double2* d1, const double2* d2, double2* t) {
 //   o[6 + 4q + i]   Gb[i][q] + conj(Gb[q][i])   (wbar_q = sum_i w_i (.) + r0 conj(zb_q))
 //   o[9 + 4q]       conj(zb_q)
 // all zero when the forward sweep had r0 = 0.
-__global__ void ka_gm_back(const double2* t, const double2* cb, double2* o) {
+__device__ inline void gm_back(const double2* t, const double2* cb, double2* o) {
     for (int k = 0; k < 18; ++k) o[k] = make_double2(0, 0);
     if (t[15].x != 0.0) return;
     double2 GH[3][3], c[3], zb[3], Gb[3][3];
@@ -314,6 +242,153 @@ __global__ void ka_gm_back(const double2* t, const double2* cb, double2* o) {
         for (int i = 0; i < 3; ++i) o[6 + 4 * q + i] = dadd(Gb[i][q], dconj(Gb[q][i]));
         o[9 + 4 * q] = dconj(zb[q]);
     }
+}
+
+// What the last block of a dot-product launch does with the sums: nothing
+// more, the GMRES(3) least squares into the tape `to`, its adjoint
+// coefficients from the tape `from` into `to`, or a weight gradient
+// dst += s0 Re out_0 + s1 Re out_1.  (As launches of one thread these took 9
+// to 12 us each.)
+enum DotEnd : int { DOT_SUMS = 0, DOT_SOLVE, DOT_BACK, DOT_ACCUM };
+struct DotTail {
+    int end = DOT_SUMS;
+    const double2* from = nullptr;
+    double2* to = nullptr;
+    double* dst = nullptr;
+    double s0 = 0, s1 = 0;
+};
+
+// up to ADOTS (x, y) vector pairs of a dot-product launch, passed by value
+constexpr int ADOTS = 9;
+struct DotPtrs {
+    const double2* x[ADOTS];
+    const double2* y[ADOTS];
+};
+
+// up to ADOTS dot products sum conj(x_k) y_k into out[k].  FP64 issues at a
+// small fraction of the FP32 rate on this GPU, so the reductions are laid out
+// to spend few FP64 instructions: each thread accumulates many elements (the
+// host launches a few blocks per SM), a warp then transposes its 2 ADOTS
+// partial sums through shared memory and lane l adds up column l (31 adds
+// instead of a 5-level shuffle tree per value), the warps' sums are added in
+// warp order, and the last block to finish (counter) adds the blocks'
+// partials in 8 interleaved groups, then the groups in order.  The order is
+// fixed, so the result is reproducible.
+constexpr int ADV = 2 * ADOTS;   // doubles per thread
+// The end of a dot-product launch: block sums, the last block's totals and
+// tail work.
+__device__ __forceinline__ void dots_end(const double2 (&acc)[ADOTS], int npair, double* part, unsigned* count,
+                                         double2* out, const DotTail& tail, double (*tr)[32][ADV + 1],
+                                         double (*ws)[ADV], bool* last) {
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+#pragma unroll
+    for (int k = 0; k < ADOTS; ++k) {
+        tr[wid][lane][2 * k] = acc[k].x;
+        tr[wid][lane][2 * k + 1] = acc[k].y;
+    }
+    __syncwarp();
+    if (lane < 2 * npair) {
+        double sm = tr[wid][0][lane];
+        for (int r = 1; r < 32; ++r) sm += tr[wid][r][lane];
+        ws[wid][lane] = sm;
+    }
+    __syncthreads();
+    if (tid < 2 * npair) {
+        double sm = ws[0][tid];
+#pragma unroll
+        for (int w = 1; w < ANT / 32; ++w) sm += ws[w][tid];
+        part[(long long)blockIdx.x * ADV + tid] = sm;
+        __threadfence();   // every writer publishes its partial before the count
+    }
+    __syncthreads();
+    if (tid == 0) *last = atomicAdd(count, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!*last) return;
+    __threadfence();
+    // value v = tid % ADV of group g = tid / ADV sums blocks g, g + 8, ...
+    const int v = tid % ADV, g = tid / ADV;
+    if (g < 8 && v < 2 * npair) {
+        double sm = 0.0;
+        for (int b = g; b < (int)gridDim.x; b += 8) sm += __ldcg(&part[(long long)b * ADV + v]);
+        tr[0][g][v] = sm;
+    }
+    __syncthreads();
+    if (tid < 2 * npair) {
+        double sm = tr[0][0][tid];
+#pragma unroll
+        for (int q = 1; q < 8; ++q) sm += tr[0][q][tid];
+        reinterpret_cast<double*>(out)[tid] = sm;
+    }
+    if (tid == 0) *count = 0;
+    if (tail.end == DOT_SUMS) return;
+    __syncthreads();
+    if (tid != 0) return;
+    if (tail.end == DOT_SOLVE) gm_solve(out, tail.to);
+    else if (tail.end == DOT_BACK) gm_back(tail.from, out, tail.to);
+    else tail.dst[0] += tail.s0 * out[0].x + (npair > 1 ? tail.s1 * out[1].x : 0.0);
+}
+
+__global__ void __launch_bounds__(ANT) ka_dots(int n, int ny, int pitch, int npair, DotPtrs P, double* part,
+                                               unsigned* count, double2* out, DotTail tail) {
+    __shared__ double tr[ANT / 32][32][ADV + 1];
+    __shared__ double ws[ANT / 32][ADV];
+    __shared__ bool last;
+    const int tid = threadIdx.x;
+    double2 acc[ADOTS];
+#pragma unroll
+    for (int k = 0; k < ADOTS; ++k) acc[k] = make_double2(0, 0);
+    const unsigned N = (unsigned)n * (unsigned)ny, un = (unsigned)n;
+    for (unsigned q = blockIdx.x * ANT + tid; q < N; q += gridDim.x * ANT) {
+        const unsigned j = q / un, i = q - j * un;
+        const long long p = (long long)j * pitch + i;
+#pragma unroll
+        for (int k = 0; k < ADOTS; ++k)
+            if (k < npair) {
+                // a norm pair (x = y) accumulates |x|^2 only, any other pair
+                // Re and Im of conj(x) y, as FMA chains
+                const double2 xv = P.x[k][p];
+                if (P.x[k] == P.y[k]) {
+                    acc[k].x = fma(xv.x, xv.x, acc[k].x);
+                    acc[k].x = fma(xv.y, xv.y, acc[k].x);
+                } else {
+                    const double2 yv = P.y[k][p];
+                    acc[k].x = fma(xv.x, yv.x, acc[k].x);
+                    acc[k].x = fma(xv.y, yv.y, acc[k].x);
+                    acc[k].y = fma(xv.x, yv.y, acc[k].y);
+                    acc[k].y = fma(-xv.y, yv.x, acc[k].y);
+                }
+            }
+    }
+    dots_end(acc, npair, part, count, out, tail, tr, ws, &last);
+}
+
+// The middle of a reverse Chebyshev step: db = xbar + c db (c = c1[m+1];
+// first: db = xbar) and, with s = A^H t formed here, the weight gradient
+// dst += s0 Re<s, db> + s1 Re<x_m - x_{m-1}, db>.
+__global__ void __launch_bounds__(ANT) ka_cheb_back(LevelDesc d, const double2* t, const double2* xbar, double2* db,
+                                                    double c, int first, const double2* xm, const double2* xp,
+                                                    double* part, unsigned* count, double2* out, DotTail tail) {
+    __shared__ double tr[ANT / 32][32][ADV + 1];
+    __shared__ double ws[ANT / 32][ADV];
+    __shared__ bool last;
+    double2 acc[ADOTS];
+#pragma unroll
+    for (int k = 0; k < ADOTS; ++k) acc[k] = make_double2(0, 0);
+    const unsigned N = (unsigned)d.n * (unsigned)d.ny, un = (unsigned)d.n;
+    for (unsigned q = blockIdx.x * ANT + threadIdx.x; q < N; q += gridDim.x * ANT) {
+        const int j = (int)(q / un), i = (int)(q - (q / un) * un);
+        const long long p = (long long)j * d.pitch + i;
+        double2 v = xbar[p];
+        if (!first) v = dadd(v, dsc(db[p], c));
+        db[p] = v;
+        const double2 s = helm_apply_pt<double, true>(d, t, i, j);
+        acc[0].x = fma(s.y, v.y, fma(s.x, v.x, acc[0].x));
+        if (xm) {
+            const double2 e = xp ? dsub(xm[p], xp[p]) : xm[p];
+            acc[1].x = fma(e.y, v.y, fma(e.x, v.x, acc[1].x));
+        }
+    }
+    dots_end(acc, xm ? 2 : 1, part, count, out, tail, tr, ws, &last);
 }
 
 // out (+)= sum_t c_t x_t with c_t read from device memory (cp_t) when
@@ -355,24 +430,16 @@ __global__ void ka_gm_back_vec(int n, int ny, int pitch, const double2* xbar, co
                         dmul(o[9 + 4 * q], rv));
 }
 
-// dst += scale Re(src)  (weight gradients accumulated on the device)
-__global__ void ka_accum_re(double* dst, const double2* src, double scale) { dst[0] += scale * src[0].x; }
-__global__ void ka_accum_re2(double* dst, const double2* src, double s0, double s1) {
-    dst[0] += s0 * src[0].x;
-    dst[0] += s1 * src[1].x;
-}
-
 // ADR coefficient gradients of y = s L a with cotangent ybar:
-// qbar = (phix_bar, phiy_bar, d_bar.re, d_bar.im) per node.
-// qbar(i, j) += the gradient of Re<ybar, L a> with respect to the node's ADR
-// coefficient quad (phi_x, phi_y, diagonal), yb = s ybar at the node
-__device__ __forceinline__ void adr_grad_pt(const LevelDesc& d, int i, int j, long long p, double2 yb,
-                                            const double2* a, double* qbar) {
+// qbar = (phix_bar, phiy_bar, d_bar.re, d_bar.im) per node; o += the gradient
+// of Re<ybar, L a> with respect to the node's coefficient quad q (phi_x,
+// phi_y, diagonal), yb = s ybar at the node.
+__device__ __forceinline__ void adr_grad_pt(const LevelDesc& d, const quad<double>& q, int i, int j, long long p,
+                                            double2 yb, const double2* a, double (&o)[4]) {
     const int n = d.n;
     const double2 z = make_double2(0, 0);
     const double2 aW = i > 0 ? a[p - 1] : z, aE = i < n - 1 ? a[p + 1] : z;
     const double2 aS = j > 0 ? a[p - d.pitch] : z, aN = j < d.ny - 1 ? a[p + d.pitch] : z;
-    const quad<double> q = reinterpret_cast<const quad<double>*>(d.adr)[p];
     const double wh = d.wh;
     // d(La)/d phix = i wh [(1+sx) aW - (1-sx) aE], sx = sign(phix): the factors
     // are 0, 1 or 2, so the bracket is 2 aW, -2 aE or aW - aE, formed as the sum
@@ -381,7 +448,6 @@ __device__ __forceinline__ void adr_grad_pt(const LevelDesc& d, int i, int j, lo
     const double2 tx = dadd(q.x > 0 ? aW : (q.x < 0 ? nE : aW), q.x > 0 ? aW : nE);
     const double2 ty = dadd(q.y > 0 ? aS : (q.y < 0 ? nN : aS), q.y > 0 ? aS : nN);
     const double2 ac = a[p];
-    double* o = qbar + 4 * ((long long)j * n + i);
     // Re(conj(yb) i wh t) = wh (yb.y t.x - yb.x t.y)
     o[0] = fma(wh, fma(yb.y, tx.x, -yb.x * tx.y), o[0]);
     o[1] = fma(wh, fma(yb.y, ty.x, -yb.x * ty.y), o[1]);
@@ -389,53 +455,107 @@ __device__ __forceinline__ void adr_grad_pt(const LevelDesc& d, int i, int j, lo
     o[2] += db.x;
     o[3] += db.y;
 }
+__device__ __forceinline__ void qbar_add(double* qbar, const LevelDesc& d, int i, int j, const double (&o)[4]) {
+    double* w = qbar + 4 * ((long long)j * d.n + i);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) w[k] += o[k];
+}
 
 __global__ void ka_adr_grad(LevelDesc d, const double2* ybar, const double2* a, double s, double* qbar) {
     int i, j;
     if (!ij_of((long long)blockIdx.x * ANT + threadIdx.x, d.n, d.ny, i, j)) return;
     const long long p = (long long)j * d.pitch + i;
-    adr_grad_pt(d, i, j, p, dsc(ybar[p], s), a, qbar);
+    double o[4] = {0, 0, 0, 0};
+    adr_grad_pt(d, load_adr<double>(d, p), i, j, p, dsc(ybar[p], s), a, o);
+    qbar_add(qbar, d, i, j, o);
 }
 
-// the reverse of y = s L a in one pass: out += s L^H ybar and the ADR
-// coefficient gradient of Re<ybar, s L a> into qbar
-__global__ void ka_lh_grad(LevelDesc d, const double2* ybar, const double2* a, double s, double2* out,
-                           double* qbar) {
+// the reverse of y = s L a in one pass: out = base + s L^H ybar (base null:
+// out itself) and the ADR coefficient gradient of Re<ybar, s L a> into qbar.
+// With out2 given, out2 = out too.
+__global__ void ka_lh_grad(LevelDesc d, const double2* ybar, const double2* a, double s, const double2* base,
+                           double2* out, double2* out2, double* qbar) {
     int i, j;
     if (!ij_of((long long)blockIdx.x * ANT + threadIdx.x, d.n, d.ny, i, j)) return;
     const long long p = (long long)j * d.pitch + i;
-    const double2 r = dmul(make_double2(s, 0), adr_apply_t_pt<double, true>(d, ybar, i, j));
-    out[p] = dadd(out[p], r);
-    adr_grad_pt(d, i, j, p, dsc(ybar[p], s), a, qbar);
+    const double2 v = dadd(base ? base[p] : out[p], dsc(adr_apply_t_pt<double, true>(d, ybar, i, j), s));
+    out[p] = v;
+    if (out2) out2[p] = v;
+    double o[4] = {0, 0, 0, 0};
+    adr_grad_pt(d, load_adr<double>(d, p), i, j, p, dsc(ybar[p], s), a, o);
+    qbar_add(qbar, d, i, j, o);
 }
 
-// demodulation b = conj(m) r:      rbar += m bbar,    mbar += r conj(bbar)
-// modulated update u += m a:       abar  = conj(m) ubar, mbar += conj(a) ubar
-__global__ void ka_mod(LevelDesc d, int mode, const double2* x, const double2* xbar, double2* ybar, double2* mbar) {
+// the same for w_q = L k_q, q = 0..2: kb_q += L^H wb_q
+struct Vec3 { double2* v[3]; };
+struct CVec3 { const double2* v[3]; };
+__global__ void ka_lh_grad3(LevelDesc d, CVec3 wb, CVec3 k, Vec3 kb, double* qbar) {
     int i, j;
     if (!ij_of((long long)blockIdx.x * ANT + threadIdx.x, d.n, d.ny, i, j)) return;
     const long long p = (long long)j * d.pitch + i;
-    const double2 m = reinterpret_cast<const double2*>(d.mod)[p];
-    const long long q = (long long)j * d.n + i;
-    if (mode == 0) {
-        const double2 bb = xbar[p];
-        ybar[p] = dadd(ybar[p], dmul(m, bb));
-        mbar[q] = dadd(mbar[q], dmul(x[p], make_double2(bb.x, -bb.y)));
-    } else {
-        const double2 ub = xbar[p];
-        ybar[p] = dmulc(m, ub);
-        mbar[q] = dadd(mbar[q], dmulc(x[p], ub));
+    const quad<double> q = load_adr<double>(d, p);
+    double2 v[3];
+    double o[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        v[c] = dadd(kb.v[c][p], adr_apply_t_pt<double, true>(d, wb.v[c], i, j));
+        adr_grad_pt(d, q, i, j, p, wb.v[c][p], k.v[c], o);
     }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) kb.v[c][p] = v[c];
+    qbar_add(qbar, d, i, j, o);
 }
-
-// forward modulation: mode 0: out = conj(m) x ; mode 1: out = u + m x
-__global__ void ka_apply_mod(LevelDesc d, int mode, const double2* x, const double2* u, double2* out) {
+// the last link, k_1 = s L k_0 and r0 = k_0: r0b += kb_0 + s L^H kb_1; bbar
+// (+)= r0b (fresh: =)
+__global__ void ka_lh_grad_r0(LevelDesc d, const double2* kb1, const double2* k0, double s, const double2* kb0,
+                              double2* r0b, double2* bbar, int fresh, double* qbar) {
     int i, j;
     if (!ij_of((long long)blockIdx.x * ANT + threadIdx.x, d.n, d.ny, i, j)) return;
     const long long p = (long long)j * d.pitch + i;
-    const double2 m = reinterpret_cast<const double2*>(d.mod)[p];
-    if (mode == 0) out[p] = dmulc(m, x[p]);
-    else out[p] = dadd(u[p], dmul(m, x[p]));
+    const double2 v = dadd(kb0[p], dsc(adr_apply_t_pt<double, true>(d, kb1, i, j), s));
+    const double2 r = dadd(r0b[p], v);
+    r0b[p] = r;
+    bbar[p] = fresh ? r : dadd(bbar[p], r);
+    double o[4] = {0, 0, 0, 0};
+    adr_grad_pt(d, load_adr<double>(d, p), i, j, p, dsc(kb1[p], s), k0, o);
+    qbar_add(qbar, d, i, j, o);
+}
+
+// forward residual and demodulation: r = g - A u, b = conj(m) r
+__global__ void ka_res_demod(LevelDesc d, const double2* u, const double2* g, double2* r, double2* b) {
+    int i, j;
+    if (!ij_of((long long)blockIdx.x * ANT + threadIdx.x, d.n, d.ny, i, j)) return;
+    const long long p = (long long)j * d.pitch + i;
+    const double2 v = dsub(g[p], helm_apply_pt<double, false>(d, u, i, j));
+    r[p] = v;
+    b[p] = dmulc(reinterpret_cast<const double2*>(d.mod)[p], v);
+}
+// forward update: out = u + m a
+__global__ void ka_mod_up(LevelDesc d, const double2* u, const double2* a, double2* out) {
+    int i, j;
+    if (!ij_of((long long)blockIdx.x * ANT + threadIdx.x, d.n, d.ny, i, j)) return;
+    const long long p = (long long)j * d.pitch + i;
+    out[p] = dadd(u[p], dmul(reinterpret_cast<const double2*>(d.mod)[p], a[p]));
+}
+// reverse of the update: abar = conj(m) ubar, mbar += conj(a) ubar
+__global__ void ka_mod_up_back(LevelDesc d, const double2* a, const double2* ub, double2* ab, double2* mbar) {
+    int i, j;
+    if (!ij_of((long long)blockIdx.x * ANT + threadIdx.x, d.n, d.ny, i, j)) return;
+    const long long p = (long long)j * d.pitch + i, q = (long long)j * d.n + i;
+    const double2 u = ub[p];
+    ab[p] = dmulc(reinterpret_cast<const double2*>(d.mod)[p], u);
+    mbar[q] = dadd(mbar[q], dmulc(a[p], u));
+}
+// reverse of the demodulation: rbar = m bbar, mbar += r conj(bbar), gbar += rbar
+__global__ void ka_demod_back(LevelDesc d, const double2* r, const double2* bb, double2* rb, double2* gbar,
+                              double2* mbar) {
+    int i, j;
+    if (!ij_of((long long)blockIdx.x * ANT + threadIdx.x, d.n, d.ny, i, j)) return;
+    const long long p = (long long)j * d.pitch + i, q = (long long)j * d.n + i;
+    const double2 b = bb[p], v = dmul(reinterpret_cast<const double2*>(d.mod)[p], b);
+    rb[p] = v;
+    gbar[p] = dadd(gbar[p], v);
+    mbar[q] = dadd(mbar[q], dmul(r[p], make_double2(b.x, -b.y)));
 }
 
 // y (+)= M x or M^H x with the dense coarsest-level inverse M (N = n ny rows):
@@ -604,9 +724,9 @@ struct Adjoint {
     }
     // y (+)= s op(x); with b: y = b + s op(x); with z: also z += x
     void apply(int l, int op, const double2* x, double2* y, cd s = 1.0, bool acc = false,
-               const double2* b = nullptr, double2* z = nullptr) {
+               const double2* b = nullptr, double2* z = nullptr, double2* y2 = nullptr, double s2 = 0.0) {
         AdjLevel& L = lv[l];
-        ka_apply<<<blocks(L), ANT, 0, st>>>(L.d, op, x, y, make_double2(s.real(), s.imag()), acc, b, z);
+        ka_apply<<<blocks(L), ANT, 0, st>>>(L.d, op, x, y, make_double2(s.real(), s.imag()), acc, b, z, y2, s2);
     }
     void diag(int l, const double2* x, double2* y, bool herm, double s, bool acc) {
         AdjLevel& L = lv[l];
@@ -616,18 +736,21 @@ struct Adjoint {
         AdjLevel &F = lv[l], &Cc = lv[l + 1];
         ka_restrict<<<blocks(Cc), ANT, 0, st>>>(F.n, F.ny, F.pitch, Cc.n, Cc.ny, Cc.pitch, xf, yc, s, acc);
     }
-    void prolong_(int l, const double2* ec, double2* yf, double s, bool acc) {
+    // yf = base + s P ec; z += yf
+    void prolong_(int l, const double2* ec, double2* yf, double s, const double2* base = nullptr,
+                  double2* z = nullptr) {
         AdjLevel &F = lv[l], &Cc = lv[l + 1];
-        ka_prolong<<<blocks(F), ANT, 0, st>>>(F.n, F.ny, F.pitch, Cc.n, Cc.ny, Cc.pitch, ec, yf, s, acc);
+        ka_prolong<<<blocks(F), ANT, 0, st>>>(F.n, F.ny, F.pitch, Cc.n, Cc.ny, Cc.pitch, ec, yf, s, base, z);
     }
     void adr_grad(int l, const double2* ybar, const double2* a, double s) {
         AdjLevel& L = lv[l];
         ka_adr_grad<<<blocks(L), ANT, 0, st>>>(L.d, ybar, a, s, L.qbar);
     }
-    // reverse of y = s L a: out += s L^H ybar, ADR gradient (one pass)
-    void lh_grad(int l, const double2* ybar, const double2* a, double s, double2* out) {
+    // reverse of y = s L a: out = base + s L^H ybar (base null: out), ADR gradient (one pass)
+    void lh_grad(int l, const double2* ybar, const double2* a, double s, double2* out, const double2* base = nullptr,
+                 double2* out2 = nullptr) {
         AdjLevel& L = lv[l];
-        ka_lh_grad<<<blocks(L), ANT, 0, st>>>(L.d, ybar, a, s, out, L.qbar);
+        ka_lh_grad<<<blocks(L), ANT, 0, st>>>(L.d, ybar, a, s, base, out, out2, L.qbar);
     }
     // k device scalars of this reverse step
     double2* scalars(int k) {
@@ -640,8 +763,7 @@ struct Adjoint {
         return p;
     }
     // conj(x_k)^T y_k for up to 8 pairs into device scalars (no synchronisation)
-    double2* dots(int l, std::vector<std::pair<const double2*, const double2*>> pr,
-                  std::vector<const double2*> sub = {}) {
+    double2* dots(int l, std::vector<std::pair<const double2*, const double2*>> pr, const DotTail& tail = DotTail()) {
         AdjLevel& L = lv[l];
         const int np = (int)pr.size();
         if (np > ADOTS) {
@@ -652,11 +774,10 @@ struct Adjoint {
         for (int k = 0; k < ADOTS; ++k) {
             P.x[k] = k < np ? pr[k].first : pr[0].first;
             P.y[k] = k < np ? pr[k].second : pr[0].second;
-            P.z[k] = k < (int)sub.size() ? sub[k] : nullptr;
         }
         const int nb = std::min(blocks(L), 2 * num_sms());
         double2* out = scalars(np);
-        ka_dots<<<nb, ANT, 0, st>>>(L.n, L.ny, L.pitch, np, P, reinterpret_cast<double*>(part), dcount, out);
+        ka_dots<<<nb, ANT, 0, st>>>(L.n, L.ny, L.pitch, np, P, reinterpret_cast<double*>(part), dcount, out, tail);
         return out;
     }
     // out (+)= sum_t cp_t x_t, coefficients in device memory
@@ -728,72 +849,69 @@ struct Adjoint {
         AdjLevel& L = lv[l];
         T.b = b;
         T.x0 = x0;
-        T.r0 = get(l);
         if (x0) {
-            apply(l, 2, x0, T.r0, 1.0);
-            lin(l, T.r0, false, b, 1.0, T.r0, -1.0);
+            T.r0 = get(l);
+            apply(l, 2, x0, T.r0, -1.0, false, b);
         } else {
-            lin(l, T.r0, false, b, 1.0);
+            T.r0 = b;   // (tape vectors are free only after the reverse sweep)
         }
         const double s = L.kscale;
+        T.k[0] = T.r0;
         for (int q = 0; q < 3; ++q) {
-            T.k[q] = get(l);
+            if (q > 0) T.k[q] = get(l);
             T.w[q] = get(l);
         }
-        lin(l, T.k[0], false, T.r0, 1.0);
-        apply(l, 2, T.k[0], T.w[0], 1.0);
-        lin(l, T.k[1], false, T.w[0], s);
-        apply(l, 2, T.k[1], T.w[1], 1.0);
-        lin(l, T.k[2], false, T.w[1], s);
+        // w_q = L k_q, k_{q+1} = s w_q
+        apply(l, 2, T.k[0], T.w[0], 1.0, false, nullptr, nullptr, T.k[1], s);
+        apply(l, 2, T.k[1], T.w[1], 1.0, false, nullptr, nullptr, T.k[2], s);
         apply(l, 2, T.k[2], T.w[2], 1.0);
-        double2* d1 = dots(l, {{T.w[0], T.w[0]}, {T.w[0], T.w[1]}, {T.w[0], T.w[2]}, {T.w[1], T.w[1]},
-                               {T.w[1], T.w[2]}, {T.w[2], T.w[2]}, {T.w[0], T.r0}, {T.w[1], T.r0}, {T.w[2], T.r0}});
-        double2* d2 = d1 + 8;
         T.sc = scalars(16);
-        ka_gm_solve<<<1, 1, 0, st>>>(d1, d2, T.sc);
+        DotTail solve;
+        solve.end = DOT_SOLVE;
+        solve.to = T.sc;
+        dots(l, {{T.w[0], T.w[0]}, {T.w[0], T.w[1]}, {T.w[0], T.w[2]}, {T.w[1], T.w[1]}, {T.w[1], T.w[2]},
+                 {T.w[2], T.w[2]}, {T.w[0], T.r0}, {T.w[1], T.r0}, {T.w[2], T.r0}}, solve);
         // x = x0 + K c
         lin_dev(l, x, false, T.k[0], T.sc + 0, T.k[1], T.sc + 1, T.k[2], T.sc + 2, x0, nullptr, make_double2(1, 0));
     }
 
-    // reverse of gm_forward: xbar given; adds to bbar, x0bar (if x0), ADR gradients
-    // (with r0 = 0 in the forward sweep every coefficient is zero and the
-    // sweep below reduces to x0bar += xbar)
-    void gm_backward(int l, GmTape& T, double2* xbar, double2* bbar, double2* x0bar) {
+    // reverse of gm_forward: xbar given; adds to bbar (fresh: writes it) and
+    // the ADR gradients; x0bar = xbar - L^H r0bar (also to x0bar2) if x0.
+    // (With r0 = 0 in the forward sweep every coefficient is zero and the
+    // sweep below reduces to x0bar = xbar.)
+    void gm_backward(int l, GmTape& T, double2* xbar, double2* bbar, bool fresh, double2* x0bar, double2* x0bar2) {
         AdjLevel& L = lv[l];
         const double s = L.kscale;
         // x = x0 + K c; c = G^{-1} z: zbar = G^{-H} cbar, Gbar = -zbar c^H
-        double2* cb = dots(l, {{T.k[0], xbar}, {T.k[1], xbar}, {T.k[2], xbar}});
         double2* co = scalars(18);
-        ka_gm_back<<<1, 1, 0, st>>>(T.sc, cb, co);
+        DotTail back;
+        back.end = DOT_BACK;
+        back.from = T.sc;
+        back.to = co;
+        dots(l, {{T.k[0], xbar}, {T.k[1], xbar}, {T.k[2], xbar}}, back);
         double2* r0b = get(l);
-        double2* kb[3];
-        double2* wb[3];
+        Vec3 kb, wb;
         for (int q = 0; q < 3; ++q) {
-            kb[q] = get(l);
-            wb[q] = get(l);
+            kb.v[q] = get(l);
+            wb.v[q] = get(l);
         }
         // in one pass over xbar, w_0..w_2, r0:
         //   kbar_j = conj(c_j) xbar;
         //   z_i = w_i^H r0: r0bar = sum_i w_i zbar_i, wbar_i += r0 conj(zbar_i);
         //   G_ij = w_i^H w_j: wbar_j += sum_i w_i Gbar_ij, wbar_i += sum_j w_j conj(Gbar_ij)
-        ka_gm_back_vec<<<blocks(L), ANT, 0, st>>>(L.n, L.ny, L.pitch, xbar, T.w[0], T.w[1], T.w[2], T.r0, co, kb[0],
-                                                     kb[1], kb[2], r0b, wb[0], wb[1], wb[2]);
+        ka_gm_back_vec<<<blocks(L), ANT, 0, st>>>(L.n, L.ny, L.pitch, xbar, T.w[0], T.w[1], T.w[2], T.r0, co, kb.v[0],
+                                                     kb.v[1], kb.v[2], r0b, wb.v[0], wb.v[1], wb.v[2]);
         // w_q = L k_q
-        for (int q = 0; q < 3; ++q) lh_grad(l, wb[q], T.k[q], 1.0, kb[q]);
-        // k_2 = s L k_1, k_1 = s L k_0
-        lh_grad(l, kb[2], T.k[1], s, kb[1]);
-        lh_grad(l, kb[1], T.k[0], s, kb[0]);
-        lin(l, r0b, true, kb[0], 1.0);
-        // r0 = b - L x0 (or b)
-        lin(l, bbar, true, r0b, 1.0);
-        if (T.x0) {
-            lin(l, x0bar, true, xbar, 1.0);
-            lh_grad(l, r0b, T.x0, -1.0, x0bar);
-        }
+        ka_lh_grad3<<<blocks(L), ANT, 0, st>>>(L.d, CVec3{{wb.v[0], wb.v[1], wb.v[2]}},
+                                               CVec3{{T.k[0], T.k[1], T.k[2]}}, kb, L.qbar);
+        // k_2 = s L k_1; k_1 = s L k_0, r0 = k_0 = b - L x0 (or b)
+        lh_grad(l, kb.v[2], T.k[1], s, kb.v[1]);
+        ka_lh_grad_r0<<<blocks(L), ANT, 0, st>>>(L.d, kb.v[1], T.k[0], s, kb.v[0], r0b, bbar, fresh, L.qbar);
+        if (T.x0) lh_grad(l, r0b, T.x0, -1.0, x0bar, xbar, x0bar2);
         put(l, r0b);
         for (int q = 0; q < 3; ++q) {
-            put(l, kb[q]);
-            put(l, wb[q]);
+            put(l, kb.v[q]);
+            put(l, wb.v[q]);
         }
     }
 
@@ -813,50 +931,42 @@ struct Adjoint {
         T->x1 = get(l);
         gm_forward(l, T->pre, b, nullptr, T->x1);
         double2* r = get(l);
-        apply(l, 2, T->x1, r, 1.0);
-        lin(l, r, false, b, 1.0, r, -1.0);
+        apply(l, 2, T->x1, r, -1.0, false, b);
         T->rc = get(l + 1);
         restrict_(l, r, T->rc, 1.0, false);
         put(l, r);
         double2* ec = get(l + 1);
         T->child = adr_forward(l + 1, T->rc, ec);
         T->x2 = get(l);
-        lin(l, T->x2, false, T->x1, 1.0);
-        prolong_(l, ec, T->x2, 1.0, true);
+        prolong_(l, ec, T->x2, 1.0, T->x1);
         gm_forward(l, T->post, b, T->x2, x_out);
         T->x3 = x_out;
         return T;
     }
 
+    // bbar = the cotangent of the right-hand side (written, not added to)
     void adr_backward(AdrTape* T, double2* xbar, double2* bbar) {
         const int l = T->l;
         if (l == I.L) {
             AdjLevel& L = lv[l];
-            // x = X b: bbar += X^H xbar ; L_bar = -bbar_new x^H
-            double2* bb = get(l);
-            ka_gemv<<<(L.n * L.ny + GEMV_ROWS - 1) / GEMV_ROWS, ANT, 0, st>>>(L.n, L.ny, L.pitch, (const double2*)I.lv[l - 1].inv_adr, xbar, bb, 1, 0);
-            lin(l, bbar, true, bb, 1.0);
-            adr_grad(l, bb, T->coarse_x, -1.0);
-            put(l, bb);
+            // x = X b: bbar = X^H xbar ; L_bar = -bbar x^H
+            ka_gemv<<<(L.n * L.ny + GEMV_ROWS - 1) / GEMV_ROWS, ANT, 0, st>>>(L.n, L.ny, L.pitch, (const double2*)I.lv[l - 1].inv_adr, xbar, bbar, 1, 0);
+            adr_grad(l, bbar, T->coarse_x, -1.0);
             return;
         }
-        double2* x2b = get(l);
-        lin(l, x2b, false, nullptr, 0.0);
-        gm_backward(l, T->post, xbar, bbar, x2b);
         // x2 = x1 + P ec
+        double2* x2b = get(l);
         double2* x1b = get(l);
-        lin(l, x1b, false, x2b, 1.0);
+        gm_backward(l, T->post, xbar, bbar, true, x2b, x1b);
         double2* ecb = get(l + 1);
         restrict_(l, x2b, ecb, 4.0, false);       // P^T = 4 R
         double2* rcb = get(l + 1);
-        lin(l + 1, rcb, false, nullptr, 0.0);
         adr_backward(T->child, ecb, rcb);
         // rc = R r, r = b - L x1
         double2* rb = get(l);
-        prolong_(l, rcb, rb, 0.25, false);        // R^T = P/4
-        lin(l, bbar, true, rb, 1.0);
+        prolong_(l, rcb, rb, 0.25, nullptr, bbar);        // R^T = P/4
         lh_grad(l, rb, T->x1, -1.0, x1b);
-        gm_backward(l, T->pre, x1b, bbar, nullptr);
+        gm_backward(l, T->pre, x1b, bbar, false, nullptr, nullptr);
         put(l, x2b);
         put(l, x1b);
         put(l + 1, ecb);
@@ -871,25 +981,17 @@ struct Adjoint {
         cheb_coeffs(l, I.lv[l - 1].alpha, q, c1, c2, d1, d2);
         T.x.assign(q + 1, nullptr);
         T.x[0] = x0;
+        AdjLevel& L = lv[l];
         double2* d = get(l);
-        double2* s = get(l);
         double2* t = get(l);
         for (int m = 0; m < q; ++m) {
-            // s = A^H (g - A x_m)
-            if (T.x[m]) {
-                apply(l, 0, T.x[m], t, 1.0);
-                lin(l, t, false, g, 1.0, t, -1.0);
-            } else {
-                lin(l, t, false, g, 1.0);
-            }
-            apply(l, 1, t, s, 1.0);
-            lin(l, d, false, s, c2[m], m > 0 ? d : nullptr, c1[m]);
+            // t = g - A x_m; d = c2 A^H t + c1 d; x_{m+1} = x_m + d
+            if (T.x[m]) apply(l, 0, T.x[m], t, -1.0, false, g);
             double2* xn = (m == q - 1) ? xout : get(l);
-            lin(l, xn, false, d, 1.0, T.x[m], 1.0);
+            ka_cheb_update<<<blocks(L), ANT, 0, st>>>(L.d, T.x[m] ? t : g, d, c1[m], c2[m], m == 0, T.x[m], xn);
             T.x[m + 1] = xn;
         }
         put(l, d);
-        put(l, s);
         put(l, t);
     }
 
@@ -897,27 +999,25 @@ struct Adjoint {
         const int q = (int)T.x.size() - 1;
         double c1[16], c2[16], d1[16], d2[16];
         cheb_coeffs(l, I.lv[l - 1].alpha, q, c1, c2, d1, d2);
+        AdjLevel& L = lv[l];
         double2* db = get(l);      // d_m bar
-        double2* s = get(l);
         double2* t = get(l);
+        const int nb = std::min(blocks(L), 2 * num_sms());
         for (int m = q - 1; m >= 0; --m) {
             // x_{m+1} = x_m + d_m: d_m bar = x_{m+1} bar + (c1[m+1] d_{m+1} bar, the
             // reverse of d_{m+1} = c1[m+1] d_m + ...); x_m bar = x_{m+1} bar (kept in xbar)
-            if (m == q - 1) lin(l, db, false, xbar, 1.0);
-            else lin(l, db, false, db, c1[m + 1], xbar, 1.0);
-            // s_m = A^H (g - A x_m)
+            // s_m = A^H (g - A x_m); d_m = c1 d_{m-1} + c2 s_m;
+            // alpha_bar += Re<s_m, d_m bar> dc2/dalpha + Re<d_{m-1}, d_m bar> dc1/dalpha,
+            // d_{m-1} = x_m - x_{m-1}
             if (T.x[m]) apply(l, 0, T.x[m], t, -1.0, false, T.g);
-            else lin(l, t, false, T.g, 1.0);
-            apply(l, 1, t, s, 1.0);
-            // d_m = c1 d_{m-1} + c2 s_m; alpha_bar += Re<s_m, d_m bar> dc2/dalpha
-            //                                       + Re<d_{m-1}, d_m bar> dc1/dalpha,
-            // d_{m-1} = x_m - x_{m-1} formed inside the dot launch
-            if (m > 0) {
-                double2* dd = dots(l, {{s, db}, {T.x[m], db}}, {nullptr, T.x[m - 1]});
-                ka_accum_re2<<<1, 1, 0, st>>>(wsum + l, dd, d2[m], d1[m]);
-            } else {
-                ka_accum_re<<<1, 1, 0, st>>>(wsum + l, dots(l, {{s, db}}), d2[m]);
-            }
+            DotTail tail;
+            tail.end = DOT_ACCUM;
+            tail.dst = wsum + l;
+            tail.s0 = d2[m];
+            tail.s1 = d1[m];
+            ka_cheb_back<<<nb, ANT, 0, st>>>(L.d, T.x[m] ? t : T.g, xbar, db, m == q - 1 ? 0.0 : c1[m + 1], m == q - 1,
+                                             m > 0 ? T.x[m] : nullptr, m > 0 ? T.x[m - 1] : nullptr,
+                                             reinterpret_cast<double*>(part), dcount, scalars(2), tail);
             // s = A^H t, t = g - A x_m: t_bar = A s_bar with s_bar = c2 d_m bar;
             // g_bar += t_bar, x_m bar -= A^H t_bar
             apply(l, 0, db, t, c2[m]);
@@ -925,7 +1025,6 @@ struct Adjoint {
             else lin(l, gbar, true, t, 1.0);
         }
         put(l, db);
-        put(l, s);
         put(l, t);
     }
 
@@ -951,8 +1050,7 @@ struct Adjoint {
         double2* t = get(l);
         if (l == 1) {
             T->v1 = get(l);
-            apply(l, 0, u_in, t, 1.0);
-            lin(l, t, false, g, 1.0, t, -1.0);
+            apply(l, 0, u_in, t, -1.0, false, g);
             diag(l, t, T->v1, false, 1.0, false);
             T->u1 = get(l);
             lin(l, T->u1, false, u_in, 1.0, T->v1, wj);
@@ -964,30 +1062,20 @@ struct Adjoint {
             cheb_forward(l, T->pre, nullptr, g, H.p.cheb_iters, u);
         }
         // rc = R (g - A u)
-        if (u) {
-            apply(l, 0, u, t, 1.0);
-            lin(l, t, false, g, 1.0, t, -1.0);
-        } else {
-            lin(l, t, false, g, 1.0);
-        }
+        if (u) apply(l, 0, u, t, -1.0, false, g);
         T->rc = get(l + 1);
-        restrict_(l, t, T->rc, 1.0, false);
+        restrict_(l, u ? t : g, T->rc, 1.0, false);
         double2* ec = get(l + 1);
         T->child = wave_forward(l + 1, nullptr, T->rc, ec);
-        double2* u2 = get(l);
-        if (u) lin(l, u2, false, u, 1.0);
-        else lin(l, u2, false, nullptr, 0.0);
-        prolong_(l, ec, u2, 1.0, true);
+        double2* u2 = l == 3 ? u_out : get(l);
+        prolong_(l, ec, u2, 1.0, u);
         if (l == 1) {
             T->u2 = u2;
             T->v2 = get(l);
-            apply(l, 0, u2, t, 1.0);
-            lin(l, t, false, g, 1.0, t, -1.0);
+            apply(l, 0, u2, t, -1.0, false, g);
             diag(l, t, T->v2, false, 1.0, false);
             lin(l, u_out, false, u2, 1.0, T->v2, wj);
-        } else if (l == 3) {
-            lin(l, u_out, false, u2, 1.0);
-        } else {
+        } else if (l != 3) {
             const bool adr = (l == 2 && H.p.adr && H.p.M > 0 && lv[2].d.adr);
             double2* y = adr ? get(l) : u_out;
             cheb_forward(l, T->post, u2, g, H.p.cheb_iters, y);
@@ -996,15 +1084,12 @@ struct Adjoint {
                 double2* cur = y;
                 for (int m = 0; m < H.p.M; ++m) {
                     double2* r = get(l);
-                    apply(l, 0, cur, r, 1.0);
-                    lin(l, r, false, g, 1.0, r, -1.0);
                     double2* b = get(l);
-                    // b = conj(m) r  (pointwise via the modulation field)
-                    ka_mod_demod(l, r, b);
+                    ka_res_demod<<<blocks(L), ANT, 0, st>>>(L.d, cur, g, r, b);
                     double2* a = get(l);
                     AdrTape* at = adr_forward(2, b, a);
                     double2* nx = (m == H.p.M - 1) ? u_out : get(l);
-                    ka_mod_update(l, cur, a, nx);
+                    ka_mod_up<<<blocks(L), ANT, 0, st>>>(L.d, cur, a, nx);
                     T->corr_u.push_back(cur);
                     T->corr_r.push_back(r);
                     T->corr_adr.push_back(at);
@@ -1016,8 +1101,13 @@ struct Adjoint {
         return T;
     }
 
-    void ka_mod_demod(int l, const double2* r, double2* b);
-    void ka_mod_update(int l, const double2* u, const double2* a, double2* out);
+    DotTail weight_j() const {   // d/d omega_J += Re of the sum
+        DotTail t;
+        t.end = DOT_ACCUM;
+        t.dst = wsum;
+        t.s0 = 1.0;
+        return t;
+    }
 
     // ubar_out given; produces ubar_in (if u_in) and adds to gbar
     void wave_backward(WaveTape* T, double2* uob, double2* uib, double2* gbar) {
@@ -1035,7 +1125,7 @@ struct Adjoint {
         double2* t = get(l);
         if (l == 1) {
             // u_out = u2 + wj v2, v2 = D^{-1}(g - A u2)
-            ka_accum_re<<<1, 1, 0, st>>>(wsum, dots(l, {{T->v2, uob}}), 1.0);
+            dots(l, {{T->v2, uob}}, weight_j());
             lin(l, u2b, false, uob, 1.0);
             diag(l, uob, t, true, wj, false);        // t = wj D^{-H} ubar
             lin(l, gbar, true, t, 1.0);
@@ -1050,16 +1140,12 @@ struct Adjoint {
                 for (int m = (int)T->corr_adr.size() - 1; m >= 0; --m) {
                     // nx = cur + mod a  -> cur_bar = nx_bar, a_bar = conj(mod) nx_bar, mod_bar
                     double2* ab = get(l);
-                    ka_mod_update_back(l, T->corr_adr[m]->x3, curb, ab);
+                    ka_mod_up_back<<<blocks(L), ANT, 0, st>>>(L.d, T->corr_adr[m]->x3, curb, ab, L.mbar);
                     double2* bb = get(l);
-                    lin(l, bb, false, nullptr, 0.0);
                     adr_backward(T->corr_adr[m], ab, bb);
-                    // b = conj(mod) r -> r_bar = mod b_bar, mod_bar += r conj(b_bar)
+                    // b = conj(mod) r -> r_bar = mod b_bar, mod_bar += r conj(b_bar); r = g - A cur
                     double2* rb = get(l);
-                    lin(l, rb, false, nullptr, 0.0);
-                    ka_mod_demod_back(l, T->corr_r[m], bb, rb);
-                    // r = g - A cur
-                    lin(l, gbar, true, rb, 1.0);
+                    ka_demod_back<<<blocks(L), ANT, 0, st>>>(L.d, T->corr_r[m], bb, rb, gbar, L.mbar);
                     apply(l, 1, rb, curb, -1.0, true);
                     put(l, ab);
                     put(l, bb);
@@ -1078,8 +1164,7 @@ struct Adjoint {
         wave_backward(T->child, ecb, nullptr, rcb);
         // rc = R (g - A u)
         double2* rb = get(l);
-        prolong_(l, rcb, rb, 0.25, false);
-        lin(l, gbar, true, rb, 1.0);
+        prolong_(l, rcb, rb, 0.25, nullptr, gbar);
         double2* ub = u2b;    // bar of the pre-smoothed iterate u
         if (l == 3) {
             // u = 0 on entry
@@ -1087,7 +1172,7 @@ struct Adjoint {
             apply(l, 1, rb, ub, -1.0, true);
             if (l == 1) {
                 // u1 = u_in + wj v1, v1 = D^{-1}(g - A u_in)
-                ka_accum_re<<<1, 1, 0, st>>>(wsum, dots(l, {{T->v1, ub}}), 1.0);
+                dots(l, {{T->v1, ub}}, weight_j());
                 if (uib) lin(l, uib, true, ub, 1.0);
                 diag(l, ub, t, true, wj, false);
                 lin(l, gbar, true, t, 1.0);
@@ -1102,9 +1187,6 @@ struct Adjoint {
         put(l + 1, rcb);
         put(l, rb);
     }
-
-    void ka_mod_update_back(int l, const double2* a, const double2* nxb, double2* ab);
-    void ka_mod_demod_back(int l, const double2* r, const double2* bb, double2* rb);
 };
 
 void Adjoint::delete_tape(void* t) {
@@ -1171,23 +1253,6 @@ static void chain_to_phi(const InstHost& I, const std::vector<AdjLevel>& lv, cud
     }
 }
 
-void Adjoint::ka_mod_demod(int l, const double2* r, double2* b) {
-    // b = conj(m) r
-    AdjLevel& L = lv[l];
-    ka_apply_mod<<<blocks(L), ANT, 0, st>>>(L.d, 0, r, nullptr, b);
-}
-void Adjoint::ka_mod_update(int l, const double2* u, const double2* a, double2* out) {
-    AdjLevel& L = lv[l];
-    ka_apply_mod<<<blocks(L), ANT, 0, st>>>(L.d, 1, a, u, out);
-}
-void Adjoint::ka_mod_update_back(int l, const double2* a, const double2* nxb, double2* ab) {
-    AdjLevel& L = lv[l];
-    ka_mod<<<blocks(L), ANT, 0, st>>>(L.d, 1, a, nxb, ab, L.mbar);
-}
-void Adjoint::ka_mod_demod_back(int l, const double2* r, const double2* bb, double2* rb) {
-    AdjLevel& L = lv[l];
-    ka_mod<<<blocks(L), ANT, 0, st>>>(L.d, 0, r, bb, rb, L.mbar);
-}
 
 }  // namespace wadr
 
@@ -1310,14 +1375,17 @@ extern "C" int mg_cycle_backward(mg_handle* h, const void* u0, const void* g, in
         cudaMemcpyAsync(B.ub, B.ubin, bytes, cudaMemcpyDeviceToDevice, ss[b]);
         A.reset();
     };
-    // first step of every instance (eager), then the captured step
+    // first step of every instance (eager), then the captured step; below four
+    // cycles the remaining steps run eagerly too (capturing and instantiating
+    // a step costs more than emitting it twice)
+    const bool replay = K >= 4;
     for (int b = 0; b < ni && !rc; ++b) {
         const size_t bytes = sizeof(double2) * H.inst[b].lv[0].slot_stride;
         cudaMemcpyAsync(bf[b].uin, ck[b][K - 1], bytes, cudaMemcpyDeviceToDevice, ss[b]);
         step(b);
         if (adj[b]->err) rc = adj[b]->err;
     }
-    for (int b = 0; b < ni && !rc && K > 1; ++b) {
+    for (int b = 0; b < ni && !rc && replay; ++b) {
         cudaGraph_t gr = nullptr;
         if (cudaStreamBeginCapture(ss[b], cudaStreamCaptureModeRelaxed) != cudaSuccess) { rc = MG_ECUDA; break; }
         step(b);
@@ -1330,7 +1398,13 @@ extern "C" int mg_cycle_backward(mg_handle* h, const void* u0, const void* g, in
         for (int b = 0; b < ni; ++b) {
             const size_t bytes = sizeof(double2) * H.inst[b].lv[0].slot_stride;
             cudaMemcpyAsync(bf[b].uin, ck[b][k], bytes, cudaMemcpyDeviceToDevice, ss[b]);
-            if (cudaGraphLaunch(gexec[b], ss[b]) != cudaSuccess) { rc = MG_ECUDA; break; }
+            if (!replay) {
+                step(b);
+                if (adj[b]->err) { rc = adj[b]->err; break; }
+            } else if (cudaGraphLaunch(gexec[b], ss[b]) != cudaSuccess) {
+                rc = MG_ECUDA;
+                break;
+            }
         }
     if (rc) {
         const cudaError_t e = cudaGetLastError();
