@@ -34,7 +34,7 @@
 // where four orderings, twice, were swept before; the chain of an update is
 // shortened by integer comparisons, one fused multiply-add per sum and a
 // Goldschmidt square root, and nothing is read from global memory inside it.
-// n = 2047, layered medium: 738 -> 155 us per pass, 59.8 -> 12.4 ms per call.
+// n = 2047, layered medium: 738 -> 130 us per pass, 60.0 -> 10.4 ms per call.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -90,37 +90,38 @@ __global__ void k_eik_init(int n, int ny, double h, const double* __restrict__ s
 }
 
 // Square root of a normal x well inside the exponent range: Goldschmidt's
-// coupled iteration for sqrt(x) and 1/(2 sqrt(x)) from an approximate
-// reciprocal square root, and one residual correction (five dependent
-// operations after the seed; the seed's ~20 bits square twice).
+// coupled iteration from an approximate reciprocal square root (~20 bits,
+// squared once), then one correction by the residual x - g^2 (as many bits
+// again as the seed has): five dependent operations after the seed.
 __device__ __forceinline__ double sqrt_gs(double x) {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    double g = x * y, h = 0.5 * y;
-    const double r = fma(-g, h, 0.5);
-    g = fma(g, r, g);
-    h = fma(h, r, h);
+    const double h = __longlong_as_double(__double_as_longlong(y) - (1ll << 52));   // y / 2
+    double g = x * y;
+    g = fma(g, fma(-g, h, 0.5), g);
     return fma(fma(-g, g, x), h, g);
 }
 
 // Order of two values.  FAST: both are >= 0 (or +inf, NaN last), where
 // doubles order like their bits and an integer comparison takes a few
-// instructions; else the FP64 comparison (~32 ns).
+// instructions; else the FP64 comparison.
 template <bool FAST> __device__ __forceinline__ bool dlt(double a, double b) {
     return FAST ? __double_as_longlong(a) < __double_as_longlong(b) : a < b;
 }
 template <bool FAST> __device__ __forceinline__ double dmin2(double a, double b) { return dlt<FAST>(b, a) ? b : a; }
 
-// Godunov update from the smaller neighbour in x (a) and in y (b), f = s h:
-// one-sided where |a - b| >= f (also with an infinite neighbour).  FAST:
-// values >= 0 and f inside the range of sqrt_gs; without branches, so that
-// independent updates overlap.
-template <bool FAST> __device__ __forceinline__ double godunov_upd(double a, double b, double f) {
-    const double d = a - b;
-    const double one = dmin2<FAST>(a, b) + f;
-    const double rad = fma(-d, d, (2.0 * f) * f);
-    const double two = fma(0.5, FAST ? sqrt_gs(rad) : sqrt(rad), 0.5 * (a + b));
-    return dlt<FAST>(fabs(d), f) ? two : one;
+// Godunov update from the smaller neighbour in x (a) and in y (b), f = s h,
+// r0 = 2 f^2: m + f with m = min(a, b) where |a - b| >= f (also with an
+// infinite neighbour), else m + (|a - b| + sqrt(r0 - (a - b)^2)) / 2.  A warp's
+// FP64 instruction holds its scheduler's pipe for 64 cycles, so their number
+// counts: nine here, without branches so that independent updates overlap.
+// FAST: values >= 0 and f inside the range of sqrt_gs.
+template <bool FAST> __device__ __forceinline__ double godunov_upd(double a, double b, double f, double r0) {
+    const double d = fabs(a - b), m = dmin2<FAST>(a, b), rad = fma(-d, d, r0);
+    const double two = d + (FAST ? sqrt_gs(rad) : sqrt(rad));
+    // twice f: an exponent step (FAST: f is normal)
+    const double one = FAST ? __longlong_as_double(__double_as_longlong(f) + (1ll << 52)) : f + f;
+    return fma(0.5, dlt<FAST>(d, f) ? two : one, m);
 }
 
 // One pass over the active tiles (see the file comment).  act_in[t] != 0:
@@ -133,7 +134,7 @@ __global__ void __launch_bounds__(32) k_eik_pass(int n, int ny, double h, const 
                                                  unsigned char* __restrict__ act_clr, unsigned* nchanged, double tol) {
     // odd distances between the nodes of a diagonal (in 8-byte banks): no conflicts
     __shared__ double T[ET + 2][ET + 2];
-    __shared__ double Fs[ET][ET];
+    __shared__ double Fs[ET][ET], Rs[ET][ET];
     const int lane = threadIdx.x;
     const int ntx = (n + ET - 1) / ET, nty = (ny + ET - 1) / ET;
     for (int t = blockIdx.x; t < ntx * nty; t += gridDim.x) {
@@ -159,7 +160,9 @@ __global__ void __launch_bounds__(32) k_eik_pass(int n, int ny, double h, const 
         for (int r = 0; r < ET; ++r) {
             const int gi = gx0 + lane, gj = gy0 + r;
             const bool in = gi < n && gj < ny;
-            Fs[r][lane] = in ? __dmul_rn(__ldg(&s[(long long)gj * n + gi]), h) : 0.0;
+            const double f = in ? __dmul_rn(__ldg(&s[(long long)gj * n + gi]), h) : 0.0;
+            Fs[r][lane] = f;
+            Rs[r][lane] = (f + f) * f;
             if (in) upd |= 1u << r;
         }
         if (near)
@@ -169,84 +172,125 @@ __global__ void __launch_bounds__(32) k_eik_pass(int n, int ny, double h, const 
             }
         const unsigned updr = __shfl_sync(0xffffffffu, upd, ET - 1 - lane);   // of column 31 - lane
         __syncwarp();
+        // FAST: no negative value in the tile, every f between 1e-140 and 1e140
+        // (by their bits)
+        const long long fl = __double_as_longlong(1e-140), fh = __double_as_longlong(1e140);
+        long long neg = __double_as_longlong(T[0][lane + 1]) | __double_as_longlong(T[ET + 1][lane + 1]) |
+                        __double_as_longlong(T[lane + 1][0]) | __double_as_longlong(T[lane + 1][ET + 1]);
         bool fast = true;
 #pragma unroll 8
-        for (int r = 0; r < ET; ++r)
-            fast = fast && T[r + 1][lane + 1] >= 0.0 && (!((upd >> r) & 1) || (Fs[r][lane] > 1e-140 && Fs[r][lane] < 1e140));
-        fast = fast && T[0][lane + 1] >= 0.0 && T[ET + 1][lane + 1] >= 0.0 && T[lane + 1][0] >= 0.0 &&
-               T[lane + 1][ET + 1] >= 0.0;
-        fast = __all_sync(0xffffffffu, fast);
+        for (int r = 0; r < ET; ++r) {
+            const long long f = __double_as_longlong(Fs[r][lane]);
+            neg |= __double_as_longlong(T[r + 1][lane + 1]);
+            fast = fast && (!((upd >> r) & 1) || (f > fl && f < fh));
+        }
+        fast = __all_sync(0xffffffffu, fast && neg >= 0);
         unsigned left;
         auto visit = [&](auto fc) -> bool {
             constexpr bool FAST = decltype(fc)::value;
-            bool big = false;
-            // vote of node (i, j), if it would decrease: one byte counter per
-            // ordering (bit 0: information from the east, bit 1: from the
-            // north).  A decrease that rounding alone can make (two ulp) does
-            // not vote unless tol is smaller still; one above tol counts as
-            // a change of the tile.
-            auto look = [&](int i, int j, bool ok) -> unsigned {
+            // the nodes that would decrease, by the ordering their information
+            // comes from (bit 0 of the index: from the east, bit 1: from the
+            // north): vote[q] has bit j for row j of the lane's column.  A
+            // decrease that rounding alone can make (two units in the last
+            // place) does not vote unless it exceeds tol; one above tol makes
+            // the tile a changed one (big, looked for until it is known).
+            unsigned vote[4] = {0, 0, 0, 0};
+            bool big = false, known = false;
+            // ordering (0..3) of node (i, j)'s vote, or -1
+            auto look = [&](int i, int j, bool ok) -> int {
                 const double w = T[j + 1][i], e = T[j + 1][i + 2], so = T[j][i + 1], no = T[j + 2][i + 1];
                 const bool fe = dlt<FAST>(e, w), fn = dlt<FAST>(no, so);
                 const double a = fe ? e : w, b = fn ? no : so;
-                const double cur = T[j + 1][i + 1], v = godunov_upd<FAST>(a, b, Fs[j][i]);
-                const double dec = cur - v;
+                const double cur = T[j + 1][i + 1], v = godunov_upd<FAST>(a, b, Fs[j][i], Rs[j][i]);
                 ok = ok && dlt<FAST>(dmin2<FAST>(a, b), EINF) && dlt<FAST>(v, cur);
-                const bool over = ok && (cur >= EINF || dec > tol);
-                big = big || over;
-                return over || (ok && dec > 4.5e-16 * cur) ? 1u << (8 * ((fe ? 1 : 0) + (fn ? 2 : 0))) : 0u;
+                bool yes;
+                if (FAST && known) {
+                    yes = ok && __double_as_longlong(cur) - __double_as_longlong(v) > 2;
+                } else {
+                    const double dec = cur - v;
+                    const bool over = ok && (cur >= EINF || dec > tol);
+                    big = big || over;
+                    yes = over || (ok && dec > 4.5e-16 * fabs(cur));
+                }
+                return yes ? (fe ? 1 : 0) + (fn ? 2 : 0) : -1;
             };
-            auto look_all = [&]() -> unsigned {
-                unsigned v = 0;
+            auto look_all = [&]() {
+                if (tol < 1e-15) known = false;   // every decrease above tol votes
 #pragma unroll 8
-                for (int r = 0; r < ET; ++r) v += look(lane, r, (upd >> r) & 1);
-                return v;
+                for (int r = 0; r < ET; ++r) {
+                    const int o = look(lane, r, (upd >> r) & 1);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (o == q) vote[q] |= 1u << r;
+                }
             };
-            unsigned votes;
             if (self == 2) {
-                votes = look_all();
+                look_all();
             } else {
                 // the interior was at rest for the halo of its last visit
                 const unsigned c0 = __shfl_sync(0xffffffffu, upd, 0), c1 = __shfl_sync(0xffffffffu, upd, ET - 1);
-                votes = look(lane, 0, upd & 1) + look(lane, ET - 1, upd >> (ET - 1)) + look(0, lane, (c0 >> lane) & 1) +
-                        look(ET - 1, lane, (c1 >> lane) & 1);
+                const int s0 = look(lane, 0, upd & 1), s1 = look(lane, ET - 1, upd >> (ET - 1));
+                const int w0 = look(0, lane, (c0 >> lane) & 1), w1 = look(ET - 1, lane, (c1 >> lane) & 1);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (s0 == q) vote[q] |= 1u;
+                    if (s1 == q) vote[q] |= 1u << (ET - 1);
+                    const unsigned b0 = __ballot_sync(0xffffffffu, w0 == q), b1 = __ballot_sync(0xffffffffu, w1 == q);
+                    if (lane == 0) vote[q] |= b0;
+                    if (lane == ET - 1) vote[q] |= b1;
+                }
             }
             bool swept = false;
             int n_left = EMAXS;
             while (true) {
-                // ordering with most votes over the warp (counts <= 32 per lane)
-                unsigned lo = (votes & 0xffu) | ((votes & 0xff00u) << 8);
-                unsigned hi = ((votes >> 16) & 0xffu) | ((votes >> 24) << 16);
-                lo = __reduce_add_sync(0xffffffffu, lo);
-                hi = __reduce_add_sync(0xffffffffu, hi);
+                known = __any_sync(0xffffffffu, big);
+                // ordering with most votes over the warp (at most 1024 each)
+                const unsigned lo = __reduce_add_sync(0xffffffffu, __popc(vote[0]) | (unsigned)__popc(vote[1]) << 16);
+                const unsigned hi = __reduce_add_sync(0xffffffffu, __popc(vote[2]) | (unsigned)__popc(vote[3]) << 16);
                 left = lo | hi;
                 if (left == 0 || n_left == 0) break;
                 const unsigned c[4] = {lo & 0xffffu, lo >> 16, hi & 0xffffu, hi >> 16};
                 int dir = 0;
-                unsigned most = c[0];
+                unsigned most = c[0], vm = vote[0];
 #pragma unroll
                 for (int q = 1; q < 4; ++q)
-                    if (c[q] > most) { most = c[q]; dir = q; }
+                    if (c[q] > most) { most = c[q]; dir = q; vm = vote[q]; }
                 const bool fwx = (dir & 1) == 0, fwy = (dir & 2) == 0;
                 const unsigned um = fwx ? upd : updr;
                 const int i = fwx ? lane : ET - 1 - lane;
-                for (int u = 0; u < 2 * ET - 1; ++u) {
+                // the diagonals of its first and last vote: nothing changes
+                // before the first, nor after the last once a few diagonals
+                // in a row changed nothing
+                const int ul = i;   // (lane of column `lane` in the sweep's order)
+                const int first = vm ? ul + (fwy ? __ffs((int)vm) - 1 : __clz((int)vm)) : 2 * ET;
+                const int last = vm ? ul + (fwy ? 31 - __clz((int)vm) : 32 - __ffs((int)vm)) : 0;
+                const int u0 = (int)__reduce_min_sync(0xffffffffu, (unsigned)first);
+                const int u1 = (int)__reduce_max_sync(0xffffffffu, (unsigned)last);
+                bool moved = false;
+                for (int u = u0; u < 2 * ET - 1; ++u) {
                     const int jj = u - lane, j = fwy ? jj : ET - 1 - jj;
                     if ((unsigned)jj < (unsigned)ET && ((um >> j) & 1)) {
                         const double a = dmin2<FAST>(T[j + 1][i], T[j + 1][i + 2]);
                         const double b = dmin2<FAST>(T[j][i + 1], T[j + 2][i + 1]);
-                        const double v = godunov_upd<FAST>(a, b, Fs[j][i]);
-                        if (dlt<FAST>(dmin2<FAST>(a, b), EINF) && dlt<FAST>(v, T[j + 1][i + 1])) T[j + 1][i + 1] = v;
+                        const double v = godunov_upd<FAST>(a, b, Fs[j][i], Rs[j][i]);
+                        if (dlt<FAST>(dmin2<FAST>(a, b), EINF) && dlt<FAST>(v, T[j + 1][i + 1])) {
+                            T[j + 1][i + 1] = v;
+                            moved = true;
+                        }
                     }
                     __syncwarp();
+                    if ((u & 3) == 3) {
+                        if (!__any_sync(0xffffffffu, moved) && u >= u1) break;
+                        moved = false;
+                    }
                 }
                 swept = true;
                 --n_left;
-                votes = look_all();
+                vote[0] = vote[1] = vote[2] = vote[3] = 0;
+                look_all();
             }
-            big = __any_sync(0xffffffffu, big);
             // below-tol decreases are written but do not wake the neighbours
-            if (swept && lane == 0 && (big || left)) {
+            if (swept && lane == 0 && (known || left)) {
                 act_out[t] = left ? 2 : 1;
                 atomicAdd(nchanged, 1u);
             }
