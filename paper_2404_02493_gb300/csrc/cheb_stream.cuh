@@ -76,20 +76,12 @@ __device__ __forceinline__ P2<T> diag_row(const LevelDesc& d, int j, int col, T 
     return P2<T>{helm_diag_h2<T>(d, col, j, k0, sg0), helm_diag_h2<T>(d, col + 1, j, k1, sg1)};
 }
 
-// the same for a row and columns strictly inside the grid (the absorbing
-// boundary terms are zero there; equal to helm_diag_h2 bit for bit)
+// the same for rows and columns strictly inside the grid of a level whose
+// diagonal is real there (no sponge, no shift): the boundary terms are zero
 template <typename T>
-__device__ __forceinline__ cplx<T> helm_diag_in(const LevelDesc& d, T k, T sig) {
-    const T h = LC<T>::h(d), kh = k * h;
-    const T re = T(4) - kh * kh;
-    T im = T(0);
-    if (d.bc == BC_SPONGE) im -= h * h * sig;
-    if (d.has_shift) im -= LC<T>::shift(d) * kh * kh;
-    return mk<T>(re, im);
-}
-template <typename T>
-__device__ __forceinline__ P2<T> diag_in_row(const LevelDesc& d, T k0, T k1, T sg0, T sg1) {
-    return P2<T>{helm_diag_in<T>(d, k0, sg0), helm_diag_in<T>(d, k1, sg1)};
+__device__ __forceinline__ P2<T> diag_in_row(const LevelDesc& d, T k0, T k1) {
+    const T h = LC<T>::h(d), a = k0 * h, b = k1 * h;
+    return P2<T>{mk<T>(T(4) - a * a, T(0)), mk<T>(T(4) - b * b, T(0))};
 }
 
 // (A v) at one row of the lane's pair (A^* v with CONJ), from the centre
@@ -109,6 +101,25 @@ __device__ __forceinline__ P2<T> helm_row(const P2<T>& dg, const P2<T>& c, const
     o.v0 = cscale<T>(csub<T>(cmul<T>(d0, c.v0), cadd<T>(cadd<T>(w0, c.v1), cadd<T>(s.v0, nn.v0))), ih2);
     o.v1 = cscale<T>(csub<T>(cmul<T>(d1, c.v1), cadd<T>(cadd<T>(c.v0, e1), cadd<T>(s.v1, nn.v1))), ih2);
     return o;
+}
+
+// the same without the factor 1/h^2, for a row with a real diagonal (then
+// A^* = A): 5 operations per component instead of 7
+template <typename T>
+__device__ __forceinline__ P2<T> helm_row_real(const P2<T>& dg, const P2<T>& c, const P2<T>& s, const P2<T>& nn) {
+    const cplx<T> w0 = shfl_up1<T>(c.v1);
+    const cplx<T> e1 = shfl_dn1<T>(c.v0);
+    const cplx<T> a = cadd<T>(cadd<T>(w0, c.v1), cadd<T>(s.v0, nn.v0));
+    const cplx<T> b = cadd<T>(cadd<T>(c.v0, e1), cadd<T>(s.v1, nn.v1));
+    return P2<T>{mk<T>(fma(dg.v0.x, c.v0.x, -a.x), fma(dg.v0.x, c.v0.y, -a.y)),
+                 mk<T>(fma(dg.v1.x, c.v1.x, -b.x), fma(dg.v1.x, c.v1.y, -b.y))};
+}
+// acc - s v, s v + acc
+template <typename T> __device__ __forceinline__ cplx<T> cfms(T s, cplx<T> v, cplx<T> acc) {
+    return mk<T>(fma(-s, v.x, acc.x), fma(-s, v.y, acc.y));
+}
+template <typename T> __device__ __forceinline__ cplx<T> cfmr(T s, cplx<T> v, cplx<T> acc) {
+    return mk<T>(fma(s, v.x, acc.x), fma(s, v.y, acc.y));
 }
 
 template <typename T>
@@ -146,7 +157,8 @@ __global__ void __launch_bounds__(32 * cs_wpb<HS>()) k_cheb_stream(const __grid_
     const T c1a = scalp<T>(d)[S::CHEB_C1 + m], c2a = scalp<T>(d)[S::CHEB_C2 + m];
     const T c1b = NS == 2 ? scalp<T>(d)[S::CHEB_C1 + m + 1] : T(0);
     const T c2b = NS == 2 ? scalp<T>(d)[S::CHEB_C2 + m + 1] : T(0);
-    const bool rd = c1a != T(0);
+    const T c2ai = c2a * ih2, c2bi = c2b * ih2;
+    const bool rd = c1a != T(0), real = !HS && !d.has_shift && d.bc != BC_SPONGE;
     const bool own = lane >= NS && lane < 32 - NS;
     constexpr int WPB = cs_wpb<HS>();
     for (int u = c.lb * WPB + warp; u < nunits; u += c.nb * WPB) {
@@ -209,25 +221,37 @@ __global__ void __launch_bounds__(32 * cs_wpb<HS>()) k_cheb_stream(const __grid_
             T k0, k1, s0 = T(0), s1 = T(0);
             ring_read<T>(Kr, r1, lane, k0, k1);
             if (HS) ring_read<T>(Sr, r1, lane, s0, s1);
-            const P2<T> dg1 = E ? diag_row<T>(d, r1, col, k0, k1, s0, s1) : diag_in_row<T>(d, k0, k1, s0, s1);
+            const P2<T> dg1 = E ? diag_row<T>(d, r1, col, k0, k1, s0, s1) : diag_in_row<T>(d, k0, k1);
             // level 1: t_m = g - A x_m at row j - 1
             const bool ro1 = (unsigned)r1 < (unsigned)ny;
             P2<T> t1 = ring_pair<T>(Gr, r1, lane);
             if (!xzero) {
-                const P2<T> ax = helm_row<T, false>(dg1, xa1, xa2, x0, ih2);
-                t1.v0 = csub<T>(t1.v0, ax.v0);
-                t1.v1 = csub<T>(t1.v1, ax.v1);
+                if constexpr (E) {
+                    const P2<T> ax = helm_row<T, false>(dg1, xa1, xa2, x0, ih2);
+                    t1.v0 = csub<T>(t1.v0, ax.v0);
+                    t1.v1 = csub<T>(t1.v1, ax.v1);
+                } else {
+                    const P2<T> ax = helm_row_real<T>(dg1, xa1, xa2, x0);
+                    t1.v0 = cfms<T>(ih2, ax.v0, t1.v0);
+                    t1.v1 = cfms<T>(ih2, ax.v1, t1.v1);
+                }
             }
             if constexpr (E) t1 = p2sel<T>(t1, ro1 && cin0, ro1 && cin1);
             // level 2: d_m, x_{m+1} at row j - 2
             const int r2 = j - 2;
             const bool ro2 = (unsigned)r2 < (unsigned)ny;
-            const P2<T> sv = helm_row<T, true>(dg2, ta2, ta3, t1, ih2);
-            P2<T> dm{cscale<T>(sv.v0, c2a), cscale<T>(sv.v1, c2a)};
+            P2<T> dm;
+            if constexpr (E) {
+                const P2<T> sv = helm_row<T, true>(dg2, ta2, ta3, t1, ih2);
+                dm = P2<T>{cscale<T>(sv.v0, c2a), cscale<T>(sv.v1, c2a)};
+            } else {
+                const P2<T> sv = helm_row_real<T>(dg2, ta2, ta3, t1);
+                dm = P2<T>{cscale<T>(sv.v0, c2ai), cscale<T>(sv.v1, c2ai)};
+            }
             if (rd) {
                 const P2<T> dp = ring_pair<T>(Dr, r2, lane);
-                dm.v0 = cadd<T>(dm.v0, cscale<T>(dp.v0, c1a));
-                dm.v1 = cadd<T>(dm.v1, cscale<T>(dp.v1, c1a));
+                dm.v0 = cfmr<T>(c1a, dp.v0, dm.v0);
+                dm.v1 = cfmr<T>(c1a, dp.v1, dm.v1);
             }
             const P2<T> xm1{cadd<T>(xa2.v0, dm.v0), cadd<T>(xa2.v1, dm.v1)};
             if constexpr (NS == 1) {
@@ -243,17 +267,29 @@ __global__ void __launch_bounds__(32 * cs_wpb<HS>()) k_cheb_stream(const __grid_
                 const int r3 = j - 3;
                 const bool ro3 = (unsigned)r3 < (unsigned)ny;
                 P2<T> t2 = ring_pair<T>(Gr, r3, lane);
-                const P2<T> ax = helm_row<T, false>(dg3, xb3, xb4, xn, ih2);
-                t2.v0 = csub<T>(t2.v0, ax.v0);
-                t2.v1 = csub<T>(t2.v1, ax.v1);
-                if constexpr (E) t2 = p2sel<T>(t2, ro3 && cin0, ro3 && cin1);
+                if constexpr (E) {
+                    const P2<T> ax = helm_row<T, false>(dg3, xb3, xb4, xn, ih2);
+                    t2.v0 = csub<T>(t2.v0, ax.v0);
+                    t2.v1 = csub<T>(t2.v1, ax.v1);
+                    t2 = p2sel<T>(t2, ro3 && cin0, ro3 && cin1);
+                } else {
+                    const P2<T> ax = helm_row_real<T>(dg3, xb3, xb4, xn);
+                    t2.v0 = cfms<T>(ih2, ax.v0, t2.v0);
+                    t2.v1 = cfms<T>(ih2, ax.v1, t2.v1);
+                }
                 // level 4: d_{m+1}, x_{m+2} at row j - 4
                 const int r4 = j - 4;
-                const P2<T> s2 = helm_row<T, true>(dg4, tb4, tb5, t2, ih2);
+                P2<T> s2;
+                if constexpr (E) {
+                    s2 = helm_row<T, true>(dg4, tb4, tb5, t2, ih2);
+                    s2 = P2<T>{cscale<T>(s2.v0, c2b), cscale<T>(s2.v1, c2b)};
+                } else {
+                    s2 = helm_row_real<T>(dg4, tb4, tb5, t2);
+                    s2 = P2<T>{cscale<T>(s2.v0, c2bi), cscale<T>(s2.v1, c2bi)};
+                }
                 if (own && r4 >= y0 && r4 < y1) {
                     const long long p = (long long)r4 * pitch + col;
-                    const P2<T> e{cadd<T>(cscale<T>(s2.v0, c2b), cscale<T>(db4.v0, c1b)),
-                                  cadd<T>(cscale<T>(s2.v1, c2b), cscale<T>(db4.v1, c1b))};
+                    const P2<T> e{cfmr<T>(c1b, db4.v0, s2.v0), cfmr<T>(c1b, db4.v1, s2.v1)};
                     store_pair<T>(xout, p, P2<T>{cadd<T>(xb4.v0, e.v0), cadd<T>(xb4.v1, e.v1)}, cin0, cin1);
                     if (wd) store_pair<T>(dout, p, e, cin0, cin1);
                 }
@@ -265,13 +301,14 @@ __global__ void __launch_bounds__(32 * cs_wpb<HS>()) k_cheb_stream(const __grid_
             xa2 = x0;
             dg4 = dg3; dg3 = dg2; dg2 = dg1;
         };
-        // rows and columns strictly inside the grid (warp-uniform): no zero
-        // selects, no boundary terms in the diagonal
+        // every row whose diagonal is used (j - 4 .. j - 1) and every column
+        // strictly inside the grid (warp-uniform), the diagonal real: no zero
+        // selects, no boundary terms
         auto step = [&](int j, auto odd) {
             if (j + AH <= j1) issue(j + AH);
             cp_async_commit();
             cp_async_wait<AH>();
-            const bool in = colint && j >= 3 && j <= ny - 1;
+            const bool in = real && colint && j >= 5 && j <= ny - 1;
             if constexpr (decltype(odd)::value) {
                 if (in) row(std::false_type{}, j, xaQ, xaP, taQ, taP, xbQ, xbP, dbQ, dbP, tbQ, tbP);
                 else row(std::true_type{}, j, xaQ, xaP, taQ, taP, xbQ, xbP, dbQ, dbP, tbQ, tbP);

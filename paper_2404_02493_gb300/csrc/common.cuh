@@ -227,6 +227,13 @@ __device__ __forceinline__ cplx<T> helm_diff(cplx<T> dg4, cplx<T> c, cplx<T> w, 
     return cscale<T>(cfma<T>(dg4, c, t), ih2);
 }
 
+// the same with a real diagonal
+template <typename T>
+__device__ __forceinline__ cplx<T> helm_diff_real(T dg4, cplx<T> c, cplx<T> w, cplx<T> e, cplx<T> s, cplx<T> n, T ih2) {
+    const cplx<T> t = cadd<T>(cadd<T>(csub<T>(c, w), csub<T>(c, e)), cadd<T>(csub<T>(c, s), csub<T>(c, n)));
+    return mk<T>(fma(dg4, c.x, t.x) * ih2, fma(dg4, c.y, t.y) * ih2);
+}
+
 template <typename T> __device__ __forceinline__ T load_k(const LevelDesc& d, int i, int j) {
     return __ldg(reinterpret_cast<const T*>(d.kf) + (long long)j * d.pitch + i);
 }

@@ -793,20 +793,24 @@ struct Engine : EngineBase {
     static bool adr_per_level(Handle& H, int b, int l) {
         return H.inst[b].la > 0 && l >= H.inst[b].la && H.inst[b].L > l && !in_tail(H, b, l);
     }
+    // A level's size is within the tail's bound: mg_params.tail_nmax where it
+    // is set, else the number of nodes chosen at setup.
+    static bool tail_size(Handle& H, int n, int ny) {
+        return std::max(n, ny) <= H.p.tail_nmax && (long long)n * ny <= H.tail_nodes;
+    }
     // Level l (not the coarsest) of instance b starts or lies in the coarse
     // tail: l >= 3 (below the ADR-correction level), max(n_l, ny_l) <=
     // tail_nmax and the levels from l down fit in one cluster.
     static bool in_tail(Handle& H, int b, int l) {
         const int n = H.inst[b].lv[l - 1].n, ny = H.inst[b].lv[l - 1].ny;
-        return l >= 3 && l > H.inst[b].la && std::max(n, ny) <= H.p.tail_nmax && ct_fits(H, b, l, false);
+        return l >= 3 && l > H.inst[b].la && tail_size(H, n, ny) && ct_fits(H, b, l, false);
     }
     // The ADR corrections of instance b run whole in one cluster launch: the
     // correction level itself is within the tail's bound and fits (Wave-Ray
     // changes the operators from one correction to the next).
     static bool adr_whole(Handle& H, int b) {
         const InstHost& I = H.inst[b];
-        return I.la > 0 && !H.p.ray && std::max(I.lv[I.la - 1].n, I.lv[I.la - 1].ny) <= H.p.tail_nmax &&
-               ct_fits(H, b, I.la, true);
+        return I.la > 0 && !H.p.ray && tail_size(H, I.lv[I.la - 1].n, I.lv[I.la - 1].ny) && ct_fits(H, b, I.la, true);
     }
     // ADR V-cycle on levels l..L (Section 3.2.2), right-hand side in SAB of
     // level l, result in SAX (or, at level 2 with `modulate`, added as

@@ -990,14 +990,16 @@ int mg_setup(mg_handle** out, const mg_instance* inst, int ninst, const mg_param
     mg_handle* mh = new mg_handle();
     mh->H.p = *p;
     mh->H.alloc_limit = p->workspace_limit;
-    // automatic coarse tail (one cluster per instance, tail_cluster.cuh) for a
-    // handle with one instance: levels with n <= 127 in FP32, where a launch
-    // costs more than its work, n <= 63 in FP64, whose arithmetic wants all
-    // SMs above that; with many instances the per-level launches spread the
-    // work over more SMs
-    // the wave-cycle tail (tail_wave.cuh) follows an explicit tail_nmax; automatic: levels with n <= 63
-    mh->H.wave_tail_nmax = mh->H.p.tail_nmax >= 0 ? mh->H.p.tail_nmax : 63;
-    if (mh->H.p.tail_nmax < 0) mh->H.p.tail_nmax = ninst == 1 ? (p->precision == MG_PREC_FP64 ? 63 : 127) : 0;
+    // automatic coarse tail (one cluster per instance, tail_cluster.cuh), by
+    // nodes, for as many instances as clusters fit the GPU at once: levels of up
+    // to 128 x 128 nodes in FP32, where a launch costs more than its work, 64 x
+    // 64 in FP64, whose arithmetic wants all SMs above that; with more
+    // instances the per-level launches spread the work over more SMs
+    // the wave-cycle tail (tail_wave.cuh) follows an explicit tail_nmax;
+    // automatic: what one block takes (64 columns)
+    mh->H.wave_tail_nmax = mh->H.p.tail_nmax >= 0 ? mh->H.p.tail_nmax : 64;
+    mh->H.tail_nodes = mh->H.p.tail_nmax >= 0 ? (1ll << 40) : (p->precision == MG_PREC_FP64 ? 64 * 64 : 128 * 128);
+    if (mh->H.p.tail_nmax < 0) mh->H.p.tail_nmax = ninst <= 8 ? (1 << 30) : 0;
     // the two tails follow the index roles: with a role list every level has
     // its own launches
     if (roles_set(*p)) {

@@ -68,10 +68,18 @@ __global__ void __launch_bounds__(32 * RS_WPB) k_restrict_jac0_stream(const __gr
         const int col = X0 + 2 * lane;
         const bool cin0 = (unsigned)col < (unsigned)n, cin1 = (unsigned)(col + 1) < (unsigned)n;
         const int I = X0 / 2 + lane;   // coarse column of the lane
+        // the copies of a row share the element offset r * pitch + col
+        const int cntc = cin0 ? min(2, n - col) : 0;
+        const unsigned sga = (unsigned)__cvta_generic_to_shared(Gr + 2 * lane);
+        const unsigned ska = (unsigned)__cvta_generic_to_shared(Kr + 2 * lane);
+        constexpr int CE = (int)sizeof(cplx<T>), RE = (int)sizeof(T);
         auto issue = [&](int r) {
-            ring_issue2<cplx<T>>(Gr, gv, n, ny, pitch, X0, r, lane);
-            ring_issue2<T>(Kr, kf, n, ny, pitch, X0, r, lane);
-            if (HS) ring_issue2<T>(Sr, sgf, n, ny, pitch, X0, r, lane);
+            const int cnt = (unsigned)r < (unsigned)ny ? cntc : 0;
+            const long long off = cnt ? (long long)r * pitch + col : 0;
+            const unsigned so = (unsigned)((r & (SW_DEP - 1)) * SW_COLS);
+            cp_pair<2 * CE>(sga + so * CE, gv + off, cnt * CE);
+            cp_pair<2 * RE>(ska + so * RE, kf + off, cnt * RE);
+            if (HS) cp_pair<2 * RE>(ska + SW_DEP * SW_COLS * RE + so * RE, sgf + off, cnt * RE);
         };
 #pragma unroll
         for (int r = 0; r < RS_AH; ++r) {
@@ -81,37 +89,39 @@ __global__ void __launch_bounds__(32 * RS_WPB) k_restrict_jac0_stream(const __gr
         P2<T> ua2 = p2zero<T>(), ua1 = p2zero<T>();   // u1 at j-2, j-1
         P2<T> dg1 = p2zero<T>();                      // diagonal at j-1
         P2<T> r3 = p2zero<T>(), r2 = p2zero<T>();     // r at j-3, j-2
+        // all columns inside the grid's boundary and a real diagonal there
+        const bool colin = !HS && !d.has_shift && d.bc != BC_SPONGE && X0 >= 1 && X0 + SW_COLS - 1 <= n - 2;
         for (int j = j0; j <= j1; ++j) {
             if (j + RS_AH <= j1) issue(j + RS_AH);
             cp_async_commit();
             cp_async_wait<RS_AH>();
-            // u1 = w h^2 g / (h^2 D) at row j (one division per node)
-            P2<T> g0;
-            ring_read<cplx<T>>(Gr, j, lane, g0.v0, g0.v1);
-            if (fgv) g0 = P2<T>{cscale<T>(g0.v0, gsc), cscale<T>(g0.v1, gsc)};
+            P2<T> g0 = ring_pair<T>(Gr, j, lane), gp = ring_pair<T>(Gr, j - 1, lane);
+            if (fgv) {
+                g0 = P2<T>{cscale<T>(g0.v0, gsc), cscale<T>(g0.v1, gsc)};
+                gp = P2<T>{cscale<T>(gp.v0, gsc), cscale<T>(gp.v1, gsc)};
+            }
             T k0, k1, s0 = T(0), s1 = T(0);
             ring_read<T>(Kr, j, lane, k0, k1);
             if (HS) ring_read<T>(Sr, j, lane, s0, s1);
-            const P2<T> dg0 = diag_row<T>(d, j, col, k0, k1, s0, s1);
-            P2<T> u0;
-            {
+            P2<T> u0, rr, dg0;
+            // u1 = w h^2 g / (h^2 D) at row j (one division per node), r = g - A u1 at row j - 1
+            if (colin && j >= 2 && j <= ny - 2) {
+                dg0 = diag_in_row<T>(d, k0, k1);
+                u0 = P2<T>{cscale<T>(g0.v0, wj * h2 / dg0.v0.x), cscale<T>(g0.v1, wj * h2 / dg0.v1.x)};
+                const P2<T> au = helm_row_real<T>(dg1, ua1, ua2, u0);
+                rr = P2<T>{cfms<T>(ih2, au.v0, gp.v0), cfms<T>(ih2, au.v1, gp.v1)};
+            } else {
+                dg0 = diag_row<T>(d, j, col, k0, k1, s0, s1);
                 const T a0 = wj * h2 / (dg0.v0.x * dg0.v0.x + dg0.v0.y * dg0.v0.y);
                 const T a1 = wj * h2 / (dg0.v1.x * dg0.v1.x + dg0.v1.y * dg0.v1.y);
                 u0.v0 = mk<T>((g0.v0.x * dg0.v0.x + g0.v0.y * dg0.v0.y) * a0,
                               (g0.v0.y * dg0.v0.x - g0.v0.x * dg0.v0.y) * a0);
                 u0.v1 = mk<T>((g0.v1.x * dg0.v1.x + g0.v1.y * dg0.v1.y) * a1,
                               (g0.v1.y * dg0.v1.x - g0.v1.x * dg0.v1.y) * a1);
+                const P2<T> au = helm_row<T, false>(dg1, ua1, ua2, u0, ih2);
+                rr = P2<T>{csub<T>(gp.v0, au.v0), csub<T>(gp.v1, au.v1)};
             }
-            if (own && j >= fy0 && j < fy1) {
-                store_pair<T>(xs, (long long)j * pitch + col, u0, cin0, cin1);
-            }
-            // r = g - A u1 at row j - 1
-            P2<T> rr;
-            ring_read<cplx<T>>(Gr, j - 1, lane, rr.v0, rr.v1);
-            if (fgv) rr = P2<T>{cscale<T>(rr.v0, gsc), cscale<T>(rr.v1, gsc)};
-            const P2<T> au = helm_row<T, false>(dg1, ua1, ua2, u0, ih2);
-            rr.v0 = csub<T>(rr.v0, au.v0);
-            rr.v1 = csub<T>(rr.v1, au.v1);
+            if (own && j >= fy0 && j < fy1) store_pair<T>(xs, (long long)j * pitch + col, u0, cin0, cin1);
             // coarse row J = (j - 3) / 2 from r rows 2 J (r3), 2 J + 1 (r2), 2 J + 2 (rr)
             if (((j - j0) & 1) == 0 && j >= j0 + 4) {
                 const int J = (j - 3) >> 1;
@@ -199,11 +209,18 @@ __global__ void __launch_bounds__(32 * RS_WPB) k_prolong_jac_stream(const __grid
         const bool cin0 = (unsigned)col < (unsigned)n, cin1 = (unsigned)(col + 1) < (unsigned)n;
         const int ci = X0 / 2 + lane;   // the lane's coarse column
         const bool cci = (unsigned)ci < (unsigned)nc;
+        const int cntc = cin0 ? min(2, n - col) : 0;
+        constexpr int CE = (int)sizeof(cplx<T>), RE = (int)sizeof(T);
+        const unsigned sxa = (unsigned)__cvta_generic_to_shared(Xr + 2 * lane);
+        const unsigned ska = (unsigned)__cvta_generic_to_shared(Kr + 2 * lane);
         auto issue = [&](int r) {
-            ring_issue2<cplx<T>>(Xr, xv, n, ny, pitch, X0, r, lane);
-            ring_issue2<cplx<T>>(Gr, gv, n, ny, pitch, X0, r, lane);
-            ring_issue2<T>(Kr, kf, n, ny, pitch, X0, r, lane);
-            if (HS) ring_issue2<T>(Sr, sgf, n, ny, pitch, X0, r, lane);
+            const int cnt = (unsigned)r < (unsigned)ny ? cntc : 0;
+            const long long off = cnt ? (long long)r * pitch + col : 0;
+            const unsigned so = (unsigned)((r & (SW_DEP - 1)) * SW_COLS);
+            cp_pair<2 * CE>(sxa + so * CE, xv + off, cnt * CE);
+            cp_pair<2 * CE>(sxa + SW_DEP * SW_COLS * CE + so * CE, gv + off, cnt * CE);
+            cp_pair<2 * RE>(ska + so * RE, kf + off, cnt * RE);
+            if (HS) cp_pair<2 * RE>(ska + SW_DEP * SW_COLS * RE + so * RE, sgf + off, cnt * RE);
             if (!(r & 1) || r == j0) {
                 // coarse row r / 2 (for the first row, the row below it as well)
                 const int cr = (r & 1) ? (r - 1) >> 1 : r >> 1;
@@ -226,6 +243,7 @@ __global__ void __launch_bounds__(32 * RS_WPB) k_prolong_jac_stream(const __grid
         P2<T> ua2 = p2zero<T>(), ua1 = p2zero<T>();   // u at j-2, j-1
         P2<T> ob3 = p2zero<T>(), ob2 = p2zero<T>();   // FG: z at j-3, j-2
         P2<T> dgp = p2zero<T>();                      // FG: diagonal less 4 at j-2
+        const bool colin = !HS && !d.has_shift && d.bc != BC_SPONGE && X0 >= 1 && X0 + SW_COLS - 1 <= n - 2;
         for (int j = j0; j <= j1; ++j) {
             if (j + PS_AH <= j1) issue(j + PS_AH);
             cp_async_commit();
@@ -241,54 +259,59 @@ __global__ void __launch_bounds__(32 * RS_WPB) k_prolong_jac_stream(const __grid
             u0.v0 = cscale<T>(cadd<T>(cscale<T>(plo, T(0.5)), cscale<T>(elo, T(0.5))), wb0);
             u0.v0 = cadd<T>(u0.v0, cscale<T>(cadd<T>(cscale<T>(phi, T(0.5)), cscale<T>(ehi, T(0.5))), wb1));
             u0.v1 = cadd<T>(cscale<T>(elo, wb0), cscale<T>(ehi, wb1));
-            P2<T> x0;
-            ring_read<cplx<T>>(Xr, j, lane, x0.v0, x0.v1);
+            const P2<T> x0 = ring_pair<T>(Xr, j, lane);
             u0.v0 = cadd<T>(x0.v0, u0.v0);
             u0.v1 = cadd<T>(x0.v1, u0.v1);
-            const bool roj = (unsigned)j < (unsigned)ny;
-            u0 = p2sel<T>(u0, roj && cin0, roj && cin1);
-            // Jacobi at row j - 1
-            const int r1 = j - 1;
+            // Jacobi at row j - 1; FG: W = A z at row j - 2 (z zero outside the grid)
+            const int r1 = j - 1, r2 = j - 2;
             T k0, k1, s0 = T(0), s1 = T(0);
             ring_read<T>(Kr, r1, lane, k0, k1);
             if (HS) ring_read<T>(Sr, r1, lane, s0, s1);
-            const P2<T> dg = diag_row<T>(d, r1, col, k0, k1, s0, s1);
-            P2<T> rr;
-            ring_read<cplx<T>>(Gr, r1, lane, rr.v0, rr.v1);
+            P2<T> rr = ring_pair<T>(Gr, r1, lane), o1, dg;
             if (FG) rr = P2<T>{cscale<T>(rr.v0, gsc), cscale<T>(rr.v1, gsc)};
-            const P2<T> au = helm_row<T, false>(dg, ua1, ua2, u0, ih2);
-            rr.v0 = csub<T>(rr.v0, au.v0);
-            rr.v1 = csub<T>(rr.v1, au.v1);
-            const bool wr1 = own && r1 >= y0 && r1 < y1;
-            if (FG || wr1) {
-                P2<T> o1;
-                {
-                    const T a = wjh2 / (dg.v0.x * dg.v0.x + dg.v0.y * dg.v0.y);
-                    o1.v0 = cadd<T>(ua1.v0, mk<T>((rr.v0.x * dg.v0.x + rr.v0.y * dg.v0.y) * a,
-                                                  (rr.v0.y * dg.v0.x - rr.v0.x * dg.v0.y) * a));
-                }
-                {
-                    const T a = wjh2 / (dg.v1.x * dg.v1.x + dg.v1.y * dg.v1.y);
-                    o1.v1 = cadd<T>(ua1.v1, mk<T>((rr.v1.x * dg.v1.x + rr.v1.y * dg.v1.y) * a,
-                                                  (rr.v1.y * dg.v1.x - rr.v1.x * dg.v1.y) * a));
-                }
-                if (wr1) {
-                    store_pair<T>(os, (long long)r1 * pitch + col, o1, cin0, cin1);
-                }
-                if constexpr (FG) {
-                    // W = A z at row j - 2 (z zero outside the grid)
+            // rows j - 2 .. j and all columns inside the grid, rows j - 2 and
+            // j - 1 and all columns off its boundary, the diagonal real
+            const bool in = colin && j >= 3 && j <= ny - 1;
+            if (in) {
+                dg = diag_in_row<T>(d, k0, k1);
+                const P2<T> au = helm_row_real<T>(dg, ua1, ua2, u0);
+                const T a = wjh2 / dg.v0.x, b = wjh2 / dg.v1.x;
+                o1.v0 = cfmr<T>(a, cfms<T>(ih2, au.v0, rr.v0), ua1.v0);
+                o1.v1 = cfmr<T>(b, cfms<T>(ih2, au.v1, rr.v1), ua1.v1);
+            } else {
+                const bool roj = (unsigned)j < (unsigned)ny;
+                u0 = p2sel<T>(u0, roj && cin0, roj && cin1);
+                dg = diag_row<T>(d, r1, col, k0, k1, s0, s1);
+                const P2<T> au = helm_row<T, false>(dg, ua1, ua2, u0, ih2);
+                rr.v0 = csub<T>(rr.v0, au.v0);
+                rr.v1 = csub<T>(rr.v1, au.v1);
+                const T a = wjh2 / (dg.v0.x * dg.v0.x + dg.v0.y * dg.v0.y);
+                o1.v0 = cadd<T>(ua1.v0, mk<T>((rr.v0.x * dg.v0.x + rr.v0.y * dg.v0.y) * a,
+                                              (rr.v0.y * dg.v0.x - rr.v0.x * dg.v0.y) * a));
+                const T b = wjh2 / (dg.v1.x * dg.v1.x + dg.v1.y * dg.v1.y);
+                o1.v1 = cadd<T>(ua1.v1, mk<T>((rr.v1.x * dg.v1.x + rr.v1.y * dg.v1.y) * b,
+                                              (rr.v1.y * dg.v1.x - rr.v1.x * dg.v1.y) * b));
+                if (FG) {
                     const bool ro1 = (unsigned)r1 < (unsigned)ny;
                     o1 = p2sel<T>(o1, ro1 && cin0, ro1 && cin1);
-                    const int r2 = j - 2;
-                    const cplx<T> zw = shfl_up1<T>(ob2.v1), ze = shfl_dn1<T>(ob2.v0);
-                    const P2<T> w{helm_diff<T>(dgp.v0, ob2.v0, zw, ob2.v1, ob3.v0, o1.v0, ih2),
-                                  helm_diff<T>(dgp.v1, ob2.v1, ob2.v0, ze, ob3.v1, o1.v1, ih2)};
-                    if (own && r2 >= y0 && r2 < y1) {
-                        store_pair<T>(wv, (long long)r2 * pitch + col, w, cin0, cin1);
-                    }
-                    ob3 = ob2; ob2 = o1;
+                }
+            }
+            if (own && r1 >= y0 && r1 < y1) store_pair<T>(os, (long long)r1 * pitch + col, o1, cin0, cin1);
+            if constexpr (FG) {
+                const cplx<T> zw = shfl_up1<T>(ob2.v1), ze = shfl_dn1<T>(ob2.v0);
+                P2<T> w;
+                if (in) {
+                    w = P2<T>{helm_diff_real<T>(dgp.v0.x, ob2.v0, zw, ob2.v1, ob3.v0, o1.v0, ih2),
+                              helm_diff_real<T>(dgp.v1.x, ob2.v1, ob2.v0, ze, ob3.v1, o1.v1, ih2)};
+                    const T h = LC<T>::h(d), e = k0 * h, f = k1 * h;
+                    dgp = P2<T>{mk<T>(-(e * e), T(0)), mk<T>(-(f * f), T(0))};
+                } else {
+                    w = P2<T>{helm_diff<T>(dgp.v0, ob2.v0, zw, ob2.v1, ob3.v0, o1.v0, ih2),
+                              helm_diff<T>(dgp.v1, ob2.v1, ob2.v0, ze, ob3.v1, o1.v1, ih2)};
                     dgp = P2<T>{helm_diag4<T>(d, col, r1, k0, s0), helm_diag4<T>(d, col + 1, r1, k1, s1)};
                 }
+                if (own && r2 >= y0 && r2 < y1) store_pair<T>(wv, (long long)r2 * pitch + col, w, cin0, cin1);
+                ob3 = ob2; ob2 = o1;
             }
             ua2 = ua1; ua1 = u0;
         }
