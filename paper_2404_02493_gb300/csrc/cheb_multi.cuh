@@ -14,7 +14,7 @@
 // shared memory.  Nodes outside the grid hold zero, as in k_cheb_step; the
 // arithmetic per node and its order are those of k_cheb_step.
 #pragma once
-#include "kernels.cuh"
+#include "wave_nodes.cuh"
 
 namespace wadr {
 
@@ -109,6 +109,71 @@ __global__ void __launch_bounds__(NT) k_cheb_multi(const __grid_constant__ KDesc
             for (int cc = H + tx; cc < H + TS; cc += BX) {
                 const int gi = x0 + cc, gj = y0 + r;
                 if (gi < n && gj < ny) xout[(long long)gj * pitch + gi] = X[r * W + cc];
+            }
+        __syncthreads();
+    }
+}
+
+// The same smoothing with the region in registers (wave_nodes.cuh): a block of
+// 1024 threads holds 64 columns of 16 RPT rows, of which all but 2q on each
+// side are its output tile (values on the outer ring go wrong by one node per
+// stencil).  With every operand in shared memory, an in-grid test per node and
+// stage and 256 threads per region, k_cheb_multi is bound by issue slots and
+// barriers; here a stage is bound by its shared-memory loads, so that two rows
+// per thread are the faster form while their tiles fit the SMs, and four
+// (which recompute less) above.  q = 5: n = 511 24 us there, 13.3 here, n =
+// 255 12.6 and 7.0, n = 127 9.2 and 7.3.  k_cheb_multi remains for
+// longer smoothings, whose ring would leave too small a tile.
+constexpr int CR_W = 64, CR_MAXQ = 8;
+template <typename T, int RPT> __host__ __device__ constexpr int cr_smem() {
+    return 2 * (CR_W + 2) * (CR_W / 4 * RPT + 2) * (int)sizeof(cplx<T>);
+}
+template <typename T, int RPT>
+__global__ void __launch_bounds__(WT_THREADS, 1) k_cheb_region(const __grid_constant__ KDesc A,
+                                                               const Seg* __restrict__ Sg, int nseg, int sxin,
+                                                               int sxout, int q, int xzero) {
+    constexpr int RH = WT_THREADS / WT_MAXN * RPT, NE = (CR_W + 2) * (RH + 2);
+    static_assert(RH == CR_W / 4 * RPT && WT_MAXN == CR_W, "region");
+    extern __shared__ __align__(16) unsigned char cr_smem_[];
+    __shared__ LevelDesc d;
+    __shared__ T cc[2][16];
+    SegCtx c = seg_begin(A, Sg, nseg, d);
+    cplx<T>* const X = reinterpret_cast<cplx<T>*>(cr_smem_);
+    cplx<T>* const Tt = X + NE;
+    const int tid = threadIdx.x, H = 2 * q, TX = CR_W - 2 * H, TY = RH - 2 * H;
+    const int n = d.n, ny = d.ny, pitch = d.pitch;
+    const int ntx = (n + TX - 1) / TX, ntiles = ntx * ((ny + TY - 1) / TY);
+    const cplx<T>* const xin = slot<T>(d, sxin);
+    const cplx<T>* const gv = slot<T>(d, SG);
+    cplx<T>* const xout = slot<T>(d, sxout);
+    const T ih2 = LC<T>::ih2(d);
+    if (tid < 32) cc[tid >> 4][tid & 15] = scalp<T>(d)[((tid >> 4) ? S::CHEB_C2 : S::CHEB_C1) + (tid & 15)];
+    for (int e = tid; e < NE; e += WT_THREADS) X[e] = Tt[e] = zero2<T>();
+    __syncthreads();
+    for (int t = c.lb; t < ntiles; t += c.nb) {
+        const int x0 = (t % ntx) * TX - H, y0 = (t / ntx) * TY - H;
+        WtNodes<T, RPT> N;
+        N.place(CR_W, n, ny, x0, y0);
+#pragma unroll
+        for (int r = 0; r < RPT; ++r) {
+            if (N.in[r]) {
+                const int gi = x0 + N.i, gj = y0 + N.j0 + r;
+                const long long p = (long long)gj * pitch + gi;
+                if (!xzero) N.x[r] = xin[p];
+                N.g[r] = gv[p];
+                N.dg[r] = helm_diag_at<T>(d, gi, gj);
+            }
+            // (nodes outside the grid are zero in both vectors)
+            X[N.at(r)] = N.x[r];
+            Tt[N.at(r)] = zero2<T>();
+        }
+        __syncthreads();
+        wt_cheb<T>(N, q, xzero, X, Tt, ih2, cc);
+        if (N.i >= H && N.i < CR_W - H)
+#pragma unroll
+            for (int r = 0; r < RPT; ++r) {
+                const int j = N.j0 + r;
+                if (N.in[r] && j >= H && j < RH - H) xout[(long long)(y0 + j) * pitch + x0 + N.i] = N.x[r];
             }
         __syncthreads();
     }

@@ -217,6 +217,27 @@ struct Engine : EngineBase {
     void launch_cheb_multi(Handle& H, const std::vector<int>& ds, int ts, double bpp, int sin, int sout, int q,
                            int xzero, cudaStream_t st) {
         if constexpr (std::is_same<T, float>::value) {
+            if (q <= CR_MAXQ) {
+                // two rows per thread while all tiles are resident (and give at least 8 rows of output)
+                long long tiles = 0;
+                const int tx = CR_W - 4 * q, ty = CR_W / 2 - 4 * q;
+                if (ty >= 8)
+                    for (int qd : ds) {
+                        const LevelDesc& L = H.hdesc[(size_t)qd];
+                        tiles += (long long)((L.n + tx - 1) / tx) * ((L.ny + ty - 1) / ty);
+                    }
+                auto run = [&](auto kern, int rows, int smem) {
+                    const SegTable& t = H.seg_tiles(ds, tx, rows - 4 * q, false, occ_cap(kern, smem, WT_THREADS));
+                    go(H, st, KK_CHEB, bpp * (double)t.pts, [&] {
+                        kl(kern, t.nblocks, dim3(WT_THREADS), smem, st, kd(H, t), t.d, t.nseg, sin, sout, q, xzero);
+                    }, t.pts);
+                };
+                if (tiles > 0 && tiles <= occ_cap(k_cheb_region<T, 2>, cr_smem<T, 2>(), WT_THREADS))
+                    run(k_cheb_region<T, 2>, CR_W / 2, cr_smem<T, 2>());
+                else
+                    run(k_cheb_region<T, 4>, CR_W, cr_smem<T, 4>());
+                return;
+            }
             const int smem = cm_smem<T>(ts, q);
             auto run = [&](auto kern) {
                 const SegTable& t = H.seg_tiles(ds, ts, ts, false, occ_cap_at(kern, smem));

@@ -31,15 +31,11 @@
 // read it).  Only block barriers are used; every thread runs the same level
 // loop.
 #pragma once
-#include "kernels.cuh"
+#include "wave_nodes.cuh"
 
 namespace wadr {
 
 constexpr int TS_MAXL = 8;    // levels of a chain, the coarsest included
-constexpr int WT_THREADS = 1024;
-constexpr int WT_MAXN = 64;   // columns; nodes map to threads as 64 columns x 16 groups of rows
-// rows per thread (64 registers a thread at 1024 threads)
-template <typename T> __host__ __device__ constexpr int wt_rpt() { return sizeof(T) == 4 ? 4 : 2; }
 template <typename T> __host__ __device__ constexpr int wt_maxny() { return WT_THREADS / WT_MAXN * wt_rpt<T>(); }
 
 // dynamic shared memory for a first level of n x ny nodes: x and t with a
@@ -70,70 +66,6 @@ __device__ __forceinline__ int wt_chain(const LevelDesc* __restrict__ D, const i
     return nl;
 }
 
-// One thread's nodes of a level: rows j0 .. j0 + RPT - 1 of column i.
-template <typename T> struct WtNodes {
-    static constexpr int RPT = wt_rpt<T>();
-    cplx<T> x[RPT], g[RPT], dg[RPT];
-    int i, j0, W;
-    bool in[RPT];
-    __device__ __forceinline__ void place(const LevelDesc& d) {
-        i = threadIdx.x & (WT_MAXN - 1);
-        j0 = (threadIdx.x / WT_MAXN) * RPT;
-        W = d.n + 2;
-#pragma unroll
-        for (int r = 0; r < RPT; ++r) {
-            in[r] = i < d.n && j0 + r < d.ny;
-            x[r] = g[r] = dg[r] = zero2<T>();
-        }
-    }
-    __device__ __forceinline__ int at(int r) const { return (j0 + r + 1) * W + i + 1; }
-    // sum of the four neighbours of row r: own rows in v, the others in V
-    __device__ __forceinline__ cplx<T> nsum(const cplx<T> (&v)[RPT], const cplx<T>* V, int r) const {
-        const int p = at(r);
-        const cplx<T> s = r > 0 ? v[r > 0 ? r - 1 : 0] : V[p - W];
-        const cplx<T> n = r < RPT - 1 ? v[r < RPT - 1 ? r + 1 : 0] : V[p + W];
-        return cadd<T>(cadd<T>(V[p - 1], V[p + 1]), cadd<T>(s, n));
-    }
-    // t = g - A x, to the shared vector Tt
-    __device__ __forceinline__ void residual(cplx<T> (&t)[RPT], const cplx<T>* X, cplx<T>* Tt, T ih2, bool xz) const {
-#pragma unroll
-        for (int r = 0; r < RPT; ++r) {
-            t[r] = g[r];
-            if (!xz && in[r]) t[r] = csub<T>(g[r], cscale<T>(csub<T>(cmul<T>(dg[r], x[r]), nsum(x, X, r)), ih2));
-            if (in[r]) Tt[at(r)] = t[r];
-        }
-    }
-};
-
-// q Chebyshev steps on a level: s = A^H t, t = g - A x; d = c2[m] s + c1[m] d
-// (c1[0] = 0); x += d.  x of the nodes in registers and (unless xzero) in X.
-template <typename T>
-__device__ __forceinline__ void wt_cheb(WtNodes<T>& N, int q, bool xzero, cplx<T>* X, cplx<T>* Tt, T ih2,
-                                        const T (*c)[16]) {
-    constexpr int RPT = WtNodes<T>::RPT;
-    cplx<T> d[RPT], t[RPT];
-#pragma unroll
-    for (int r = 0; r < RPT; ++r) d[r] = zero2<T>();
-    for (int m = 0; m < q; ++m) {
-        N.residual(t, X, Tt, ih2, xzero && m == 0);
-        __syncthreads();
-        const T c1 = c[0][m], c2 = c[1][m];
-#pragma unroll
-        for (int r = 0; r < RPT; ++r)
-            if (N.in[r]) {
-                cplx<T> dg = N.dg[r];
-                dg.y = -dg.y;
-                const cplx<T> sv = cscale<T>(csub<T>(cmul<T>(dg, t[r]), N.nsum(t, Tt, r)), ih2);
-                cplx<T> dn = cscale<T>(sv, c2);
-                if (c1 != T(0)) dn = cadd<T>(dn, cscale<T>(d[r], c1));
-                d[r] = dn;
-                N.x[r] = cadd<T>(N.x[r], dn);
-                X[N.at(r)] = N.x[r];
-            }
-        __syncthreads();
-    }
-}
-
 // zero the borders (and everything else) of the two shared vectors of a level
 template <typename T> __device__ __forceinline__ void wt_zero(cplx<T>* X, cplx<T>* Tt, const LevelDesc& d) {
     const int e = (d.n + 2) * (d.ny + 2);
@@ -159,7 +91,7 @@ __global__ void __launch_bounds__(WT_THREADS, 1) k_wave_down(const LevelDesc* __
         const LevelDesc& dc = Lv[k + 1];
         const T ih2 = LC<T>::ih2(d);
         WtNodes<T> N;
-        N.place(d);
+        N.place(d.n, d.n, d.ny);
         const cplx<T>* gg = slot<T>(d, SG);
 #pragma unroll
         for (int r = 0; r < RPT; ++r)
@@ -221,7 +153,7 @@ __global__ void __launch_bounds__(WT_THREADS, 1) k_wave_up(const LevelDesc* __re
         const int Wc = Lv[k + 1].n + 2;
         const T ih2 = LC<T>::ih2(d);
         WtNodes<T> N;
-        N.place(d);
+        N.place(d.n, d.n, d.ny);
         const cplx<T>* xg = slot<T>(d, SU);
         const cplx<T>* gg = slot<T>(d, SG);
 #pragma unroll
