@@ -669,7 +669,7 @@ struct Engine : EngineBase {
             return 0;
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit) != cudaSuccess) return 0;
         cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute at[1];
+        cudaLaunchAttribute at[2];
         ct_config(cfg, at, CS, 1, limit, nullptr);
         int nc = 0;
         return cudaOccupancyMaxActiveClusters(&nc, kern, &cfg) == cudaSuccess && nc > 0 ? CS : 0;
@@ -683,8 +683,10 @@ struct Engine : EngineBase {
         at[0].id = cudaLaunchAttributeClusterDimension;
         at[0].val.clusterDim.x = (unsigned)cs;
         at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = at;
-        cfg.numAttrs = 1;
+        cfg.numAttrs = pdl_on() ? 2 : 1;
     }
     static long long ct_smem_limit() {
         static const long long lim = [] {
@@ -750,7 +752,7 @@ struct Engine : EngineBase {
         const double vc = (2 * (3 * C + Q) + (4 * C + Q + C / 4) + (4 * C + Q + C) + 5 * C) * (double)pts + C * (double)mat;
         go(H, st, KK_ADR_TAIL, std::max(corr, 1) * vc + corr * (6 * C + R) * (double)top, [&] {
             cudaLaunchConfig_t cfg = {};
-            cudaLaunchAttribute at[1];
+            cudaLaunchAttribute at[2];
             ct_config(cfg, at, cs, (unsigned)tail.size(), sm, st);
             const LevelDesc* D = H.ddesc;
             if (cs == 16) cudaLaunchKernelEx(&cfg, k_adr_cluster<T, 16>, D, dchain, corr);

@@ -99,31 +99,27 @@ __global__ void __launch_bounds__(CT_THREADS, 1) k_adr_cluster(const LevelDesc* 
     cplx<T>* const K2 = K1 + E0;
     cplx<T>* const U = corr > 0 ? K2 + E0 : nullptr;
     cplx<T>* const Bd = K2 + (corr > 0 ? 2 : 1) * E0;           // dense coarsest right-hand side
-    if (tid == 0) {
+    if (tid < nl) {
         unsigned char* p = reinterpret_cast<unsigned char*>(
             ((uintptr_t)(Bd + Lv[nl - 1].n * Lv[nl - 1].ny) + 15) & ~(uintptr_t)15);
-        for (int k = 0, R = R0; k < nl; ++k, R /= 2) {
-            CtLevel<T>& l = L[k];
-            const LevelDesc& d = Lv[k];
-            l.n = d.n;
-            l.ny = d.ny;
-            l.W = d.n + 2;
-            l.R = R;
-            l.r0 = rank * R;
-            l.r1 = min(l.r0 + R, d.ny);
-            const int e = (R + 2 * CT_HALO) * l.W;
-            l.Q = nullptr;
-            if (ct_quads<T>()) {
-                l.Q = reinterpret_cast<quad<T>*>(p);
-                p += (size_t)e * sizeof(quad<T>);
-            }
-            l.B = reinterpret_cast<cplx<T>*>(p);
-            l.X = l.B + e;
-            p += 2 * (size_t)e * sizeof(cplx<T>);
-            l.ih2 = LC<T>::ih2(d);
-            l.wh = LC<T>::wh(d);
-            l.s = LC<T>::gs(d);
-        }
+        const size_t per = (ct_quads<T>() ? sizeof(quad<T>) : 0) + 2 * sizeof(cplx<T>);
+        int R = R0;
+        for (int k = 0; k < tid; ++k, R /= 2) p += (size_t)(R + 2 * CT_HALO) * (Lv[k].n + 2) * per;
+        CtLevel<T>& l = L[tid];
+        const LevelDesc& d = Lv[tid];
+        l.n = d.n;
+        l.ny = d.ny;
+        l.W = d.n + 2;
+        l.R = R;
+        l.r0 = rank * R;
+        l.r1 = min(l.r0 + R, d.ny);
+        const int e = (R + 2 * CT_HALO) * l.W;
+        l.Q = ct_quads<T>() ? reinterpret_cast<quad<T>*>(p) : nullptr;
+        l.B = reinterpret_cast<cplx<T>*>(p + (ct_quads<T>() ? (size_t)e * sizeof(quad<T>) : 0));
+        l.X = l.B + e;
+        l.ih2 = LC<T>::ih2(d);
+        l.wh = LC<T>::wh(d);
+        l.s = LC<T>::gs(d);
     }
     __syncthreads();
     // f(local offset, row, column) for rows [r0 + a, r0 + R + b) of level l
@@ -141,21 +137,27 @@ __global__ void __launch_bounds__(CT_THREADS, 1) k_adr_cluster(const LevelDesc* 
         }
     };
     auto none = [](int) {};
-    // everything starts as zero: the halo columns and the rows outside the
-    // grid of b, x and the iterate are never written
+    // Constants of the setup and zeros first, so that this part may run beside
+    // the end of the previous kernel: asynchronous copies of the quads of all
+    // levels, then b, x and the iterate as zero (their halo columns and the
+    // rows outside the grid are never written).
+    if constexpr (ct_quads<T>())
+        for (int k = 0; k + 1 < nl; ++k) {
+            const quad<T>* const a = reinterpret_cast<const quad<T>*>(Lv[k].adr);
+            const int pitch = Lv[k].pitch;
+            quad<T>* const Q = L[k].Q;
+            over(L[k], -3, 3,
+                 [&](int o, int row, int c) { cp_async_elem(Q + o, a + (long long)row * pitch + c, true); }, none);
+        }
     for (int k = 0; k < nl; ++k) {
         const int e = (L[k].R + 2 * CT_HALO) * L[k].W;
         for (int q = tid; q < 2 * e; q += CT_THREADS) L[k].B[q] = zero2<T>();
     }
     if (corr > 0)
         for (int q = tid; q < E0; q += CT_THREADS) U[q] = zero2<T>();
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     cl.sync();   // every block of the cluster runs and its memory is set
-    if (ct_quads<T>())
-        for (int k = 0; k + 1 < nl; ++k) {
-            const LevelDesc& d = Lv[k];
-            quad<T>* const Q = L[k].Q;
-            over(L[k], -3, 3, [&](int o, int row, int c) { Q[o] = load_adr<T>(d, (long long)row * d.pitch + c); }, none);
-        }
     auto quad_at = [&](const CtLevel<T>& l, const LevelDesc& d, int o, int row, int c) {
         return ct_quads<T>() ? l.Q[o] : load_adr<T>(d, (long long)row * d.pitch + c);
     };
@@ -214,7 +216,10 @@ __global__ void __launch_bounds__(CT_THREADS, 1) k_adr_cluster(const LevelDesc* 
     const LevelDesc& d0 = Lv[0];
     if (corr > 0) {
         const cplx<T>* u = slot<T>(d0, SU);
-        over(L[0], -1, 1, [&](int o, int row, int c) { U[o] = u[(long long)row * d0.pitch + c]; }, none);
+        over(L[0], -1, 1,
+             [&](int o, int row, int c) { cp_async_elem(U + o, u + (long long)row * d0.pitch + c, true); }, none);
+        cp_async_commit();
+        cp_async_wait<0>();
         __syncthreads();
     }
     const int rounds = corr > 0 ? corr : 1;
@@ -239,10 +244,25 @@ __global__ void __launch_bounds__(CT_THREADS, 1) k_adr_cluster(const LevelDesc* 
         } else {
             const cplx<T>* b = slot<T>(d0, SAB);
             cplx<T>* const B0 = L[0].B;
-            over(L[0], -CT_HALO, CT_HALO, [&](int o, int row, int c) { B0[o] = b[(long long)row * d0.pitch + c]; },
-                 none);
+            over(L[0], -CT_HALO, CT_HALO,
+                 [&](int o, int row, int c) { cp_async_elem(B0 + o, b + (long long)row * d0.pitch + c, true); }, none);
+            cp_async_commit();
+            cp_async_wait<0>();
         }
         __syncthreads();
+        // the first 256 values of a row of the inverse; this warp's first row
+        // (FP32) is fetched while the last level above the coarsest is smoothed
+        const int N = L[nl - 1].n * L[nl - 1].ny, p0 = L[nl - 1].r0 * L[nl - 1].n + w, p1 = L[nl - 1].r1 * L[nl - 1].n;
+        const cplx<T>* const inv = reinterpret_cast<const cplx<T>*>(Lv[nl - 1].inv_adr);
+        constexpr bool early = ct_quads<T>();   // (FP64 has no registers to spare)
+        cplx<T> av[8];
+        auto fetch = [&](int p) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int q = lane + 32 * u;
+                av[u] = q < N ? __ldg(inv + (long long)p * N + q) : zero2<T>();
+            }
+        };
         // down: GMRES(3) from x = 0, x kept, the residual restricted to the next b
         for (int k = 0; k + 1 < nl; ++k) {
             const CtLevel<T>& l = L[k];
@@ -266,6 +286,7 @@ __global__ void __launch_bounds__(CT_THREADS, 1) k_adr_cluster(const LevelDesc* 
                      [&](int o) { K0[o] = zero2<T>(); });
             }
             solve(g);
+            if (early && k + 2 == nl && p0 < p1) fetch(p0);
             {
                 const cplx<T> c0 = sload2<T>(scl, S::GC), c1 = sload2<T>(scl, S::GC + 2), c2 = sload2<T>(scl, S::GC + 4);
                 const cplx<T> sc0 = cscale<T>(c0, l.s), sc1 = cscale<T>(c1, l.s), sc2 = cscale<T>(c2, l.s);
@@ -302,33 +323,36 @@ __global__ void __launch_bounds__(CT_THREADS, 1) k_adr_cluster(const LevelDesc* 
         {
             // coarsest solve: the whole right-hand side in every block, a warp per own row of the inverse
             const CtLevel<T>& l = L[nl - 1];
-            const int n = l.n, N = n * l.ny;
+            const int n = l.n;
             for (int row = w; row < l.ny; row += CT_WARPS) {
                 const int own = row / l.R;
                 const cplx<T>* src = cl.map_shared_rank(l.B, own) + (row - own * l.R + CT_HALO) * l.W + 1;
                 for (int c = lane; c < n; c += 32) Bd[row * n + c] = src[c];
             }
             __syncthreads();
-            const cplx<T>* inv = reinterpret_cast<const cplx<T>*>(Lv[nl - 1].inv_adr);
-            for (int p = l.r0 * n + w; p < l.r1 * n; p += CT_WARPS) {
-                const cplx<T>* a = inv + (long long)p * N;
+            for (int p = p0; p < p1; p += CT_WARPS) {
+                if (!early || p != p0 || nl < 2) fetch(p);
                 // as k_coarse: four independent accumulators
                 cplx<T> ac[4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u) ac[u] = zero2<T>();
-                for (int q0 = lane; q0 < N; q0 += 128) {
+                auto add = [&](int u, int q, cplx<T> a) {
+                    if (q < N) {
+                        const cplx<T> bv = Bd[q];
+                        ac[u].x = fma(a.x, bv.x, ac[u].x);
+                        ac[u].x = fma(-a.y, bv.y, ac[u].x);
+                        ac[u].y = fma(a.x, bv.y, ac[u].y);
+                        ac[u].y = fma(a.y, bv.x, ac[u].y);
+                    }
+                };
+#pragma unroll
+                for (int u = 0; u < 8; ++u) add(u & 3, lane + 32 * u, av[u]);
+                for (int q0 = lane + 256; q0 < N; q0 += 128)
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         const int q = q0 + 32 * u;
-                        if (q < N) {
-                            const cplx<T> av = __ldg(a + q), bv = Bd[q];
-                            ac[u].x = fma(av.x, bv.x, ac[u].x);
-                            ac[u].x = fma(-av.y, bv.y, ac[u].x);
-                            ac[u].y = fma(av.x, bv.y, ac[u].y);
-                            ac[u].y = fma(av.y, bv.x, ac[u].y);
-                        }
+                        add(u, q, q < N ? __ldg(inv + (long long)p * N + q) : zero2<T>());
                     }
-                }
                 cplx<T> acc = cadd<T>(cadd<T>(ac[0], ac[1]), cadd<T>(ac[2], ac[3]));
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) {
