@@ -17,8 +17,8 @@
 //               the next level; post-smoothing: x = x' + z, pointwise (at
 //               level 2 added to the wave iterate as exp(+i w phi) x).
 // The same minimiser as the Arnoldi form; in the working precision the Gram
-// form loses accuracy like cond(K)^2, which the small block-tree reductions
-// keep below the Arnoldi form's error on the ADR levels of the cycle.
+// form loses accuracy like cond(K)^2, which in FP32 compensated sums over the
+// warps and one refinement step of the small solve take back (gs_solve).
 //
 // The gram pass exists as a shared-memory tile kernel (two tile shapes) and
 // as a warp-streaming kernel (two band heights); the pre-smoothing update as
@@ -59,65 +59,188 @@ template <typename T> struct GsEps;
 template <> struct GsEps<float> { static constexpr float tau = 32.0f * 1.1920929e-7f; };
 template <> struct GsEps<double> { static constexpr double tau = 32.0 * 2.220446049250313e-16; };
 
-// 1 / sqrt(x): in FP64 one call (a square root and a division are ~560 ns of
-// dependent FP64 operations here)
-__device__ __forceinline__ float inv_sqrt(float x) { return 1.0f / sqrtf(x); }
-__device__ __forceinline__ double inv_sqrt(double x) { return rsqrt(x); }
+// 1 / sqrt(x) in one call (a square root and a division are ~560 ns of
+// dependent FP64 operations here); its 2 ulp in FP32 are within what the
+// refinement in gs_solve removes.
+__device__ __forceinline__ float gs_rsqrt(float x) { return rsqrtf(x); }
+__device__ __forceinline__ double gs_rsqrt(double x) { return rsqrt(x); }
 
-// Normal equations of the s-step GMRES(3) in the last block (thread 0).
-// G[0] = (|K0|^2, |K1|^2), G[1] = (|K2|^2, |K3|^2), G[2..4] = <K0, K1..K3>,
-// G[5] = <K1,K2>, G[6] = <K1,K3>, G[7] = <K2,K3>  (<a,b> = sum conj(a) b).
+// A sum over parts of a level, e.g. the warps of a block.  In FP32 it carries
+// what the additions lost (two-sum, h + l), in FP64 it is the plain sum.
+// The last few additions of a long sum are the ones whose rounding does not
+// average out: with plain FP32 sums the ten Gram entries were each off by ~1
+// ulp, the normal equations multiply that by cond(K)^2, and this was nearly
+// all of the mixed cycle's error against 64 bits (see gs_solve).  Sums within
+// a warp stay plain (an FP64 addition holds a warp's pipe for 64 cycles, a
+// two-sum takes 7 pipelined FP32 instructions).
+template <typename T> struct GsSum;
+template <> struct __align__(8) GsSum<float> {
+    float h, l;
+    __device__ __forceinline__ void clear() { h = l = 0.0f; }
+    // h + x and its error (exact in either order)
+    static __device__ __forceinline__ float two_sum(float a, float b, float& err) {
+        const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+        err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+        return s;
+    }
+    __device__ __forceinline__ void add(float x) {
+        float e;
+        h = two_sum(h, x, e);
+        l += e;
+    }
+    // (the same bits whichever of the two is added to the other)
+    __device__ __forceinline__ void add(const GsSum& o) {
+        float e;
+        h = two_sum(h, o.h, e);
+        l = e + (l + o.l);
+    }
+    // minus a x, x in working precision
+    __device__ __forceinline__ void sub_prod(const GsSum& a, float x) {
+        const float p = __fmul_rn(a.h, x);
+        float e;
+        h = two_sum(h, -p, e);
+        l = __fmaf_rn(-a.l, x, l + (e - __fmaf_rn(a.h, x, -p)));
+    }
+    __device__ __forceinline__ GsSum from(int lane) const {
+        return GsSum{__shfl_sync(0xffffffffu, h, lane), __shfl_sync(0xffffffffu, l, lane)};
+    }
+    __device__ __forceinline__ GsSum peer(int o) const {
+        return GsSum{__shfl_xor_sync(0xffffffffu, h, o), __shfl_xor_sync(0xffffffffu, l, o)};
+    }
+    // h the nearest value, l the rest; a sum that overflowed stays as it is
+    __device__ __forceinline__ void norm() {
+        float e;
+        const float s = two_sum(h, l, e);
+        const bool fin = fabsf(s) <= 3.402823466e38f;
+        h = fin ? s : h;
+        l = fin ? e : 0.0f;
+    }
+    static __device__ __forceinline__ GsSum ldcg(const GsSum* p) {
+        const float2 v = __ldcg(reinterpret_cast<const float2*>(p));
+        return GsSum{v.x, v.y};
+    }
+};
+template <> struct GsSum<double> {
+    double h;
+    __device__ __forceinline__ void clear() { h = 0.0; }
+    __device__ __forceinline__ void add(double x) { h += x; }
+    __device__ __forceinline__ void add(const GsSum& o) { h += o.h; }
+    __device__ __forceinline__ GsSum peer(int o) const { return GsSum{__shfl_xor_sync(0xffffffffu, h, o)}; }
+    __device__ __forceinline__ void norm() {}
+    static __device__ __forceinline__ GsSum ldcg(const GsSum* p) { return GsSum{__ldcg(&p->h)}; }
+};
+template <typename T> __device__ __forceinline__ T gs_hi(const GsSum<T>& v) { return v.h; }
+
+// Factor of the 3 x 3 normal equations W^H W c = f, W = (K1, K2, K3):
 // Jacobi-scaled Cholesky; a column whose pivot (squared sine of its angle to
 // the previous columns) is below tau ends the Krylov space (breakdown), as
-// does r0 = 0.  Stores c (3 complex), the dimension used and ||r||^2.
-template <typename T>
-__device__ inline void gs_solve(const cplx<T> (&G)[8], T* sc) {
-    const T dg[3] = {G[0].y, G[1].x, G[1].y};
-    int m = 0;
-    T dsc[3] = {T(0), T(0), T(0)};
-    if (G[0].x > T(0))
-        while (m < 3 && dg[m] > T(0)) { dsc[m] = inv_sqrt(dg[m]); ++m; }
-    cplx<T> bb[3], c[3];
-    for (int i = 0; i < 3; ++i) {
-        bb[i] = cscale<T>(mk<T>(G[2 + i].x, -G[2 + i].y), dsc[i]);   // <K_{i+1}, K0>
-        c[i] = zero2<T>();
-    }
-    const cplx<T> r01 = cscale<T>(G[5], dsc[0] * dsc[1]);
-    const cplx<T> r02 = cscale<T>(G[6], dsc[0] * dsc[2]);
-    const cplx<T> a12 = cscale<T>(G[7], dsc[1] * dsc[2]);
-    T i11 = T(1), i22 = T(1);   // inverse pivots
-    cplx<T> r12 = zero2<T>();
-    if (m >= 2) {
+// does r0 = 0.
+// G[0] = (|K0|^2, |K1|^2), G[1] = (|K2|^2, |K3|^2), G[2..4] = <K0, K1..K3>,
+// G[5] = <K1,K2>, G[6] = <K1,K3>, G[7] = <K2,K3>  (<a,b> = sum conj(a) b).
+template <typename T> struct GsFactor {
+    T d0, d1, d2, i11, i22;      // column scales, inverse pivots (zero from the first unused column on)
+    cplx<T> r01, r02, r12;
+    bool ok0, ok1, ok2;          // columns used
+    __device__ __forceinline__ explicit GsFactor(const cplx<T> (&G)[8]) {
+        const T g0 = G[0].y, g1 = G[1].x, g2 = G[1].y;
+        const cplx<T> zero = zero2<T>();
+        ok0 = G[0].x > T(0) && g0 > T(0);
+        ok1 = ok0 && g1 > T(0);
+        ok2 = ok1 && g2 > T(0);
+        d0 = ok0 ? gs_rsqrt(g0) : T(0);
+        d1 = ok1 ? gs_rsqrt(g1) : T(0);
+        d2 = ok2 ? gs_rsqrt(g2) : T(0);
+        r01 = cscale<T>(G[5], d0 * d1);
+        r02 = cscale<T>(G[6], d0 * d2);
         const T p1 = T(1) - cabs2<T>(r01);
-        if (p1 > GsEps<T>::tau) i11 = inv_sqrt(p1);
-        else m = 1;
-    }
-    if (m >= 3) {
-        r12 = cscale<T>(csub<T>(a12, cmulc<T>(r01, r02)), i11);
+        ok1 = ok1 && p1 > GsEps<T>::tau;
+        i11 = ok1 ? gs_rsqrt(p1) : T(0);
+        r12 = cscale<T>(csub<T>(cscale<T>(G[7], d1 * d2), cmulc<T>(r01, r02)), i11);
         const T p2 = T(1) - cabs2<T>(r02) - cabs2<T>(r12);
-        if (p2 > GsEps<T>::tau) i22 = inv_sqrt(p2);
-        else m = 2;
+        ok2 = ok2 && ok1 && p2 > GsEps<T>::tau;
+        i22 = ok2 ? gs_rsqrt(p2) : T(0);
+        r01 = ok1 ? r01 : zero;
+        r02 = ok2 ? r02 : zero;
+        r12 = ok2 ? r12 : zero;
     }
-    // R^H z = bb, then R c = z, on the leading m columns
-    cplx<T> z[3];
-    z[0] = bb[0];
-    z[1] = cscale<T>(csub<T>(bb[1], cmulc<T>(r01, z[0])), i11);
-    z[2] = cscale<T>(csub<T>(csub<T>(bb[2], cmulc<T>(r02, z[0])), cmulc<T>(r12, z[1])), i22);
-    if (m == 3) {
-        c[2] = cscale<T>(z[2], i22);
-        c[1] = cscale<T>(csub<T>(z[1], cmul<T>(r12, c[2])), i11);
-        c[0] = csub<T>(csub<T>(z[0], cmul<T>(r01, c[1])), cmul<T>(r02, c[2]));
-    } else if (m == 2) {
-        c[1] = cscale<T>(z[1], i11);
-        c[0] = csub<T>(z[0], cmul<T>(r01, c[1]));
-    } else if (m == 1) {
-        c[0] = z[0];
+    // c for the right-hand side f on the used columns: R^H z = f, R c = z;
+    // returns |z|^2
+    __device__ __forceinline__ T solve(const cplx<T> (&f)[3], cplx<T> (&c)[3]) const {
+        const cplx<T> zero = zero2<T>();
+        const cplx<T> z0 = ok0 ? cscale<T>(f[0], d0) : zero;
+        const cplx<T> z1 = ok1 ? cscale<T>(csub<T>(cscale<T>(f[1], d1), cmulc<T>(r01, z0)), i11) : zero;
+        const cplx<T> z2 =
+            ok2 ? cscale<T>(csub<T>(csub<T>(cscale<T>(f[2], d2), cmulc<T>(r02, z0)), cmulc<T>(r12, z1)), i22) : zero;
+        c[2] = cscale<T>(z2, i22);
+        c[1] = cscale<T>(csub<T>(z1, cmul<T>(r12, c[2])), i11);
+        c[0] = csub<T>(csub<T>(z0, cmul<T>(r01, c[1])), cmul<T>(r02, c[2]));
+        c[0] = cscale<T>(c[0], d0);
+        c[1] = cscale<T>(c[1], d1);
+        c[2] = cscale<T>(c[2], d2);
+        return cabs2<T>(z0) + cabs2<T>(z1) + cabs2<T>(z2);
     }
-    T rr = G[0].x;
-    for (int i = 0; i < m; ++i) rr -= cabs2<T>(z[i]);
-    for (int i = 0; i < 3; ++i) sstore2<T>(sc, S::GC + 2 * i, cscale<T>(c[i], dsc[i]));
-    sc[S::M] = (T)m;
-    sc[S::NORM] = rr;
+};
+
+// the 16 sums of the lanes (value lane / 2) as the entries of GsFactor
+template <typename T> __device__ __forceinline__ void gram_entries(T t, cplx<T> (&G)[8]) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+        G[k] = mk<T>(__shfl_sync(0xffffffffu, t, 4 * k), __shfl_sync(0xffffffffu, t, 4 * k + 2));
+}
+
+// Normal equations of the s-step GMRES(3), one warp; t: the Gram sums, value
+// lane / 2 in each lane.  Stores c (3 complex), the dimension used and
+// ||r||^2.  In FP32 the factor is that of the rounded entries, and one step
+// of refinement takes the residual f - W^H W c from the full sums (lane r:
+// row r), so neither the rounding of the entries nor that of the elimination
+// is multiplied by cond(K)^2.  Error of one mixed cycle against 64 bits over 24
+// media of n = 100 to 700: 4.6e-7 .. 2.1e-6 (median 9e-7) with plain sums, now
+// 1.5e-7 .. 9.7e-7 (2.5e-7), in the same time (the branch-free factor with
+// reciprocal square roots pays for the refinement: cycle at n = 127 98 us
+// before and after, n = 1024 388 -> 393 us).
+template <typename T> __device__ __forceinline__ void gs_solve(GsSum<T> t, int lane, T* sc) {
+    t.norm();
+    cplx<T> G[8], f[3], c[3];
+    gram_entries<T>(gs_hi(t), G);
+    const GsFactor<T> F(G);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) f[i] = mk<T>(G[2 + i].x, -G[2 + i].y);   // <K_{i+1}, K0>
+    const T rr = G[0].x - F.solve(f, c);
+    if constexpr (std::is_same<T, float>::value) {
+        const int r = lane % 3;
+        const GsSum<float> dg = t.from(2 + 2 * r);
+        GsSum<float> re = t.from(8 + 4 * r), im = t.from(10 + 4 * r);
+        // the row's two entries beside the diagonal: (0,1), (0,2) | (1,0), (1,2) | (2,0), (2,1)
+        const int qa = r == 2 ? 24 : 20, qb = r == 0 ? 24 : 28;
+        const GsSum<float> ax = t.from(qa), ay = t.from(qa + 2), bx = t.from(qb), by = t.from(qb + 2);
+        const float2 cd = r == 0 ? c[0] : r == 1 ? c[1] : c[2], ca = r == 0 ? c[1] : c[0], cb = r == 2 ? c[1] : c[2];
+        const float sa = r == 0 ? 1.0f : -1.0f, sb = r == 2 ? -1.0f : 1.0f;   // (lower entries conjugated)
+        im.h = -im.h;
+        im.l = -im.l;
+        re.sub_prod(dg, cd.x);
+        im.sub_prod(dg, cd.y);
+        re.sub_prod(ax, ca.x);
+        re.sub_prod(ay, -sa * ca.y);
+        im.sub_prod(ax, ca.y);
+        im.sub_prod(ay, sa * ca.x);
+        re.sub_prod(bx, cb.x);
+        re.sub_prod(by, -sb * cb.y);
+        im.sub_prod(bx, cb.y);
+        im.sub_prod(by, sb * cb.x);
+        const float vx = re.h + re.l, vy = im.h + im.l;
+        float2 dc[3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) f[i] = make_float2(__shfl_sync(0xffffffffu, vx, i), __shfl_sync(0xffffffffu, vy, i));
+        F.solve(f, dc);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) c[i] = cadd<float>(c[i], dc[i]);
+    }
+    if (lane == 0) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) sstore2<T>(sc, S::GC + 2 * i, c[i]);
+        sc[S::M] = (T)((int)F.ok0 + (int)F.ok1 + (int)F.ok2);
+        sc[S::NORM] = rr;
+    }
 }
 
 // s L at an on-chip point b of a region of row stride W, with the point's
@@ -222,32 +345,29 @@ template <typename T> __device__ __forceinline__ T warp_sum16(T (&v)[16], int la
     }
     return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
-// Sum over q < cnt rows of 16 values at sh, value lane / 2 in each lane
-// (one warp; each lane takes every second row).
-template <typename T> __device__ __forceinline__ T rows_sum16(const T* sh, int cnt, int lane) {
+// Sum over q < cnt rows of 16 values (or sums) at sh, value lane / 2 in each
+// lane (one warp; each lane takes every second row).
+template <typename T, typename V> __device__ __forceinline__ GsSum<T> rows_sum16(const V* sh, int cnt, int lane) {
     const int id = lane >> 1;
-    T t = T(0);
-    for (int q = lane & 1; q < cnt; q += 2) t += sh[q * 16 + id];
-    return t + __shfl_xor_sync(0xffffffffu, t, 1);
-}
-// the 16 sums of the lanes as the entries of gs_solve
-template <typename T> __device__ __forceinline__ void gram_entries(T t, cplx<T> (&G)[8]) {
+    GsSum<T> t;
+    t.clear();
 #pragma unroll
-    for (int k = 0; k < 8; ++k)
-        G[k] = mk<T>(__shfl_sync(0xffffffffu, t, 4 * k), __shfl_sync(0xffffffffu, t, 4 * k + 2));
+    for (int q = lane & 1; q < cnt; q += 2) t.add(sh[q * 16 + id]);
+    t.add(t.peer(1));
+    return t;
 }
 
-// Reduction of the Gram entries of a launch and the small solve; sh: 16
-// values per 16 threads.  This chain ends every sweep, so on small levels it
+// Reduction of the Gram entries of a launch and the small solve; sh: one value
+// per thread, on 16 bytes.  This chain ends every sweep, so on small levels it
 // is most of the pass: with a shuffle tree per value, one thread adding the
 // warps, storing the partials and adding the blocks, a 63 x 63 level took 7.3
 // us in FP32 and 61 us in FP64 (where a warp's addition holds the pipe for 16
 // cycles and a dependent one takes 32 ns).  Now 16 shuffles per warp, a lane
 // per value from there on, every sum split over two lanes or more (FP64 cycle at n = 511 3.44 -> 2.42 ms with the
 // selected upwind stencil, FP32 cycle at n = 1024 450 -> 416 us).
-template <typename T>
+template <typename T, int NTH>
 __device__ __forceinline__ void gram_finish(const LevelDesc& d, const SegCtx& c, const GramAcc<T>& g, T* sh, int* flag) {
-    const int tid = threadIdx.x + threadIdx.y * blockDim.x, nt = blockDim.x * blockDim.y;
+    const int tid = threadIdx.x + threadIdx.y * blockDim.x;
     const int lane = tid & 31, w = tid >> 5;
     {
         cplx<T> ac[8];
@@ -262,15 +382,15 @@ __device__ __forceinline__ void gram_finish(const LevelDesc& d, const SegCtx& c,
         if (!(lane & 1)) sh[w * 16 + (lane >> 1)] = ws;
     }
     __syncthreads();
-    T* const part = reinterpret_cast<T*>(d.part);
+    // 16 sums per block
+    GsSum<T>* const part = reinterpret_cast<GsSum<T>*>(d.part);
+    static_assert(16 * sizeof(GsSum<T>) <= MAXDOT * sizeof(double2), "partials of a block");
     if (w == 0) {
-        T t = rows_sum16<T>(sh, nt >> 5, lane);
+        const GsSum<T> t = rows_sum16<T>(sh, NTH / 32, lane);
         if (c.nb == 1) {
-            cplx<T> G[8];
-            gram_entries<T>(t, G);
-            if (lane == 0) gs_solve<T>(G, scalp<T>(d));
+            gs_solve<T>(t, lane, scalp<T>(d));
         } else {
-            if (!(lane & 1)) part[(long long)c.lb * (2 * MAXDOT) + (lane >> 1)] = t;
+            if (!(lane & 1)) part[(long long)c.lb * 16 + (lane >> 1)] = t;
             __syncwarp();
             if (lane == 0) {
                 __threadfence();
@@ -282,23 +402,22 @@ __device__ __forceinline__ void gram_finish(const LevelDesc& d, const SegCtx& c,
     __syncthreads();
     if (!*flag) return;
     __threadfence();
+    GsSum<T>* const rows = reinterpret_cast<GsSum<T>*>(sh);
     {
-        // value tid % 16 of the blocks tid / 16, tid / 16 + nt / 16, ...
-        const int id = tid & 15, ng = nt >> 4;
-        T s = T(0);
+        // value tid % 16 of the blocks tid / 16, tid / 16 + NTH / 16, ...; the
+        // warp's two shares together
+        const int id = tid & 15, ng = NTH / 16;
+        GsSum<T> s;
+        s.clear();
 #pragma unroll 4
-        for (int b = tid >> 4; b < c.nb; b += ng) s += __ldcg(part + (long long)b * (2 * MAXDOT) + id);
-        sh[tid] = s;
+        for (int b = tid >> 4; b < c.nb; b += ng) s.add(GsSum<T>::ldcg(part + (long long)b * 16 + id));
+        s.add(s.peer(16));
+        if (lane < 16) rows[w * 16 + id] = s;
     }
     __syncthreads();
     if (w == 0) {
-        const T t = rows_sum16<T>(sh, nt >> 4, lane);
-        cplx<T> G[8];
-        gram_entries<T>(t, G);
-        if (lane == 0) {
-            gs_solve<T>(G, scalp<T>(d));
-            *d.counter = 0u;
-        }
+        gs_solve<T>(rows_sum16<T>(rows, NTH / 32, lane), lane, scalp<T>(d));
+        if (lane == 0) *d.counter = 0u;
     }
 }
 
@@ -308,7 +427,7 @@ __device__ __forceinline__ void gram_finish(const LevelDesc& d, const SegCtx& c,
 // (halo 2) of a block's next tile stream in while the current one is
 // computed.
 template <typename T, int TX, int TY>
-__global__ void __launch_bounds__(NT) k_gs_gram_tile(const __grid_constant__ KDesc A, const Seg* __restrict__ Sg,
+__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 4 : 1) k_gs_gram_tile(const __grid_constant__ KDesc A, const Seg* __restrict__ Sg,
                                                      int nseg, int sr0) {
     constexpr int W0 = TX + 6, H0 = TY + 6, W1 = TX + 4, H1 = TY + 4, W2 = TX + 2, H2 = TY + 2;
     static_assert((TX * TY) % NT == 0, "tile");
@@ -318,7 +437,7 @@ __global__ void __launch_bounds__(NT) k_gs_gram_tile(const __grid_constant__ KDe
     cplx<T>* S1 = S0b + 2 * W0 * H0;
     cplx<T>* S2 = S1 + W1 * H1;
     __shared__ LevelDesc d;
-    __shared__ T sh[NT];
+    __shared__ __align__(16) T sh[NT];
     __shared__ int flag;
     SegCtx c = seg_begin(A, Sg, nseg, d);
     const int tid = threadIdx.x + threadIdx.y * blockDim.x;
@@ -369,7 +488,7 @@ __global__ void __launch_bounds__(NT) k_gs_gram_tile(const __grid_constant__ KDe
         buf ^= 1;
     }
     cp_async_wait<0>();
-    gram_finish<T>(d, c, ac, sh, &flag);
+    gram_finish<T, NT>(d, c, ac, sh, &flag);
 }
 
 // ------------------------------------------------------------ gram pass (streaming)
@@ -387,7 +506,7 @@ __global__ void __launch_bounds__(32 * GS_WPB, sizeof(T) == 4 ? 4 : 1) k_gs_gram
     cplx<T>* Kr = reinterpret_cast<cplx<T>*>(reinterpret_cast<quad<T>*>(gs_smem) + GS_WPB * SW_DEP * SW_COLS) +
                   warp * SW_DEP * SW_COLS;
     __shared__ LevelDesc d;
-    __shared__ T sh[32 * GS_WPB];
+    __shared__ __align__(16) T sh[32 * GS_WPB];
     __shared__ int flag;
     SegCtx c = seg_begin(A, Sg, nseg, d);
     const int n = d.n, ny = d.ny, pitch = d.pitch;
@@ -473,7 +592,7 @@ __global__ void __launch_bounds__(32 * GS_WPB, sizeof(T) == 4 ? 4 : 1) k_gs_gram
         cp_async_wait<0>();
         __syncwarp();
     }
-    gram_finish<T>(d, c, ac, sh, &flag);
+    gram_finish<T, 32 * GS_WPB>(d, c, ac, sh, &flag);
 }
 
 // ------------------------------------------------------------ pre-smoothing update

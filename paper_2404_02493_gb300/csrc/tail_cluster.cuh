@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(CT_THREADS, 1) k_adr_cluster(const LevelDesc* 
     __shared__ CtLevel<T> L[CT_MAXL];
     __shared__ int didx[CT_MAXL];
     __shared__ T shw[CT_WARPS * 16];
-    __shared__ T part[2][CS][16];
+    __shared__ GsSum<T> part[2][CS][16];
     __shared__ T scl[S::NORM + 2];
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank();
@@ -200,16 +200,12 @@ __global__ void __launch_bounds__(CT_THREADS, 1) k_adr_cluster(const LevelDesc* 
         __syncthreads();
         if (w == 0) {
             const int id = lane >> 1, h = lane & 1;
-            const T t = rows_sum16<T>(shw, CT_WARPS, lane);
+            const GsSum<T> t = rows_sum16<T>(shw, CT_WARPS, lane);
 #pragma unroll
             for (int p = 0; p < CS; p += 2) *cl.map_shared_rank(&part[par][rank][id], p + h) = t;
         }
         cl.sync();
-        if (w == 0) {
-            cplx<T> G[8];
-            gram_entries<T>(rows_sum16<T>(&part[par][0][0], CS, lane), G);
-            if (lane == 0) gs_solve<T>(G, scl);
-        }
+        if (w == 0) gs_solve<T>(rows_sum16<T>(&part[par][0][0], CS, lane), lane, scl);
         par ^= 1;
         __syncthreads();
     };
