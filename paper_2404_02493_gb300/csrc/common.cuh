@@ -198,6 +198,29 @@ __device__ __forceinline__ cplx<T> helm_diag_h2(const LevelDesc& d, int i, int j
     return mk<T>(re, im);
 }
 
+// a + b and its rounding error, exactly (Knuth's two-sum; the same in either order)
+__device__ __forceinline__ float two_sum(float a, float b, float& err) {
+    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+    err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+    return s;
+}
+
+// the same for a pair, in packed FP32x2 instructions
+__device__ __forceinline__ float2 two_sum2(float2 a, float2 b, float2& err) {
+    auto neg = [](float2 v) { return make_float2(-v.x, -v.y); };
+    const float2 s = __fadd2_rn(a, b), t = __fadd2_rn(s, neg(a));
+    err = __fadd2_rn(__fadd2_rn(a, neg(__fadd2_rn(s, neg(t)))), __fadd2_rn(b, neg(t)));
+    return s;
+}
+// (double)x by integer operations where x is normal: a conversion holds the
+// FP64 pipe (two lanes per SM and clock) like an addition
+__device__ __forceinline__ double widen(float x) {
+    const unsigned b = __float_as_uint(x), ex = b & 0x7f800000u;
+    if (ex == 0u || ex == 0x7f800000u) return (double)x;
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
 // helm_diag_h2 less the 4 of the Laplacian, formed without it: -h^2 k^2 - m
 // ... keeps its own relative precision.
 template <typename T>

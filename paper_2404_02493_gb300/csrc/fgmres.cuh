@@ -7,6 +7,10 @@
 // residual r = g - A u are FP64 (iterative refinement around FGMRES).
 // Arnoldi: classical Gram-Schmidt with one re-orthogonalisation (CGS2),
 // FP64 reductions of per-thread partial sums, Givens rotations on the device.
+// The recorded entries of H match the rounded coefficients (held), and the
+// update of u is a compensated sum: over media of n = 511 the FP64 residual
+// after a restart is 5e-8 .. 2e-7 of itself from the 64-bit one (was 3e-6 ..
+// 1e-5), the field 7e-8 (1.8e-7).
 // The inner index j lives in device memory (fs[FS_J]) so one captured graph
 // serves every inner iteration.
 #pragma once
@@ -70,6 +74,23 @@ __device__ __forceinline__ void finish_fpartials(const LevelDesc& d, int nb, dou
     }
     if (tid == 0) d.counter[2] = 0u;
     __syncthreads();
+}
+
+// The Hessenberg entries are those of the arithmetic on the vectors: a
+// projection is rounded to the vectors' type before it is recorded, a norm is
+// the reciprocal of the rounded reciprocal that scales them, and beta of the
+// restart likewise.  Then A Z = V H holds up to the rounding of single
+// values, which averages out; with FP64 entries beside coefficients rounded
+// to FP32 it is off by ~3e-8 in whole vectors, and the residual of a restart
+// by that times ||g|| / ||r||.
+template <typename TC> __device__ __forceinline__ double held(double x) { return (double)(TC)x; }
+template <typename TC> __device__ __forceinline__ double2 held2(double2 v) {
+    return make_double2(held<TC>(v.x), held<TC>(v.y));
+}
+template <typename TC> __device__ __forceinline__ double held_norm(double x) {
+    if (std::is_same<TC, double>::value) return x;
+    const TC inv = (TC)(1.0 / x);
+    return inv > TC(0) && inv < TC(1e30) ? 1.0 / (double)inv : x;
 }
 
 __device__ __forceinline__ double2 sload2d(const double* s, int off) { return make_double2(s[off], s[off + 1]); }
@@ -338,11 +359,11 @@ __global__ void __launch_bounds__(NT, 1) k_fg_gs(const __grid_constant__ KDesc A
         if (threadIdx.x == 0 && threadIdx.y == 0) {
             double* f = d.fs;
             if (PASS == 0) {
-                for (int q = 0; q <= jj; ++q) sstore2d(f, FS::HC + 2 * q, tot[q]);
+                for (int q = 0; q <= jj; ++q) sstore2d(f, FS::HC + 2 * q, held2<TC>(tot[q]));
             } else if (PASS == 1) {
-                for (int q = 0; q <= jj; ++q) sstore2d(f, FS::CC + 2 * q, tot[q]);
+                for (int q = 0; q <= jj; ++q) sstore2d(f, FS::CC + 2 * q, held2<TC>(tot[q]));
             } else {
-                const double hnext = sqrt(tot[NVF - 1].x);
+                const double hnext = held_norm<TC>(sqrt(tot[NVF - 1].x));
                 f[FS::HN + jj + 1] = hnext;
                 // column j: h_ij = first + second pass projections
                 double2 col[MAXR + 1];
@@ -607,13 +628,13 @@ __global__ void __launch_bounds__(NT, 1) k_fg_lag(const __grid_constant__ KDesc 
     const int j = jj, lane = tid;
     const double2 zero = make_double2(0.0, 0.0);
     if (PASS == 0) {
-        const double2 S1 = lane < j ? tot[lane] : zero, S2 = lane < j ? tot[j + lane] : zero;
+        const double2 S1 = lane < j ? held2<TC>(tot[lane]) : zero, S2 = lane < j ? held2<TC>(tot[j + lane]) : zero;
         const double2 s12 = dmulc(S1, S2);
         const double ss = warp_dsum(dabs2(S1));
         const double2 ps = make_double2(warp_dsum(s12.x), warp_dsum(s12.y));
         // V_0 comes normalised from the restart; later vectors lose their projections
         const double b2 = j == 0 ? 1.0 : tot[2 * j + 1].x - ss;
-        const double beta = b2 > 0.0 ? sqrt(b2) : 1e-300;
+        const double beta = b2 > 0.0 ? held_norm<TC>(sqrt(b2)) : 1e-300;
         if (j >= 1) {
             // column j-1 final: rows q < j gain ||W1_{j-1}|| S1_q, row j is ||W1_{j-1}|| beta
             const double hn = __shfl_sync(0xffffffffu, hnp, 0);
@@ -643,13 +664,13 @@ __global__ void __launch_bounds__(NT, 1) k_fg_lag(const __grid_constant__ KDesc 
             sstore2d(f, FS::H + 2 * (lane * MAXR + j), S2);
         }
         if (lane == 0) {
-            const double2 hj = dsc(dsub(tot[2 * j], ps), 1.0 / beta);
+            const double2 hj = held2<TC>(dsc(dsub(tot[2 * j], ps), 1.0 / beta));
             sstore2d(f, FS::HC + 2 * j, hj);
             sstore2d(f, FS::H + 2 * (j * MAXR + j), hj);
             f[FS::BETA] = beta;
         }
     } else {
-        const double hn = sqrt(tot[0].x);
+        const double hn = held_norm<TC>(sqrt(tot[0].x));
         // provisional rotation of the pending column j: the residual estimate
         double2 a;
         fg_rotate_warp(lane, j, hrow, cs, sn, a);
@@ -666,6 +687,21 @@ __global__ void __launch_bounds__(NT, 1) k_fg_lag(const __grid_constant__ KDesc 
     }
 }
 
+// Vectors of Z loaded at once per node: with all 22 in flight the kernel took
+// 100 registers, and the FP64 conversions held its FP64 pipes (10 steps at n =
+// 4095: 21.49 ms with plain sums and 22 loads, 21.91 compensated, 21.13 in
+// groups of five at 62 registers and with widen()).
+constexpr int FG_ZPL = 5;
+
+// (e, l) += (y + yl) z for a pair z, e the rounded sum and l what its
+// roundings lost
+__device__ __forceinline__ void fg_acc(float2& e, float2& l, float2 y, float2 yl, float2 z) {
+    const float2 p = __fmul2_rn(y, z), low = __ffma2_rn(y, z, make_float2(-p.x, -p.y));
+    float2 err;
+    e = two_sum2(e, p, err);
+    l = __ffma2_rn(yl, z, __fadd2_rn(l, __fadd2_rn(err, low)));
+}
+
 // y = R^{-1} gamma, then u += ||r|| sum_i y_i Z_i.  Every block solves the
 // (tiny) triangular system in one warp, a row per lane with R staged in shared
 // memory and the diagonal inverted up front (one thread reading R from global
@@ -677,6 +713,8 @@ __global__ void __launch_bounds__(NT) k_fg_update(const __grid_constant__ KDesc 
                                                   int nseg) {
     __shared__ LevelDesc d;
     __shared__ double2 ysh[MAXR];
+    __shared__ float4 yf[FG_ZPL * ((MAXR + FG_ZPL - 1) / FG_ZPL)];   // FP32: y rounded, and what that leaves
+    __shared__ double sc_sh;
     __shared__ double2 Rsh[MAXR * MAXR];   // [column][row]
     SegCtx c = seg_begin(A, Sg, nseg, d);
     const int tid = threadIdx.x + threadIdx.y * blockDim.x;
@@ -708,27 +746,57 @@ __global__ void __launch_bounds__(NT) k_fg_update(const __grid_constant__ KDesc 
         for (int q = m - 1; q >= 0; --q) {
             const double2 y = shfl_d2(dmul(acc, rinv), q);
             if (lane < q) acc = dsub(acc, dmul(Rsh[q * MAXR + lane], y));
-            if (lane == q) ysh[q] = y;
+            if (lane == q) {
+                ysh[q] = y;
+                if (std::is_same<TC, float>::value)
+                    yf[q] = make_float4((float)y.x, (float)y.y, (float)(y.x - held<TC>(y.x)),
+                                        (float)(y.y - held<TC>(y.y)));
+            }
         }
     }
+    if (tid == 32) {
+        const double sc0 = scalp<double>(d)[S::SCALE];
+        sc_sh = sc0 > 0 ? held_norm<TC>(sc0) : sc0;
+    }
     __syncthreads();
-    const double sc = scalp<double>(d)[S::SCALE];
-    cplx<TC> yq[MAXR];
-#pragma unroll
-    for (int q = 0; q < MAXR; ++q) yq[q] = q < m ? from_d<TC>(ysh[q]) : zero2<TC>();
+    const double sc = sc_sh;
     const int ntx = (d.n + BX - 1) / BX, nty = (d.ny + BY - 1) / BY;
     double2* u = slot<double>(d, SU);
     for (int t = c.lb; t < ntx * nty; t += c.nb) {
         const int i = (t % ntx) * BX + threadIdx.x, j = (t / ntx) * BY + threadIdx.y;
         if (i >= d.n || j >= d.ny) continue;
         const long long p = (long long)j * d.pitch + i;
-        // e = Z y accumulated in the cycle precision over <= 22 terms,
-        // then added to the FP64 solution
-        cplx<TC> e = zero2<TC>();
+        // e = Z y, added to the FP64 solution.  In FP32 the sum is a
+        // compensated one over the exact products (with y in two parts): the
+        // operator amplifies the rounding of a plain sum by ~4 / h^2, which
+        // raised the residual of a restart (n = 511, ||r|| = 0.03 ||g||) by
+        // 5e-6 of itself.  In FP64 the products would hold the FP64 pipes.
+        cplx<TC> e = zero2<TC>(), el = zero2<TC>();
+        if constexpr (std::is_same<TC, float>::value) {
+            const float2* z0 = zvec<TC>(d, 0) + p;
+            for (int q = 0; q < m; q += FG_ZPL) {
+                float2 z[FG_ZPL];
 #pragma unroll
-        for (int q = 0; q < MAXR; ++q)
-            if (q < m) e = cfma<TC>(yq[q], __ldg(zvec<TC>(d, q) + p), e);
-        u[p] = dadd(u[p], dsc(to_d(e), sc));
+                for (int k = 0; k < FG_ZPL; ++k)
+                    z[k] = q + k < m ? __ldg(z0 + (long long)(q + k) * d.slot_stride) : make_float2(0.0f, 0.0f);
+#pragma unroll
+                for (int k = 0; k < FG_ZPL; ++k) {
+                    if (q + k >= m) break;
+                    const float4 y = yf[q + k];
+                    fg_acc(e, el, make_float2(y.x, y.x), make_float2(y.z, y.z), z[k]);
+                    fg_acc(e, el, make_float2(-y.y, y.y), make_float2(-y.w, y.w), make_float2(z[k].y, z[k].x));
+                }
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < MAXR; ++q)
+                if (q < m) e = cfma<TC>(from_d<TC>(ysh[q]), __ldg(zvec<TC>(d, q) + p), e);
+        }
+        double2 v = u[p];
+        v = make_double2(fma(sc, widen(e.x), v.x), fma(sc, widen(e.y), v.y));
+        if constexpr (std::is_same<TC, float>::value)
+            v = make_double2(fma(sc, widen(el.x), v.x), fma(sc, widen(el.y), v.y));
+        u[p] = v;
     }
 }
 

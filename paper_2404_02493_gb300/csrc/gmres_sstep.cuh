@@ -77,12 +77,6 @@ template <typename T> struct GsSum;
 template <> struct __align__(8) GsSum<float> {
     float h, l;
     __device__ __forceinline__ void clear() { h = l = 0.0f; }
-    // h + x and its error (exact in either order)
-    static __device__ __forceinline__ float two_sum(float a, float b, float& err) {
-        const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
-        err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
-        return s;
-    }
     __device__ __forceinline__ void add(float x) {
         float e;
         h = two_sum(h, x, e);
