@@ -2,7 +2,7 @@
 // allocation, for callers that cannot call cudaMalloc (see
 // mg_residual_norm_noalloc in include/wave_adr.h).
 //
-// The reduction scratch (one complex partial sum per block and the
+// The reduction scratch (one partial sum per block and the
 // last-block counter) lives in file-scope __device__ arrays of fixed size;
 // every GPU that loads the library holds them until the process exits.
 #include <cuda_runtime.h>
@@ -17,10 +17,10 @@
 
 namespace wadr {
 
-constexpr int NA_MAX_BLOCKS = 1216;          // 8 blocks per SM on 152 SMs
+constexpr int NA_MAX_BLOCKS = 760;           // 5 blocks per SM on 152 SMs: what its registers let be resident
 constexpr int NA_MAX_N = 32768;              // largest accepted grid side
 
-static __device__ __align__(256) double2 na_partials[NA_MAX_BLOCKS];
+static __device__ __align__(256) double na_partials[NA_MAX_BLOCKS];
 static __device__ __align__(256) unsigned na_counter[64];
 
 // r = g - A u and ||r||^2 on a dense grid of ny rows of n nodes (pitch n),
@@ -29,16 +29,23 @@ static __device__ __align__(256) unsigned na_counter[64];
 // mg_setup: gamma(d) = omega ((W-d)/W)^p for d < W = width 2 pi/omega, d the
 // distance to the boundary of [0, lx] x [0, ly], the longer side of unit
 // length) instead of a stored field.
+//
+// What bounds it: the FP64 pipes (14 operations per interior node, 25 us at n =
+// 1023 where its bytes take 9), so what is not a node's arithmetic counts: 1216
+// blocks were 1.6 waves, and a shuffle tree per warp of a complex sum was an
+// eighth of the instructions.  One wave, the threads' sums through shared
+// memory and a single warp's tree per block: n = 1023 56.8 -> 49.2 us.  (One
+// form for interior and boundary nodes, 40 registers: 52.6 us, not kept.)
 __global__ void __launch_bounds__(NT) k_residual_norm_na(int n, int ny, double h, double ih2, double omega, int bc,
                                                          double W, double spower, double lx, double ly,
                                                          const double* __restrict__ k,
                                                          const double2* __restrict__ u, const double2* __restrict__ g,
                                                          double2* __restrict__ r, double* __restrict__ norm2,
-                                                         double2* __restrict__ part, unsigned* __restrict__ counter) {
-    __shared__ double2 sh[8];
+                                                         double* __restrict__ part, unsigned* __restrict__ counter) {
+    __shared__ double sh[NT];
     __shared__ int flag;
     const int ntx = (n + BX - 1) / BX, nty = (ny + BY - 1) / BY;
-    double2 acc[1] = {{0.0, 0.0}};
+    double acc = 0.0;
     for (int t = blockIdx.x; t < ntx * nty; t += gridDim.x) {
         const int i = (t % ntx) * BX + threadIdx.x, j = (t / ntx) * BY + threadIdx.y;
         if (i >= n || j >= ny) continue;
@@ -46,7 +53,7 @@ __global__ void __launch_bounds__(NT) k_residual_norm_na(int n, int ny, double h
         if (bc != BC_SPONGE && i > 0 && i < n - 1 && j > 0 && j < ny - 1) {
             const double2 rv = helm_residual_in(u, g, p, n, k[p], h, ih2);
             r[p] = rv;
-            acc[0].x = fma(rv.y, rv.y, fma(rv.x, rv.x, acc[0].x));
+            acc = fma(rv.y, rv.y, fma(rv.x, rv.x, acc));
             continue;
         }
         const double kk = k[p], kh = kk * h;
@@ -71,19 +78,44 @@ __global__ void __launch_bounds__(NT) k_residual_norm_na(int n, int ny, double h
         const double2 au = dsc(dsub(dmul(make_double2(re, im), uc), s), ih2);
         const double2 rv = dsub(g[p], au);
         r[p] = rv;
-        acc[0].x += dabs2(rv);
+        acc += dabs2(rv);
     }
-    block_sum<double2, 1>(acc, sh);
-    if (publish_partials<double2, 1>(part, 1, counter, blockIdx.x, gridDim.x, acc, &flag)) {
-        double2 tot[1];
-        finish_partials<double2, 1>(part, 1, counter, gridDim.x, tot, sh);
-        if (threadIdx.x == 0 && threadIdx.y == 0) *norm2 = tot[0].x;
+    const int tid = threadIdx.y * BX + threadIdx.x;
+    // sum over the block, in lane 0 of warp 0
+    auto block_total = [&](double v) {
+        sh[tid] = v;
+        __syncthreads();
+        double t = 0.0;
+        if (tid < 32) {
+            t = sh[tid];
+#pragma unroll
+            for (int q = 1; q < NT / 32; ++q) t += sh[tid + 32 * q];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+        }
+        return t;
+    };
+    const double mine = block_total(acc);
+    if (tid == 0) {
+        part[blockIdx.x] = mine;
+        __threadfence();
+        flag = atomicAdd(counter, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!flag) return;
+    __threadfence();
+    double s = 0.0;
+    for (int b = tid; b < (int)gridDim.x; b += NT) s += __ldcg(part + b);
+    const double all = block_total(s);
+    if (tid == 0) {
+        *norm2 = all;
+        *counter = 0u;
     }
 }
 
 namespace {
 struct NaSymbols {
-    double2* part = nullptr;
+    double* part = nullptr;
     unsigned* counter = nullptr;
     bool ready = false;
 };
@@ -139,7 +171,7 @@ extern "C" int mg_residual_norm_noalloc_rect(int n, int ny, double omega, const 
     cudaError_t e = cudaMemsetAsync(s->counter, 0, sizeof(unsigned), st);
     if (e != cudaSuccess) { set_error(std::string("mg_residual_norm_noalloc: ") + cudaGetErrorString(e)); return MG_ECUDA; }
     // the constants are formed here: two FP64 divisions in every thread were a
-    // third of the kernel's FP64 instructions (n = 1023: 66.5 us with them, 56.7 us without)
+    // third of the kernel's FP64 instructions (n = 1023: 66.5 -> 56.7 us when they moved)
     const int m = std::max(n, ny);
     const double h = 1.0 / (m + 1), lx = n == m ? 1.0 : (n + 1) * h, ly = ny == m ? 1.0 : (ny + 1) * h;
     const double W = bc != BC_SPONGE        ? 0.0
