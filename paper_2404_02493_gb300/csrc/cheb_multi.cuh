@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(WT_THREADS, 1) k_cheb_region(const __grid_cons
                 const long long p = (long long)gj * pitch + gi;
                 if (!xzero) N.x[r] = xin[p];
                 N.g[r] = gv[p];
-                N.dg[r] = helm_diag_at<T>(d, gi, gj);
+                N.dg[r] = wt_diag<T>(d, gi, gj);
             }
             // (nodes outside the grid are zero in both vectors)
             X[N.at(r)] = N.x[r];

@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(WT_THREADS, 1) k_wave_down(const LevelDesc* __
         for (int r = 0; r < RPT; ++r)
             if (N.in[r]) {
                 N.g[r] = k == 0 ? gg[(long long)(N.j0 + r) * d.pitch + N.i] : Gn[(N.j0 + r) * d.n + N.i];
-                N.dg[r] = helm_diag_at<T>(d, N.i, N.j0 + r);
+                N.dg[r] = wt_diag<T>(d, N.i, N.j0 + r);
             }
         wt_zero<T>(X, Tt, d);
         __syncthreads();
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(WT_THREADS, 1) k_wave_up(const LevelDesc* __re
                 const long long p = (long long)(N.j0 + r) * d.pitch + N.i;
                 N.x[r] = xg[p];
                 N.g[r] = gg[p];
-                N.dg[r] = helm_diag_at<T>(d, N.i, N.j0 + r);
+                N.dg[r] = wt_diag<T>(d, N.i, N.j0 + r);
             }
         wt_zero<T>(X, Tt, d);
         __syncthreads();
