@@ -847,11 +847,29 @@ static void* slot_ptr(const Handle& H, const LevelHost& lv, int s) {
     return (char*)lv.vec + (size_t)s * lv.slot_stride * esz(H.prec);
 }
 
-static int ensure_graph(mg_handle* h) {
+// The graph stream (non-blocking) waits for what `st` holds so far: the
+// warm-up of a capture runs on the workspace, and an asynchronous call of the
+// handle (mg_cycle on device arrays) may still be using it there.  A stream
+// that is being captured runs nothing yet.
+static int order_after(Handle& H, cudaStream_t st) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    WADR_CHECK(cudaStreamIsCapturing(st, &cap));
+    if (cap != cudaStreamCaptureStatusNone) return MG_OK;
+    cudaEvent_t ev = nullptr;
+    WADR_CHECK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+    cudaError_t e = cudaEventRecord(ev, st);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(H.g_stream, ev, 0);
+    cudaEventDestroy(ev);
+    WADR_CHECK(e);
+    return MG_OK;
+}
+
+static int ensure_graph(mg_handle* h, cudaStream_t st) {
     Handle& H = h->H;
-    if (!H.p.use_graph) return MG_OK;
+    if (!H.p.use_graph || (H.p.outer == MG_OUTER_FGMRES ? H.g_fgiter : H.g_irstep)) return MG_OK;
+    const int ro = order_after(H, st);
+    if (ro) return ro;
     if (H.p.outer == MG_OUTER_FGMRES) {
-        if (H.g_fgiter) return MG_OK;
         // plain run of start / iteration / finish on the zeroed workspace
         h->eng->fg_start(H, H.g_stream);
         int rc = capture(H, &H.g_fgiter, [&](cudaStream_t s) { h->eng->fg_iter(H, s); });
@@ -860,7 +878,6 @@ static int ensure_graph(mg_handle* h) {
         if (e != cudaSuccess) { set_error(cudaGetErrorString(e)); return MG_ECUDA; }
         return rc;
     }
-    if (H.g_irstep) return MG_OK;
     return capture(H, &H.g_irstep, [&](cudaStream_t s) { h->eng->ir_step(H, s); });
 }
 
@@ -1251,9 +1268,9 @@ int mg_cycle(mg_handle* h, void* u, const void* g, int ncycles, mg_stream stream
 int mg_solve_begin(mg_handle* h, const void* u, const void* g, mg_stream stream) {
     if (!h || !u || !g) { set_error("mg_solve_begin: bad argument"); return MG_EINVAL; }
     Handle& H = h->H;
-    int rc = ensure_graph(h);
-    if (rc) return rc;
     cudaStream_t st = (cudaStream_t)stream;
+    int rc = ensure_graph(h, st);
+    if (rc) return rc;
     for (auto& I : H.inst) {
         LevelHost& l1 = I.lv[0];
         char* ov = (char*)I.outer_vec;
