@@ -690,10 +690,7 @@ struct Adjoint {
             return p;
         }
         double2* p = nullptr;
-        if (cudaMalloc(&p, sizeof(double2) * L.sz) != cudaSuccess) {
-            err = MG_ENOMEM;
-            return nullptr;
-        }
+        if (cudaMalloc(&p, sizeof(double2) * L.sz) != cudaSuccess) throw AllocError();
         cudaMemsetAsync(p, 0, sizeof(double2) * L.sz, st);
         all.push_back(p);
         L.owned.push_back(p);
@@ -1308,7 +1305,11 @@ extern "C" int mg_cycle_backward(mg_handle* h, const void* u0, const void* g, in
                                    cudaMemcpyDeviceToDevice, st));
     }
     for (int k = 1; k < K; ++k) {
-        h->eng->cycle(H, false, st);
+        const int rc = guarded("mg_cycle_backward", h, [&] {
+            h->eng->cycle(H, false, st);
+            return MG_OK;
+        });
+        if (rc) { cleanup(); return rc; }
         for (int b = 0; b < ni; ++b) {
             LevelHost& l1 = H.inst[b].lv[0];
             const char* sd = (const char*)l1.vec + (size_t)SD * l1.slot_stride * 16;
@@ -1365,15 +1366,19 @@ extern "C" int mg_cycle_backward(mg_handle* h, const void* u0, const void* g, in
         if (adj[b]->init()) rc = MG_ENOMEM;
     }
     // one reverse step of instance b from the checkpoint in B.uin
-    auto step = [&](int b) {
+    auto step = [&](int b) -> int {
         Adjoint& A = *adj[b];
         Bufs& B = bf[b];
         const size_t bytes = sizeof(double2) * H.inst[b].lv[0].slot_stride;
-        Adjoint::WaveTape* T = A.wave_forward(1, B.uin, B.gd, B.uout);
-        cudaMemsetAsync(B.ubin, 0, bytes, ss[b]);
-        A.wave_backward(T, B.ub, B.ubin, B.gbar);
-        cudaMemcpyAsync(B.ub, B.ubin, bytes, cudaMemcpyDeviceToDevice, ss[b]);
+        const int rs = guarded("mg_cycle_backward", h, [&] {
+            Adjoint::WaveTape* T = A.wave_forward(1, B.uin, B.gd, B.uout);
+            cudaMemsetAsync(B.ubin, 0, bytes, ss[b]);
+            A.wave_backward(T, B.ub, B.ubin, B.gbar);
+            cudaMemcpyAsync(B.ub, B.ubin, bytes, cudaMemcpyDeviceToDevice, ss[b]);
+            return MG_OK;
+        });
         A.reset();
+        return rs ? rs : A.err;
     };
     // first step of every instance (eager), then the captured step; below four
     // cycles the remaining steps run eagerly too (capturing and instantiating
@@ -1382,25 +1387,22 @@ extern "C" int mg_cycle_backward(mg_handle* h, const void* u0, const void* g, in
     for (int b = 0; b < ni && !rc; ++b) {
         const size_t bytes = sizeof(double2) * H.inst[b].lv[0].slot_stride;
         cudaMemcpyAsync(bf[b].uin, ck[b][K - 1], bytes, cudaMemcpyDeviceToDevice, ss[b]);
-        step(b);
-        if (adj[b]->err) rc = adj[b]->err;
+        rc = step(b);
     }
     for (int b = 0; b < ni && !rc && replay; ++b) {
         cudaGraph_t gr = nullptr;
         if (cudaStreamBeginCapture(ss[b], cudaStreamCaptureModeRelaxed) != cudaSuccess) { rc = MG_ECUDA; break; }
-        step(b);
-        if (cudaStreamEndCapture(ss[b], &gr) != cudaSuccess || !gr) { rc = MG_ECUDA; break; }
-        const cudaError_t ie = cudaGraphInstantiate(&gexec[b], gr, 0);
+        rc = step(b);
+        if (cudaStreamEndCapture(ss[b], &gr) != cudaSuccess || !gr) { rc = rc ? rc : MG_ECUDA; break; }
+        if (!rc && cudaGraphInstantiate(&gexec[b], gr, 0) != cudaSuccess) rc = MG_ECUDA;
         cudaGraphDestroy(gr);
-        if (ie != cudaSuccess || adj[b]->err) rc = adj[b]->err ? adj[b]->err : MG_ECUDA;
     }
     for (int k = K - 2; k >= 0 && !rc; --k)
         for (int b = 0; b < ni; ++b) {
             const size_t bytes = sizeof(double2) * H.inst[b].lv[0].slot_stride;
             cudaMemcpyAsync(bf[b].uin, ck[b][k], bytes, cudaMemcpyDeviceToDevice, ss[b]);
             if (!replay) {
-                step(b);
-                if (adj[b]->err) { rc = adj[b]->err; break; }
+                if ((rc = step(b)) != MG_OK) break;
             } else if (cudaGraphLaunch(gexec[b], ss[b]) != cudaSuccess) {
                 rc = MG_ECUDA;
                 break;

@@ -1011,6 +1011,11 @@ struct Engine : EngineBase {
             launch_prolong<PMODE_JAC>(H, ds1, KK_PROLONG_JAC, 3 * C + C / 4 + R, SU, SU, SG, SD, SD, 0, st);
     }
 
+    void abandon(Handle& H) override {
+        fg_want = fg_gvec = fg_fused = false;
+        H.cur_var = 0;
+        H.prof = 0;
+    }
     void user_in(Handle& H, const void* u, const void* g, cudaStream_t st) override {
         const SegTable& t = H.seg(descs(H, 1, all(H)), false, kPts);
         kl(k_user_in<T>, t.nblocks, dim3(BX, BY), 0, st, kd(H, t), t.d, t.nseg, (const cplx<T>*)u, (const cplx<T>*)g);

@@ -4,6 +4,7 @@
 
 #include <map>
 #include <memory>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -78,6 +79,10 @@ struct TileChoice {
     int gram = -1, pre = -1;   // -1: default shape
 };
 
+// A device allocation of a handle failed (Handle::alloc); every C entry that
+// allocates or launches turns it into its status (guarded).
+struct AllocError {};
+
 std::string desc_key(const std::vector<int>& descs);
 // Blocks per segment of a launch: every segment at least one, the rest of
 // the cap given greedily to the segment with the most work units per block.
@@ -108,7 +113,7 @@ struct Handle {
     int roles[MAX_LEVELS] = {};                // effective role of level l (l >= 2, below an instance's coarsest)
     std::vector<void*> allocs;      // everything cudaMalloc'ed
     size_t alloc_bytes = 0;         // their total size
-    long long alloc_limit = 0;      // mg_params.workspace_limit (0: none)
+    long long alloc_limit = 0;      // during mg_setup: mg_params.workspace_limit (0: none)
     long long total_elems = 0;      // sum of n ny over instances
     // graphs
     cudaGraphExec_t g_cycle = nullptr;      // mg_cycle's cycle (level-1 SX2, SG -> SD)
@@ -136,6 +141,7 @@ struct Handle {
     unsigned* herr = nullptr;               // pinned copy of the device error word
     std::string last_error;
 
+    // device memory owned by the handle; throws AllocError (never null)
     void* alloc(size_t bytes);
     const SegTable& seg(const std::vector<int>& descs, bool outer, int pts_per_block);
     const SegTable& seg_rows(const std::vector<int>& descs, int rows_per_block);
@@ -168,6 +174,8 @@ struct EngineBase {
     virtual int level_op(Handle& H, int inst, int level, int what, int a0, int a1, cudaStream_t st) = 0;
     // halo-tile autotuner of the ADR launches (fills Handle::tiles)
     virtual int autotune(Handle& H, cudaStream_t st) = 0;
+    // undo what an emission that ended in an exception left set
+    virtual void abandon(Handle& H) = 0;
 };
 
 EngineBase* make_engine_f32();
@@ -222,3 +230,21 @@ struct mg_handle {
     wadr::Handle H;
     wadr::EngineBase* eng = nullptr;
 };
+
+namespace wadr {
+// f() of a C entry `where`; an allocation that failed on the way becomes
+// MG_ENOMEM (launch tables are built on first use, so any launching call can
+// meet one).
+template <class F> int guarded(const char* where, mg_handle* h, F&& f) {
+    try {
+        return f();
+    } catch (const AllocError&) {
+        set_error(std::string(where) + ": out of device memory");
+    } catch (const std::bad_alloc&) {
+        set_error(std::string(where) + ": out of host memory");
+    }
+    cudaGetLastError();
+    if (h && h->eng) h->eng->abandon(h->H);
+    return MG_ENOMEM;
+}
+}  // namespace wadr

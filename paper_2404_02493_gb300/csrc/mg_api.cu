@@ -50,8 +50,8 @@ void prof_end(Handle& H, cudaStream_t st, int kind, double bytes, long long pts)
 void* Handle::alloc(size_t bytes) {
     void* p = nullptr;
     if (bytes == 0) bytes = 16;
-    if (alloc_limit > 0 && alloc_bytes + bytes > (size_t)alloc_limit) return nullptr;
-    if (cudaMalloc(&p, bytes) != cudaSuccess) return nullptr;
+    if (alloc_limit > 0 && alloc_bytes + bytes > (size_t)alloc_limit) throw AllocError();
+    if (cudaMalloc(&p, bytes) != cudaSuccess) throw AllocError();
     allocs.push_back(p);
     alloc_bytes += bytes;
     return p;
@@ -489,7 +489,6 @@ static int build(mg_handle* mh, const mg_instance* in, int ninst, cudaStream_t s
                 lv.inv_helm = H.alloc(N * N * esz(prec));
                 if (adr) lv.inv_adr = H.alloc(N * N * esz(prec));
             }
-            if (!lv.vec || !lv.kf || !lv.k64 || !lv.phi64) { set_error("mg_setup: out of device memory"); return MG_ENOMEM; }
             cudaMemsetAsync(lv.vec, 0, npt * lv.nslot * esz(prec), st);
         }
         if (adr && p.ray) {
@@ -516,28 +515,21 @@ static int build(mg_handle* mh, const mg_instance* in, int ninst, cudaStream_t s
                     if (l == 2) v.mod = H.alloc(npt * esz(prec));
                     if (l == I.L)
                         v.inv_adr = H.alloc((size_t)v.n * v.ny * v.n * v.ny * esz(prec));
-                    if (!v.phi64 || !v.adr || (l == 2 && !v.mod) || (l == I.L && !v.inv_adr)) {
-                        set_error("mg_setup: out of device memory (Wave-Ray levels)");
-                        return MG_ENOMEM;
-                    }
                 }
         }
         const size_t npt1 = I.lv[0].slot_stride;
         I.outer_stride = npt1;
         I.outer_vec = H.alloc(npt1 * 4 * 16);
-        if (!I.outer_vec) { set_error("mg_setup: out of device memory"); return MG_ENOMEM; }
         cudaMemsetAsync(I.outer_vec, 0, npt1 * 4 * 16, st);
         if (p.outer == MG_OUTER_FGMRES) {
             const size_t nk = (size_t)(2 * p.restart + 1) * npt1 * esz(prec);
             I.kv = H.alloc(nk);
-            if (!I.kv) { set_error("mg_setup: out of device memory (Krylov vectors)"); return MG_ENOMEM; }
             cudaMemsetAsync(I.kv, 0, nk, st);
         }
     }
     H.total_elems = off;
     // --- input validation: k finite and positive, phi finite
     double* vscr = (double*)H.alloc(64);
-    if (!vscr) { set_error("mg_setup: out of device memory"); return MG_ENOMEM; }
     for (int b = 0; b < ninst; ++b) {
         long long bad_k = 0, bad_phi = 0;
         int rc = setup_check_fields(in[b].k, in[b].phi, H.inst[b].n, H.inst[b].ny, vscr, &bad_k, &bad_phi, st);
@@ -582,7 +574,6 @@ static int build(mg_handle* mh, const mg_instance* in, int ninst, cudaStream_t s
     H.scal = (double*)H.alloc(sizeof(double) * S::SIZE * nslots);
     H.part = (double2*)H.alloc(sizeof(double2) * (size_t)MAXB * MAXDOT * nslots);
     H.counter = (unsigned*)H.alloc(sizeof(unsigned) * NCOUNTERS * nslots);
-    if (!H.scal || !H.part || !H.counter) { set_error("mg_setup: out of device memory"); return MG_ENOMEM; }
     cudaMemsetAsync(H.counter, 0, sizeof(unsigned) * NCOUNTERS * nslots, st);
     std::vector<double> hs((size_t)S::SIZE * nslots, 0.0);
     double* dscr = (double*)H.alloc(64);
@@ -712,7 +703,6 @@ static int build(mg_handle* mh, const mg_instance* in, int ninst, cudaStream_t s
         H.fs = (double*)H.alloc(sizeof(double) * FS::SIZE * ninst);
         H.fpart = (double2*)H.alloc(sizeof(double2) * (size_t)MAXB * NVL * ninst);
         H.est = (double*)H.alloc(sizeof(double) * ninst);
-        if (!H.fs || !H.fpart || !H.est) { set_error("mg_setup: out of device memory"); return MG_ENOMEM; }
         cudaMemsetAsync(H.fs, 0, sizeof(double) * FS::SIZE * ninst, st);
     }
     for (int b = 0; b < ninst; ++b) {
@@ -758,7 +748,6 @@ static int build(mg_handle* mh, const mg_instance* in, int ninst, cudaStream_t s
         memset(maps.data(), 0, maps.size() * sizeof(CUtensorMap));
         H.tmaps = H.alloc(maps.size() * sizeof(CUtensorMap));
         H.err = (unsigned*)H.alloc(sizeof(unsigned));
-        if (!H.tmaps || !H.err) { set_error("mg_setup: out of device memory"); return MG_ENOMEM; }
         cudaMemsetAsync(H.err, 0, sizeof(unsigned), st);
         for (size_t q = 0; q < nd2; ++q) {
             LevelDesc& d = H.hdesc[q];
@@ -809,7 +798,12 @@ static int capture(Handle& H, cudaGraphExec_t* out, F emit, bool built = false) 
     cudaGraph_t g;
     e = cudaStreamBeginCapture(H.g_stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) { set_error(cudaGetErrorString(e)); return MG_ECUDA; }
-    emit(H.g_stream);
+    try {
+        emit(H.g_stream);
+    } catch (...) {
+        if (cudaStreamEndCapture(H.g_stream, &g) == cudaSuccess && g) cudaGraphDestroy(g);
+        throw;
+    }
     e = cudaStreamEndCapture(H.g_stream, &g);
     if (e != cudaSuccess) { set_error(cudaGetErrorString(e)); return MG_ECUDA; }
     e = cudaGraphInstantiate(out, g, 0);
@@ -1052,8 +1046,11 @@ int mg_setup(mg_handle** out, const mg_instance* inst, int ninst, const mg_param
             (f ? staged[b].phi : staged[b].k) = (const double*)d;
         }
     }
-    int rc = build(mh, staged.data(), ninst, st0);
-    if (!rc) rc = mh->eng->autotune(mh->H, st0);
+    int rc = guarded("mg_setup", mh, [&] {
+        const int r = build(mh, staged.data(), ninst, st0);
+        return r ? r : mh->eng->autotune(mh->H, st0);
+    });
+    mh->H.alloc_limit = 0;   // (launch tables of later calls are not held against it)
     cudaStreamSynchronize(st0);
     for (void* q : tmp) cudaFree(q);
     if (rc) {
@@ -1206,7 +1203,7 @@ static bool kernel_ptr(const void* p, size_t es) {
     return ok && (uintptr_t)p % es == 0;
 }
 
-int mg_cycle(mg_handle* h, void* u, const void* g, int ncycles, mg_stream stream) {
+static int cycle_call(mg_handle* h, void* u, const void* g, int ncycles, mg_stream stream) {
     if (!h || !u || !g || ncycles < 0) { set_error("mg_cycle: bad argument"); return MG_EINVAL; }
     Handle& H = h->H;
     cudaStream_t st = (cudaStream_t)stream;
@@ -1264,8 +1261,11 @@ int mg_cycle(mg_handle* h, void* u, const void* g, int ncycles, mg_stream stream
     if (is_host_ptr(u)) return check_device_error(H, st);   // synchronises: host result complete on return
     return MG_OK;
 }
+int mg_cycle(mg_handle* h, void* u, const void* g, int ncycles, mg_stream stream) {
+    return guarded("mg_cycle", h, [&] { return cycle_call(h, u, g, ncycles, stream); });
+}
 
-int mg_solve_begin(mg_handle* h, const void* u, const void* g, mg_stream stream) {
+static int solve_begin_call(mg_handle* h, const void* u, const void* g, mg_stream stream) {
     if (!h || !u || !g) { set_error("mg_solve_begin: bad argument"); return MG_EINVAL; }
     Handle& H = h->H;
     cudaStream_t st = (cudaStream_t)stream;
@@ -1283,8 +1283,11 @@ int mg_solve_begin(mg_handle* h, const void* u, const void* g, mg_stream stream)
     H.solve_ready = true;
     return MG_OK;
 }
+int mg_solve_begin(mg_handle* h, const void* u, const void* g, mg_stream stream) {
+    return guarded("mg_solve_begin", h, [&] { return solve_begin_call(h, u, g, stream); });
+}
 
-int mg_solve_steps(mg_handle* h, int nsteps, mg_stream stream) {
+static int solve_steps_call(mg_handle* h, int nsteps, mg_stream stream) {
     if (!h || nsteps < 0) { set_error("mg_solve_steps: bad argument"); return MG_EINVAL; }
     Handle& H = h->H;
     if (!H.solve_ready) { set_error("mg_solve_steps: call mg_solve_begin first"); return MG_EINVAL; }
@@ -1306,8 +1309,11 @@ int mg_solve_steps(mg_handle* h, int nsteps, mg_stream stream) {
     WADR_CHECK(cudaGetLastError());
     return MG_OK;
 }
+int mg_solve_steps(mg_handle* h, int nsteps, mg_stream stream) {
+    return guarded("mg_solve_steps", h, [&] { return solve_steps_call(h, nsteps, stream); });
+}
 
-int mg_solve_end(mg_handle* h, void* u, double* rel_residual, mg_stream stream) {
+static int solve_end_call(mg_handle* h, void* u, double* rel_residual, mg_stream stream) {
     if (!h) { set_error("mg_solve_end: bad argument"); return MG_EINVAL; }
     Handle& H = h->H;
     if (!H.solve_ready) { set_error("mg_solve_end: call mg_solve_begin first"); return MG_EINVAL; }
@@ -1331,8 +1337,11 @@ int mg_solve_end(mg_handle* h, void* u, double* rel_residual, mg_stream stream) 
     if (rel_residual) *rel_residual = max_rel(rn, gn);
     return MG_OK;
 }
+int mg_solve_end(mg_handle* h, void* u, double* rel_residual, mg_stream stream) {
+    return guarded("mg_solve_end", h, [&] { return solve_end_call(h, u, rel_residual, stream); });
+}
 
-int mg_solve(mg_handle* h, void* u, const void* g, mg_solve_info* info, mg_stream stream) {
+static int solve_call(mg_handle* h, void* u, const void* g, mg_solve_info* info, mg_stream stream) {
     if (!h || !u || !g) { set_error("mg_solve: bad argument"); return MG_EINVAL; }
     Handle& H = h->H;
     cudaStream_t st = (cudaStream_t)stream;
@@ -1428,13 +1437,16 @@ int mg_solve(mg_handle* h, void* u, const void* g, mg_solve_info* info, mg_strea
     }
     return status;
 }
+int mg_solve(mg_handle* h, void* u, const void* g, mg_solve_info* info, mg_stream stream) {
+    return guarded("mg_solve", h, [&] { return solve_call(h, u, g, info, stream); });
+}
 
 int mg_step_launches(const mg_handle* h) { return h ? h->H.launches_step : MG_EINVAL; }
 
 const char* mg_kernel_name(int kind) { return kernel_kind_name(kind); }
 
-int mg_profile_records(mg_handle* h, int nsteps, int* kind, long long* pts, double* ms, double* bytes,
-                       int* launches, int maxrec, mg_stream stream) {
+static int profile_records_call(mg_handle* h, int nsteps, int* kind, long long* pts, double* ms, double* bytes,
+                                int* launches, int maxrec, mg_stream stream) {
     if (!h || nsteps < 1 || !kind || !pts || !ms || !bytes || !launches || maxrec < 1) {
         set_error("mg_profile_records: bad argument");
         return MG_EINVAL;
@@ -1480,9 +1492,15 @@ int mg_profile_records(mg_handle* h, int nsteps, int* kind, long long* pts, doub
     }
     return nrec;
 }
+int mg_profile_records(mg_handle* h, int nsteps, int* kind, long long* pts, double* ms, double* bytes,
+                       int* launches, int maxrec, mg_stream stream) {
+    return guarded("mg_profile_records", h, [&] {
+        return profile_records_call(h, nsteps, kind, pts, ms, bytes, launches, maxrec, stream);
+    });
+}
 
-int mg_profile_steps(mg_handle* h, int nsteps, double* ms, double* bytes, int* launches, int nkinds,
-                     mg_stream stream) {
+static int profile_steps_call(mg_handle* h, int nsteps, double* ms, double* bytes, int* launches, int nkinds,
+                              mg_stream stream) {
     if (!h || nsteps < 1 || !ms || !bytes || !launches || nkinds < KK_COUNT) {
         set_error("mg_profile_steps: bad argument");
         return MG_EINVAL;
@@ -1519,6 +1537,12 @@ int mg_profile_steps(mg_handle* h, int nsteps, double* ms, double* bytes, int* l
     }
     return MG_OK;
 }
+int mg_profile_steps(mg_handle* h, int nsteps, double* ms, double* bytes, int* launches, int nkinds,
+                     mg_stream stream) {
+    return guarded("mg_profile_steps", h, [&] {
+        return profile_steps_call(h, nsteps, ms, bytes, launches, nkinds, stream);
+    });
+}
 
 // ------------------------------------------------------------ level ops
 static int check_level(mg_handle* h, int inst, int level) {
@@ -1539,7 +1563,12 @@ static int run_op(mg_handle* h, int inst, int level, int what, int a0, int a1,
         LevelHost& lv = I.lv[lvl - 1];
         WADR_CHECK(copy_in(pr.second, 0, es, slot_ptr(H, lv, s), lv.n, lv.ny, lv.pitch, st));
     }
-    int s = h->eng->level_op(H, inst, level, what, a0, a1, st);
+    int s = -1;
+    const int rc = guarded("level operation", h, [&] {
+        s = h->eng->level_op(H, inst, level, what, a0, a1, st);
+        return MG_OK;
+    });
+    if (rc) return rc;
     WADR_CHECK(cudaGetLastError());
     if (s < 0) { set_error("level op failed"); return MG_EINVAL; }
     if (out_slot_override >= 0) s = out_slot_override;
