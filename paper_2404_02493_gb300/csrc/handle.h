@@ -117,7 +117,8 @@ struct Handle {
     long long total_elems = 0;      // sum of n ny over instances
     // graphs
     cudaGraphExec_t g_cycle = nullptr;      // mg_cycle's cycle (level-1 SX2, SG -> SD)
-    int cycle_calls = 0;                    // device-array calls of mg_cycle (the second captures g_cycle)
+    int cycle_calls = 0;                    // mg_cycle on device arrays: 0 not called yet, 1 called (the next call
+                                            // captures g_cycle), -1 the capture failed
     cudaGraphExec_t g_irstep = nullptr;     // scale + cycle + update + residual
     cudaStream_t g_stream = nullptr;
     int launches_cycle = 0;                 // kernels of the last emitted cycle

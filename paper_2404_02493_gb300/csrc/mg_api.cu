@@ -1223,13 +1223,16 @@ static int cycle_call(mg_handle* h, void* u, const void* g, int ncycles, mg_stre
         // which every call from then on replays: a cycle is 30 to 250 small
         // launches, and the host took ~6.5 us to emit each of them (n = 127,
         // M = 2: 225 us per call, host-bound).  A stream that is being
-        // captured itself takes the plain launches.
+        // captured itself takes the plain launches, and so does a handle
+        // whose cycle could not be captured, for good.
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         WADR_CHECK(cudaStreamIsCapturing(st, &cap));
         const bool plain = !H.p.use_graph || cap != cudaStreamCaptureStatusNone;
-        if (!plain && !H.g_cycle && H.cycle_calls > 0) {
-            const int rc = capture(H, &H.g_cycle, [&](cudaStream_t s) { h->eng->cycle(H, false, s); }, true);
-            if (rc) return rc;
+        if (!plain && !H.g_cycle && H.cycle_calls > 0 &&
+            capture(H, &H.g_cycle, [&](cudaStream_t s) { h->eng->cycle(H, false, s); }, true) != MG_OK) {
+            H.g_cycle = nullptr;
+            H.cycle_calls = -1;
+            cudaGetLastError();
         }
         h->eng->user_in(H, u, g, st);
         for (int c = 0; c < ncycles; ++c) {
@@ -1240,7 +1243,7 @@ static int cycle_call(mg_handle* h, void* u, const void* g, int ncycles, mg_stre
         }
         h->eng->user_out(H, u, st);
         WADR_CHECK(cudaGetLastError());
-        H.cycle_calls = 1;
+        if (H.cycle_calls == 0) H.cycle_calls = 1;
         return MG_OK;
     }
     for (auto& I : H.inst) {

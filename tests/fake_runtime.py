@@ -30,6 +30,28 @@ int cudaMalloc(void** p, size_t n) {
     if (no) { ++fake_mallocs_refused; return 2; }
     return f(p, n);
 }
+/* fake_capture: 1 cudaStreamBeginCapture fails, 2 cudaStreamEndCapture reports
+   an invalidated capture (which has ended), 3 cudaGraphInstantiate fails */
+int fake_capture = 0, fake_captures_refused = 0;
+int cudaStreamBeginCapture(void* st, int mode) {
+    static int (*f)(void*, int);
+    if (!f) f = (int (*)(void*, int))real("cudaStreamBeginCapture");
+    if (fake_capture == 1) { ++fake_captures_refused; return 900; }
+    return f(st, mode);
+}
+int cudaStreamEndCapture(void* st, void** g) {
+    static int (*f)(void*, void**);
+    if (!f) f = (int (*)(void*, void**))real("cudaStreamEndCapture");
+    const int e = f(st, g);
+    if (fake_capture == 2) { ++fake_captures_refused; *g = NULL; return 901; }
+    return e;
+}
+int cudaGraphInstantiate(void** x, void* g, unsigned long long flags) {
+    static int (*f)(void**, void*, unsigned long long);
+    if (!f) f = (int (*)(void**, void*, unsigned long long))real("cudaGraphInstantiate");
+    if (fake_capture == 3) { ++fake_captures_refused; return 2; }
+    return f(x, g, flags);
+}
 """
 
 
