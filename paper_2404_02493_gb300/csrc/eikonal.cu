@@ -173,7 +173,18 @@ __global__ void __launch_bounds__(32) k_eik_pass(int n, int ny, double h, const 
         const unsigned updr = __shfl_sync(0xffffffffu, upd, ET - 1 - lane);   // of column 31 - lane
         __syncwarp();
         // FAST: no negative value in the tile, every f between 1e-140 and 1e140
-        // (by their bits)
+        // (by their bits).  big_hi, f_hi: upper words of the largest finite
+        // value and of the largest f.
+        int big_hi = 0, f_hi = 0;
+        const int inf_hi = __double2hiint(EINF);
+        auto top = [&](double v) {
+            const int b = __double2hiint(v);
+            if (b < inf_hi) big_hi = max(big_hi, b);
+        };
+        top(T[0][lane + 1]);
+        top(T[ET + 1][lane + 1]);
+        top(T[lane + 1][0]);
+        top(T[lane + 1][ET + 1]);
         const long long fl = __double_as_longlong(1e-140), fh = __double_as_longlong(1e140);
         long long neg = __double_as_longlong(T[0][lane + 1]) | __double_as_longlong(T[ET + 1][lane + 1]) |
                         __double_as_longlong(T[lane + 1][0]) | __double_as_longlong(T[lane + 1][ET + 1]);
@@ -182,9 +193,16 @@ __global__ void __launch_bounds__(32) k_eik_pass(int n, int ny, double h, const 
         for (int r = 0; r < ET; ++r) {
             const long long f = __double_as_longlong(Fs[r][lane]);
             neg |= __double_as_longlong(T[r + 1][lane + 1]);
+            top(T[r + 1][lane + 1]);
+            f_hi = max(f_hi, __double2hiint(Fs[r][lane]));
             fast = fast && (!((upd >> r) & 1) || (f > fl && f < fh));
         }
         fast = __all_sync(0xffffffffu, fast && neg >= 0);
+        // tol covers two units in the last place of every value this visit
+        // can form (at most the largest finite one and f at every node)
+        const double most = __hiloint2double(__reduce_max_sync(0xffffffffu, big_hi) + 1, 0) +
+                            ET * ET * __hiloint2double(__reduce_max_sync(0xffffffffu, f_hi) + 1, 0);
+        const bool ulps = tol >= 4.5e-16 * most;
         unsigned left;
         auto visit = [&](auto fc) -> bool {
             constexpr bool FAST = decltype(fc)::value;
@@ -193,7 +211,9 @@ __global__ void __launch_bounds__(32) k_eik_pass(int n, int ny, double h, const 
             // north): vote[q] has bit j for row j of the lane's column.  A
             // decrease that rounding alone can make (two units in the last
             // place) does not vote unless it exceeds tol; one above tol makes
-            // the tile a changed one (big, looked for until it is known).
+            // the tile a changed one (big, looked for until it is known; from
+            // then on two units are compared as integers where tol covers
+            // them, ulps).
             unsigned vote[4] = {0, 0, 0, 0};
             bool big = false, known = false;
             // ordering (0..3) of node (i, j)'s vote, or -1
@@ -215,7 +235,7 @@ __global__ void __launch_bounds__(32) k_eik_pass(int n, int ny, double h, const 
                 return yes ? (fe ? 1 : 0) + (fn ? 2 : 0) : -1;
             };
             auto look_all = [&]() {
-                if (tol < 1e-15) known = false;   // every decrease above tol votes
+                known = known && ulps;   // every decrease above tol votes
 #pragma unroll 8
                 for (int r = 0; r < ET; ++r) {
                     const int o = look(lane, r, (upd >> r) & 1);
