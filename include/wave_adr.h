@@ -145,7 +145,11 @@ typedef struct mg_params {
                                ADR corrections then amplify the residual on large grids */
     long long workspace_limit; /* 0 (default): none; > 0: mg_setup fails with MG_ENOMEM, freeing what it
                                had allocated, when the handle's device workspace would exceed this many bytes
-                               (for callers that share the GPU; mg_workspace_bytes reports the size) */
+                               (for callers that share the GPU; mg_workspace_bytes reports the size).  Not
+                               counted: launch tables that later calls build (some KB), and what mg_setup
+                               itself holds until it returns, a copy of host k and phi and, while the coarsest
+                               inverses are formed, their matrices (up to 256 MB, or the two of one operator,
+                               32 bytes per node pair, where that much is not free) */
     int roles[MG_MAX_LEVELS]; /* roles[l-1]: role of level l (MG_ROLE_*, declared below).  -1 (default): the
                                role by index of Algorithm 1 (Jacobi on level 1, Chebyshev with the ADR
                                corrections on level 2, nothing on level 3, Chebyshev below).  Levels 2..L-1

@@ -414,12 +414,12 @@ __global__ void k_gj_store(const GjMat* __restrict__ M) {
 }
 
 // The inverses of all jobs (always eliminated in FP64; see CoarseJob).  The
-// temporary matrices of one group of jobs stay below 256 MB (or one job).
+// temporary matrices of one group of jobs stay below 256 MB (or one job), and
+// where the memory for a group is not there, below half of what was asked.
 // Two 225 x 225 inverses: 39.2 ms one block per matrix -> 1.8 ms (29 panels of 49 us, 29 updates of 13 us).
 int setup_coarse_inverses(const std::vector<CoarseJob>& jobs, cudaStream_t st) {
     static_assert(GJX * GJB == 256 && GJX * 8 == 256 && GJY * GJB <= 256, "update tile");
-    constexpr size_t GROUP = 256u << 20;
-    size_t q0 = 0;
+    size_t group = 256u << 20, q0 = 0;
     while (q0 < jobs.size()) {
         size_t q1 = q0, bytes = 0;
         int nmax = 0;
@@ -427,7 +427,7 @@ int setup_coarse_inverses(const std::vector<CoarseJob>& jobs, cudaStream_t st) {
         while (q1 < jobs.size()) {
             const size_t N = (size_t)jobs[q1].n * jobs[q1].ny;
             const size_t need = (2 * N * N + N * GJB) * sizeof(double2) + (2 * N * sizeof(int) + 255) / 256 * 256;
-            if (q1 > q0 && (bytes + need > GROUP || q1 - q0 >= 32768)) break;   // (a grid slice per job)
+            if (q1 > q0 && (bytes + need > group || q1 - q0 >= 32768)) break;   // (a grid slice per job)
             at.push_back(bytes);
             bytes += need;
             nmax = std::max(nmax, (int)N);
@@ -438,6 +438,11 @@ int setup_coarse_inverses(const std::vector<CoarseJob>& jobs, cudaStream_t st) {
         unsigned char* base = nullptr;
         if (cudaMalloc(&base, mats + bytes) != cudaSuccess) {
             cudaGetLastError();
+            if (nj > 1) {
+                group = bytes / 2;
+                continue;
+            }
+            set_error("mg_setup: out of device memory (coarsest-level inverse)");
             return MG_ENOMEM;
         }
         std::vector<GjMat> hm(nj);
