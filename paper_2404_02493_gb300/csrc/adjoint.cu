@@ -643,14 +643,8 @@ struct Adjoint {
 
     int blocks(const AdjLevel& L) const { return (int)(((long long)L.n * L.ny + ANT - 1) / ANT); }
     static int num_sms() {
-        static int nsm = 0;
-        if (!nsm) {
-            int dev = 0;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-            if (nsm < 1) nsm = 1;
-        }
-        return nsm;
+        static PerDevice<int> n;
+        return (int)n.get(0, sm_count);
     }
 
     int init() {

@@ -83,20 +83,21 @@ struct Engine : EngineBase {
     }, (t).pts)
 
     // Dynamic shared memory opt-in and resident blocks per SM x SM count of a
-    // tile kernel (cached per kernel): the block count of its launches, so
-    // that one wave of blocks loops over the tiles (double-buffered).
+    // tile kernel (found once per device and kernel): the block count of its
+    // launches, so that one wave of blocks loops over the tiles
+    // (double-buffered).
     template <class K>
     static int occ_cap(K kern, int smem, int threads = NT) {
-        static std::map<const void*, int> caps;
-        auto it = caps.find((const void*)kern);
-        if (it != caps.end()) return it->second;
+        static PerDevice<const void*> caps;
+        return (int)caps.get((const void*)kern, [&](int dev) { return resident(kern, smem, threads, dev); });
+    }
+    template <class K>
+    static int resident(K kern, int smem, int threads, int dev) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-        int nb = 0, dev = 0, nsm = 0;
+        int nb = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, threads, smem);
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        return caps[(const void*)kern] = std::max(1, nb) * std::max(1, nsm);
+        return std::max(1, nb) * sm_count(dev);
     }
     void launch_cheb(Handle& H, const std::vector<int>& ds, double bpp, int sin, int sout, int m, int flags,
                      cudaStream_t st) {
@@ -170,26 +171,20 @@ struct Engine : EngineBase {
         }
     }
     // Resident blocks x SM count of a kernel at a given dynamic shared
-    // memory size (cached per pair; the kernel's opt-in limit is raised to
-    // the largest size seen).
+    // memory size, its opt-in limit at the most a block may have.
     template <class K>
     static int occ_cap_at(K kern, int smem) {
-        static std::map<std::pair<const void*, int>, int> caps;
-        static std::map<const void*, int> optin;
-        const auto key = std::make_pair((const void*)kern, smem);
-        auto it = caps.find(key);
-        if (it != caps.end()) return it->second;
-        int& o = optin[(const void*)kern];
-        if (smem > o) {
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        static PerDevice<std::pair<const void*, int>> caps;
+        return (int)caps.get(std::make_pair((const void*)kern, smem), [&](int dev) {
+            cudaFuncAttributes a = {};
+            cudaFuncGetAttributes(&a, kern);
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 smem_optin(dev) - (int)a.sharedSizeBytes);
             cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-            o = smem;
-        }
-        int nb = 0, dev = 0, nsm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, NT, smem);
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        return caps[key] = std::max(1, nb) * std::max(1, nsm);
+            int nb = 0;
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, NT, smem);
+            return std::max(1, nb) * sm_count(dev);
+        });
     }
     // Output tile side of the one-launch smoothing (k_cheb_multi) for q steps
     // on level l, or 0 where it does not apply: FP32 levels >= 2 that do not
@@ -197,12 +192,8 @@ struct Engine : EngineBase {
     // largest side that still gives 128 tiles over the launch's instances.
     static int cheb_multi_ts(Handle& H, const std::vector<int>& ds, int l, int q) {
         if (!kStream || l < 2 || q < 2 || cheb_stream_on(H, ds, l)) return 0;
-        static int optin = -1;
-        if (optin < 0) {
-            int dev = 0;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        }
+        static PerDevice<int> limit;
+        const int optin = (int)limit.get(0, smem_optin);
         for (int ts : {32, 16, 8}) {
             if (cm_smem<T>(ts, q) > optin - 1024) continue;
             long long tiles = 0;
@@ -489,23 +480,11 @@ struct Engine : EngineBase {
     // Per (kernel, candidate): dynamic shared memory opt-in and the resident
     // blocks per SM, so that a launch has at most one wave of persistent
     // blocks per segment (blocks loop over tiles).
-    static int& gs_cap_slot(int which, int cand) {
-        static int cap[3][GS_NCAND] = {};
-        return cap[which][cand];
-    }
     template <class K>
     static int gs_prepare(K kern, int smem, int which, int cand, int threads) {
-        int& cap = gs_cap_slot(which, cand);
-        if (cap == 0) {
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-            cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-            int nb = 0, dev = 0, nsm = 0;
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, threads, smem);
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-            cap = std::max(1, nb) * std::max(1, nsm);
-        }
-        return cap;
+        static PerDevice<std::pair<int, int>> caps;
+        return (int)caps.get(std::make_pair(which, cand),
+                             [&](int dev) { return resident(kern, smem, threads, dev); });
     }
     template <class F>
     static void gs_dispatch(int cand, F&& f) {
@@ -689,25 +668,22 @@ struct Engine : EngineBase {
         cfg.numAttrs = pdl_on() ? 2 : 1;
     }
     static long long ct_smem_limit() {
-        static const long long lim = [] {
-            int dev = 0, optin = 0;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        static PerDevice<int> lim;
+        return lim.get(0, [](int dev) {
             cudaFuncAttributes a = {}, b = {};
             cudaFuncGetAttributes(&a, k_adr_cluster<T, 16>);
             cudaFuncGetAttributes(&b, k_adr_cluster<T, 8>);
-            return std::max(0LL, (long long)optin - (long long)std::max(a.sharedSizeBytes, b.sharedSizeBytes));
-        }();
-        return lim;
+            return std::max(0LL, (long long)smem_optin(dev) - (long long)std::max(a.sharedSizeBytes, b.sharedSizeBytes));
+        });
     }
     static int ct_cluster() {
-        static const int cs = [] {
+        static PerDevice<int> cs;
+        return (int)cs.get(0, [](int) {
             int c = ct_try<16>(ct_smem_limit());
             if (!c) c = ct_try<8>(ct_smem_limit());
             cudaGetLastError();
             return c;
-        }();
-        return cs;
+        });
     }
     // Levels l .. L of instance b fit one cluster (whole: with the iterate of
     // the ADR corrections).
@@ -763,20 +739,18 @@ struct Engine : EngineBase {
     // Shared-memory tail of the wave cycle (tail_wave.cuh): opt-in dynamic
     // shared memory of its two kernels, set once.
     static long long wt_smem_limit() {
-        static long long lim = -1;
-        if (lim >= 0) return lim;
-        int dev = 0, optin = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        cudaFuncAttributes a1 = {}, a2 = {};
-        cudaFuncGetAttributes(&a1, k_wave_down<T>);
-        cudaFuncGetAttributes(&a2, k_wave_up<T>);
-        lim = (long long)optin - (long long)std::max(a1.sharedSizeBytes, a2.sharedSizeBytes) - 256;
-        if (lim < 0) lim = 0;
-        cudaFuncSetAttribute(k_wave_down<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim);
-        cudaFuncSetAttribute(k_wave_up<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim);
-        cudaGetLastError();
-        return lim;
+        static PerDevice<int> limit;
+        return limit.get(0, [](int dev) {
+            cudaFuncAttributes a1 = {}, a2 = {};
+            cudaFuncGetAttributes(&a1, k_wave_down<T>);
+            cudaFuncGetAttributes(&a2, k_wave_up<T>);
+            const long long lim = std::max(
+                0LL, (long long)smem_optin(dev) - (long long)std::max(a1.sharedSizeBytes, a2.sharedSizeBytes) - 256);
+            cudaFuncSetAttribute(k_wave_down<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim);
+            cudaFuncSetAttribute(k_wave_up<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim);
+            cudaGetLastError();
+            return lim;
+        });
     }
     // Level l (smoothed, l >= 4, not the coarsest) of instance b starts the
     // wave tail: n_l within the bound and its vectors fit one block.

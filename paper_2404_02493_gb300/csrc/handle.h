@@ -4,8 +4,10 @@
 
 #include <map>
 #include <memory>
+#include <mutex>
 #include <new>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "common.cuh"
@@ -78,6 +80,35 @@ const char* kernel_kind_name(int k);
 struct TileChoice {
     int gram = -1, pre = -1;   // -1: default shape
 };
+
+// Values that belong to a device, found once for each device that is current
+// when they are asked for: kernel attributes (an opt-in to more shared memory or
+// to larger clusters holds on one device only), limits, resident blocks.
+// Handles of several threads share them.
+template <class K> class PerDevice {
+    std::mutex m;
+    std::map<std::pair<int, K>, long long> v;
+
+public:
+    template <class F> long long get(const K& key, F&& f) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        std::lock_guard<std::mutex> l(m);
+        const auto k = std::make_pair(dev, key);
+        const auto it = v.find(k);
+        return it != v.end() ? it->second : (v[k] = (long long)f(dev));
+    }
+};
+inline int sm_count(int dev) {
+    int n = 0;
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return n > 1 ? n : 1;
+}
+inline int smem_optin(int dev) {
+    int n = 0;
+    cudaDeviceGetAttribute(&n, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    return n;
+}
 
 // A device allocation of a handle failed (Handle::alloc); every C entry that
 // allocates or launches turns it into its status (guarded).

@@ -52,6 +52,28 @@ int cudaGraphInstantiate(void** x, void* g, unsigned long long flags) {
     if (fake_capture == 3) { ++fake_captures_refused; return 2; }
     return f(x, g, flags);
 }
+/* fake_device >= 0: the number that cudaGetDevice gives for the one device there
+   is; func_attributes: calls of cudaFuncSetAttribute */
+int fake_device = -1;
+long func_attributes = 0;
+int cudaGetDevice(int* d) {
+    static int (*f)(int*);
+    if (!f) f = (int (*)(int*))real("cudaGetDevice");
+    const int e = f(d);
+    if (fake_device >= 0) *d = fake_device;
+    return e;
+}
+int cudaDeviceGetAttribute(int* v, int attr, int dev) {
+    static int (*f)(int*, int, int);
+    if (!f) f = (int (*)(int*, int, int))real("cudaDeviceGetAttribute");
+    return f(v, attr, fake_device >= 0 && dev == fake_device ? 0 : dev);
+}
+int cudaFuncSetAttribute(const void* fn, int attr, int v) {
+    static int (*f)(const void*, int, int);
+    if (!f) f = (int (*)(const void*, int, int))real("cudaFuncSetAttribute");
+    ++func_attributes;
+    return f(fn, attr, v);
+}
 """
 
 
