@@ -753,7 +753,7 @@ struct Adjoint {
         arena_top += (k + 1) & ~1;
         return p;
     }
-    // conj(x_k)^T y_k for up to 8 pairs into device scalars (no synchronisation)
+    // conj(x_k)^T y_k for up to ADOTS pairs into device scalars (no synchronisation)
     double2* dots(int l, std::vector<std::pair<const double2*, const double2*>> pr, const DotTail& tail = DotTail()) {
         AdjLevel& L = lv[l];
         const int np = (int)pr.size();
@@ -1315,8 +1315,9 @@ extern "C" int mg_cycle_backward(mg_handle* h, const void* u0, const void* g, in
     // ---- reverse sweep: every instance on a stream of its own.  The sweep
     // has no host synchronisation, so one step of an instance is a fixed
     // launch sequence on fixed buffers: the first step runs eagerly (it fills
-    // the vector pools), the next is captured into a CUDA graph, and the other
-    // K - 2 steps replay it.  The instances' streams run concurrently.
+    // the vector pools); where it pays (replay below) the step is then captured
+    // into a CUDA graph, which the other K - 1 steps replay.  The instances'
+    // streams run concurrently.
     std::vector<cudaStream_t> ss(ni, nullptr);
     std::vector<std::unique_ptr<Adjoint>> adj(ni);
     std::vector<cudaGraphExec_t> gexec(ni, nullptr);
@@ -1374,10 +1375,15 @@ extern "C" int mg_cycle_backward(mg_handle* h, const void* u0, const void* g, in
         A.reset();
         return rs ? rs : A.err;
     };
-    // first step of every instance (eager), then the captured step; below four
-    // cycles the remaining steps run eagerly too (capturing and instantiating
-    // a step costs more than emitting it twice)
-    const bool replay = K >= 4;
+    // First step of every instance (eager), then the captured step.  The host
+    // captures and instantiates one instance's step while its first step runs
+    // on the GPU, and replaying it is faster than emitting it again; of several
+    // instances only the last one's capture is hidden, while emitting keeps all
+    // streams busy.  n = 255, M = 8, emitted or replayed: one instance K = 2
+    // 22.2 or 21.0 ms, K = 3 32.1 or 29.1; four K = 2 47.2 or 58.3, K = 3 56.3 or
+    // 63.4; eight K = 2 84.7 or 107, K = 3 100 or 116 (n = 127, M = 2: one 5.2 or
+    // 4.9 and 7.6 or 6.6; eight 18.3 or 21.1 and 21.7 or 23.0).
+    const bool replay = K >= (ni == 1 ? 2 : 4);
     for (int b = 0; b < ni && !rc; ++b) {
         const size_t bytes = sizeof(double2) * H.inst[b].lv[0].slot_stride;
         cudaMemcpyAsync(bf[b].uin, ck[b][K - 1], bytes, cudaMemcpyDeviceToDevice, ss[b]);
