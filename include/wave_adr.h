@@ -112,9 +112,9 @@ typedef struct mg_params {
     int tail_nmax;          /* ADR levels l >= 3 with max(n_l, ny_l) <= tail_nmax and everything below them form
                                the coarse tail of an instance, run as one cluster launch (see tail_cluster); where
                                the level of the ADR corrections itself is within the bound, all M corrections are
-                               one launch; 0 = off; -1 (default): for a handle of up to 8 instances levels of
-                               at most 128 x 128 (mixed) or 64 x 64 (FP64) nodes, else off (measured fastest
-                               on this GPU).  The same bound, when set, selects the wave-cycle levels l >= 4
+                               one launch; 0 = off; -1 (default): levels of at most 128 x 128 (mixed) or 64 x 64
+                               (FP64) nodes for a handle of as many instances as clusters run at once (7 on
+                               this GPU), else off (measured fastest).  The same bound, when set, selects the wave-cycle levels l >= 4
                                that run as a shared-memory tail (Chebyshev smoothing and transfers in one block
                                per instance, at most 64 columns); -1: n_l <= 64 */
     int pdl;                /* 1: kernels are launched with programmatic dependent launch (a kernel's

@@ -639,9 +639,9 @@ struct Engine : EngineBase {
         }, t.pts);
     }
 
-    // Cluster form of the coarse ADR levels (tail_cluster.cuh): blocks per
-    // cluster, 16 where the GPU can place such a cluster with the most shared
-    // memory a block may ask for, else 8, else 0 (per-level launches).
+    // Cluster form of the coarse ADR levels (tail_cluster.cuh): clusters of CS
+    // blocks that the GPU runs at once with the most shared memory a block may
+    // ask for.
     template <int CS> static int ct_try(long long limit) {
         auto kern = k_adr_cluster<T, CS>;
         if (CS > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
@@ -651,7 +651,7 @@ struct Engine : EngineBase {
         cudaLaunchAttribute at[2];
         ct_config(cfg, at, CS, 1, limit, nullptr);
         int nc = 0;
-        return cudaOccupancyMaxActiveClusters(&nc, kern, &cfg) == cudaSuccess && nc > 0 ? CS : 0;
+        return cudaOccupancyMaxActiveClusters(&nc, kern, &cfg) == cudaSuccess ? nc : 0;
     }
     static void ct_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, int cs, unsigned clusters, long long smem,
                           cudaStream_t st) {
@@ -676,15 +676,18 @@ struct Engine : EngineBase {
             return std::max(0LL, (long long)smem_optin(dev) - (long long)std::max(a.sharedSizeBytes, b.sharedSizeBytes));
         });
     }
-    static int ct_cluster() {
-        static PerDevice<int> cs;
-        return (int)cs.get(0, [](int) {
-            int c = ct_try<16>(ct_smem_limit());
-            if (!c) c = ct_try<8>(ct_smem_limit());
+    static int ct_slots(int cs) {
+        static PerDevice<int> slots;
+        return (int)slots.get(cs, [cs](int) {
+            const int c = cs == 16 ? ct_try<16>(ct_smem_limit()) : ct_try<8>(ct_smem_limit());
             cudaGetLastError();
             return c;
         });
     }
+    // Blocks per cluster: 16 where the GPU can place such a cluster, else 8,
+    // else 0 (per-level launches).
+    static int ct_cluster() { return ct_slots(16) > 0 ? 16 : ct_slots(8) > 0 ? 8 : 0; }
+    int tail_slots() override { return ct_cluster() ? ct_slots(ct_cluster()) : 0; }
     // Levels l .. L of instance b fit one cluster (whole: with the iterate of
     // the ADR corrections).
     static bool ct_fits(Handle& H, int b, int l, bool whole) {

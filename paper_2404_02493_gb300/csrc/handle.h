@@ -206,6 +206,8 @@ struct EngineBase {
     virtual int level_op(Handle& H, int inst, int level, int what, int a0, int a1, cudaStream_t st) = 0;
     // halo-tile autotuner of the ADR launches (fills Handle::tiles)
     virtual int autotune(Handle& H, cudaStream_t st) = 0;
+    // instances whose coarse ADR tails the current device runs at once
+    virtual int tail_slots() = 0;
     // undo what an emission that ended in an exception left set
     virtual void abandon(Handle& H) = 0;
 };

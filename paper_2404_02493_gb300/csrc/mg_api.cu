@@ -1001,16 +1001,22 @@ int mg_setup(mg_handle** out, const mg_instance* inst, int ninst, const mg_param
     mg_handle* mh = new mg_handle();
     mh->H.p = *p;
     mh->H.alloc_limit = p->workspace_limit;
+    mh->eng = (p->precision == MG_PREC_FP64) ? make_engine_f64() : make_engine_f32();
     // automatic coarse tail (one cluster per instance, tail_cluster.cuh), by
-    // nodes, for as many instances as clusters fit the GPU at once: levels of up
-    // to 128 x 128 nodes in FP32, where a launch costs more than its work, 64 x
-    // 64 in FP64, whose arithmetic wants all SMs above that; with more
-    // instances the per-level launches spread the work over more SMs
-    // the wave-cycle tail (tail_wave.cuh) follows an explicit tail_nmax;
+    // nodes, for as many instances as clusters fit the GPU at once (7 of 16
+    // blocks here): levels of up to 128 x 128 nodes in FP32, where a launch costs
+    // more than its work, 64 x 64 in FP64, whose arithmetic wants all SMs above
+    // that.  One instance more is a second wave of clusters, and the per-level
+    // launches, which spread the work over all SMs, are as fast or faster.
+    // Cycle, M = 2, tail or per level, 7 instances | 8: FP32 n = 127 107 or 151 |
+    // 152 or 153 us, 255 178 or 247 | 254 or 251, 511 376 or 453 | 463 or 471; FP64
+    // n = 127 408 or 465 | 612 or 467, 255 967 or 1045 | 1194 or 1078, 511 2613 or
+    // 2698 | 3097 or 2985.
+    // The wave-cycle tail (tail_wave.cuh) follows an explicit tail_nmax;
     // automatic: what one block takes (64 columns)
     mh->H.wave_tail_nmax = mh->H.p.tail_nmax >= 0 ? mh->H.p.tail_nmax : 64;
     mh->H.tail_nodes = mh->H.p.tail_nmax >= 0 ? (1ll << 40) : (p->precision == MG_PREC_FP64 ? 64 * 64 : 128 * 128);
-    if (mh->H.p.tail_nmax < 0) mh->H.p.tail_nmax = ninst <= 8 ? (1 << 30) : 0;
+    if (mh->H.p.tail_nmax < 0) mh->H.p.tail_nmax = ninst <= mh->eng->tail_slots() ? (1 << 30) : 0;
     // the two tails follow the index roles: with a role list every level has
     // its own launches
     if (roles_set(*p)) {
@@ -1019,7 +1025,6 @@ int mg_setup(mg_handle** out, const mg_instance* inst, int ninst, const mg_param
     }
     for (int l = 2; l <= MG_MAX_LEVELS; ++l) mh->H.roles[l - 1] = level_role(l, MG_MAX_LEVELS + 1, *p);
     mh->H.prec = p->precision;
-    mh->eng = (p->precision == MG_PREC_FP64) ? make_engine_f64() : make_engine_f32();
     // k and phi may be host memory: stage them on the device for the setup kernels
     std::vector<mg_instance> staged(inst, inst + ninst);
     std::vector<void*> tmp;

@@ -68,6 +68,15 @@ int cudaDeviceGetAttribute(int* v, int attr, int dev) {
     if (!f) f = (int (*)(int*, int, int))real("cudaDeviceGetAttribute");
     return f(v, attr, fake_device >= 0 && dev == fake_device ? 0 : dev);
 }
+/* fake_clusters >= 0: the clusters that run at once */
+int fake_clusters = -1;
+int cudaOccupancyMaxActiveClusters(int* n, const void* fn, const void* cfg) {
+    static int (*f)(int*, const void*, const void*);
+    if (!f) f = (int (*)(int*, const void*, const void*))real("cudaOccupancyMaxActiveClusters");
+    const int e = f(n, fn, cfg);
+    if (fake_clusters >= 0) *n = fake_clusters;
+    return e;
+}
 int cudaFuncSetAttribute(const void* fn, int attr, int v) {
     static int (*f)(const void*, int, int);
     if (!f) f = (int (*)(const void*, int, int))real("cudaFuncSetAttribute");
