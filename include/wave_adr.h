@@ -35,7 +35,7 @@
  * or host memory (pageable or pinned); host memory is staged through the
  * handle's workspace with copies on `stream`.  The caller owns every
  * pointer it passes; the handle owns its workspace (levels, coefficient
- * fields, coarsest-level factors), allocated in mg_setup and freed by
+ * fields, coarsest-level inverses), allocated in mg_setup and freed by
  * mg_destroy.
  *
  * Errors: functions return MG_OK (0) or a negative MG_E* code; the text of
@@ -93,7 +93,8 @@ typedef struct mg_params {
                                level 1 inside FGMRES, into the basis-vector reads and the matvec); with more
                                the sweeps are passes of their own */
     int cheb_iters;         /* 5 (<= 16) */
-    int coarse;             /* MG_COARSE_LU (dense FP64 LU) | MG_COARSE_CHEB (Algorithm 1, q=10) */
+    int coarse;             /* MG_COARSE_LU (direct: dense inverse, formed in FP64) | MG_COARSE_CHEB
+                               (Algorithm 1, q=10) */
     int coarse_cheb_iters;  /* 10 */
     int M;                  /* ADR corrections at level 2 (8) */
     int adr;                /* 1: Wave-ADR cycle; 0: plain wave cycle */
@@ -116,7 +117,8 @@ typedef struct mg_params {
                                (FP64) nodes for a handle of as many instances as clusters run at once (7 on
                                this GPU), else off (measured fastest).  The same bound, when set, selects the wave-cycle levels l >= 4
                                that run as a shared-memory tail (Chebyshev smoothing and transfers in one block
-                               per instance, at most 64 columns); -1: n_l <= 64 */
+                               per instance, at most 64 columns and 64 rows (mixed) or 32 rows (FP64));
+                               -1: all that fit */
     int pdl;                /* 1: kernels are launched with programmatic dependent launch (a kernel's
                                descriptor prologue overlaps its predecessor); 0 (default): plain launches
                                (measured 0.1 ms per n=4095 cycle faster on this GPU) */
@@ -208,18 +210,19 @@ const char* mg_last_error(void);
  * and exp(i omega phi) at level 2 are formed in FP64, the Chebyshev interval
  * [lambda_max/alpha, lambda_max] (Section 3.1.1) is set from the Gershgorin
  * bound and the spectral alpha rule, and the coarsest Helmholtz and ADR
- * operators are factored by a device-side dense FP64 LU with partial
- * pivoting.  Synchronises `stream`.  Errors: MG_EINVAL (max(n, ny) <= n_cmax,
+ * operators are inverted on the device (dense FP64 Gauss-Jordan elimination
+ * with partial pivoting).  Synchronises `stream`.  Errors: MG_EINVAL (max(n, ny) <= n_cmax,
  * coarsest level of more than 1024 nodes or with a side below 2, omega <= 0,
- * null pointers, non-finite k or phi), MG_ENOMEM, MG_ECUDA.  Handles with a
- * non-square instance run every level with its own launches (the coarse and
- * wave tails are for square levels). */
+ * null pointers, non-finite k or phi), MG_ENOMEM, MG_ECUDA. */
 int mg_setup(mg_handle** h, const mg_instance* inst, int ninst, const mg_params* p, mg_stream stream);
 
 /* u <- cycle^ncycles(u, g) (Algorithm 1 from level 1), in the handle's cycle
  * precision (complex128 for FP64 handles, complex64 for MIXED handles).
  * u: in/out, g: in; dense concatenated layout.  Asynchronous on `stream`
- * when both pointers are device memory. */
+ * when both pointers are device memory: the first such call of a handle
+ * builds its launch tables (allocations and small synchronous copies), the
+ * second captures the cycle into a CUDA graph before it is queued (host work,
+ * 0.1 to 0.2 ms for the sizes of the tests), and every later call replays it. */
 int mg_cycle(mg_handle* h, void* u, const void* g, int ncycles, mg_stream stream);
 
 /* Solve A u = g to ||g - A u|| / ||g|| < p->tol with the outer iteration
@@ -238,7 +241,9 @@ int mg_solve(mg_handle* h, void* u, const void* g, mg_solve_info* info, mg_strea
 /* Building blocks of mg_solve for callers that drive the outer iteration
  * themselves (and for timing exactly K steps).
  * mg_solve_begin: load the complex128 initial guess u and right-hand side g
- *   and compute r = g - A u, ||r||, ||g|| in FP64 (asynchronous).
+ *   and compute r = g - A u, ||r||, ||g|| in FP64 (asynchronous, but for the
+ *   first call of a handle with use_graph, which waits for `stream`, runs a
+ *   step on the workspace and captures it).
  * mg_solve_steps: `nsteps` iterative-refinement steps
  *   u <- u + ||r|| cycle(0, r/||r||), each followed by the FP64 residual
  *   (Section 4.3.1 uses the cycle as the preconditioner of the outer
@@ -309,8 +314,8 @@ int mg_profile_records(mg_handle* h, int nsteps, int* kind, long long* pts, doub
 /* Level roles (Algorithm 1): MG_ROLE_JACOBI (level 1: damped Jacobi),
  * MG_ROLE_CHEB_ADR (level 2: Chebyshev, then the M ADR corrections),
  * MG_ROLE_NONE (level 3: no smoothing, Section 3.1.3), MG_ROLE_CHEB (levels
- * >= 4: Chebyshev), MG_ROLE_COARSE_LU / MG_ROLE_COARSE_CHEB (level L: dense
- * FP64 LU, or Algorithm 1's q = 10 Chebyshev steps). */
+ * >= 4: Chebyshev), MG_ROLE_COARSE_LU / MG_ROLE_COARSE_CHEB (level L: the
+ * dense inverse, or Algorithm 1's q = 10 Chebyshev steps). */
 enum { MG_ROLE_JACOBI = 0, MG_ROLE_CHEB = 1, MG_ROLE_NONE = 2, MG_ROLE_CHEB_ADR = 3, MG_ROLE_COARSE_LU = 4,
        MG_ROLE_COARSE_CHEB = 5 };
 /* The hierarchy mg_setup builds for an n x n instance with the schedule p,
@@ -370,7 +375,7 @@ int mg_adr_vcycle(mg_handle* h, int inst, const void* b, void* a, mg_stream stre
  * (Algorithm 1, post-smoothing on level 2). */
 int mg_adr_correction(mg_handle* h, int inst, void* u, const void* g, mg_stream stream);
 /* x = A_L^{-1} b (which = 0, Helmholtz) or L_L^{-1} b (which = 1, ADR) on
- * the coarsest level, with the dense FP64 LU factors. */
+ * the coarsest level, with the dense inverse (formed in FP64). */
 int mg_coarse_solve(mg_handle* h, int inst, int which, const void* b, void* x, mg_stream stream);
 
 /* Halo-tile shapes used by the ADR GMRES(3) kernels of `level` (2 <= level
@@ -443,8 +448,8 @@ int mg_eikonal_rect(int n, int ny, const double* s, double x0, double y0, double
  * are DEVICE pointers, dense row-major; the call is asynchronous on
  * `stream`.
  *
- * Scratch: 1216 complex partial sums and a counter held in fixed
- * __device__ arrays of the library (about 20 KB, kept by every GPU that
+ * Scratch: 760 partial sums and a counter held in fixed
+ * __device__ arrays of the library (about 6 KB, kept by every GPU that
  * loads the library until the process exits).  The grid size does not
  * change the scratch; n must be in 1..32768 (MG_EINVAL otherwise).  The
  * first call on each device looks up the scratch's device address

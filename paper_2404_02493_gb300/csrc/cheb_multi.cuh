@@ -114,9 +114,9 @@ __global__ void __launch_bounds__(NT) k_cheb_multi(const __grid_constant__ KDesc
     }
 }
 
-// The same smoothing with the region in registers (wave_nodes.cuh): a block of
-// 1024 threads holds 64 columns of 16 RPT rows, of which all but 2q on each
-// side are its output tile (values on the outer ring go wrong by one node per
+// The same smoothing with the region in registers and the Laplacian as a sum of
+// differences (wave_nodes.cuh): a block of 1024 threads holds 64 columns of 16
+// RPT rows, of which all but 2q on each side are its output tile (values on the outer ring go wrong by one node per
 // stencil).  With every operand in shared memory, an in-grid test per node and
 // stage and 256 threads per region, k_cheb_multi is bound by issue slots and
 // barriers; here a stage is bound by its shared-memory loads, so that two rows

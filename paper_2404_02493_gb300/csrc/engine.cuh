@@ -593,7 +593,10 @@ struct Engine : EngineBase {
                 int arg = -1;
                 for (int c = 0; c < GS_NCAND; ++c) {
                     // (in FP64 a strip march, one warp's chain of rows on a pipe
-                    // of two lanes, takes 4 to 10 times a tile's time)
+                    // of two lanes, is never the fastest: best strip against best
+                    // tile 150 and 22 us for 31 x 31 and 63 x 63 nodes, 165 and 32 for
+                    // 255 x 255, 167 and 82 for 511 x 511, 291 and 254 for 1023 x
+                    // 1023, 992 and 938 for 2047 x 2047)
                     if (!kStream && w == 0 && gs_gram_streaming(c)) continue;
                     auto run = [&] {
                         if (w == 0) gs_gram(H, ds, c, SAB, st);
@@ -1047,7 +1050,12 @@ struct Engine : EngineBase {
     // fewer, larger chunks beat deeper rings of smaller ones (each chunk costs
     // a wait and a block barrier): with 3 x 69 KB, 4 x 46 KB and 5 x 35 KB
     // stages the two passes took 5%, 25% and 50% longer.
-    static FgGeom fg_geometry() { return FgGeom{(int)(4096 / sizeof(cplx<T>)), 2}; }
+    // The stages also take the threads' sums at the end of a pass.
+    static FgGeom fg_geometry() {
+        constexpr int pw = (int)(4096 / sizeof(cplx<T>)), ns = 2;
+        static_assert(ns * (MAXR + 1) * pw >= 2 * MAXR * NT, "sums of a pass");
+        return FgGeom{pw, ns};
+    }
 
     // One inner iteration: z_j = cycle(0, V_j), W = A z_j, CGS2 against
     // V_0..V_j, Hessenberg column and Givens rotation.

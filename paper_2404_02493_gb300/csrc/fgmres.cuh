@@ -607,7 +607,8 @@ __global__ void __launch_bounds__(NT, 1) k_fg_lag(const __grid_constant__ KDesc 
     });
     if (!ok) return;
     // the thread's values, [S1 (j) | S2 (j) | s3 | ||Vt||^2] or [||W1||^2],
-    // into the stage memory (2 MAXR + 2 values of NT threads fit a stage)
+    // into the stage memory (2 MAXR values of NT threads at most, j < MAXR: in
+    // FP32 one stage holds them, in FP64 they take both, see fg_geometry)
     const int nval = PASS == 0 ? 2 * jj + 2 : 1;
     cplx<TC>* const red = stg0;
     if (PASS == 0) {

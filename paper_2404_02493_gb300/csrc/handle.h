@@ -140,7 +140,8 @@ struct Handle {
     std::map<std::string, TileChoice> tiles;  // per ADR launch (desc_key), from the autotuner
     std::map<std::string, int*> tail_first;   // per coarse-tail launch: first-level descriptors (device)
     long long tail_nodes = 0;                  // coarse ADR tail: most nodes of a level (see mg_params.tail_nmax)
-    int wave_tail_nmax = 0;                    // wave-cycle levels l >= 4 with n_l <= this run as the shared-memory tail
+    int wave_tail_nmax = 0;                    // wave-cycle levels l >= 4 of at most this many columns and rows run as
+                                               // the shared-memory tail, where they fit (tail_wave.cuh)
     int roles[MAX_LEVELS] = {};                // effective role of level l (l >= 2, below an instance's coarsest)
     std::vector<void*> allocs;      // everything cudaMalloc'ed
     size_t alloc_bytes = 0;         // their total size

@@ -879,9 +879,8 @@ __global__ void __launch_bounds__(NT) k_resdemod(const __grid_constant__ KDesc A
 
 
 // ----------------------------------------------------------- coarsest level
-// x = A^{-1} b with the dense inverse formed at setup from the LU factors in
-// FP64 and stored in the cycle precision T (N = n ny <= 1024 rows).  The
-// complex-FP32 cycle applies it in FP32: FP64 arithmetic issues at a small
+// x = A^{-1} b with the dense inverse formed at setup in FP64 and stored in the
+// cycle precision T (N = n ny <= 1024 rows).  The complex-FP32 cycle applies it in FP32: FP64 arithmetic issues at a small
 // fraction of the FP32 rate on this GPU, and the rounding of the inverse
 // moves the cycle by about 1e-7 relative, below its own FP32 rounding.  One
 // warp per matrix row; the right-hand side is staged in shared memory.

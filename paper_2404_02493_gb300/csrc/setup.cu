@@ -489,7 +489,7 @@ int setup_coarse_inverses(const std::vector<CoarseJob>& jobs, cudaStream_t st) {
         }
         for (int v : info)
             if (v != 0) {
-                set_error("coarse LU: singular coarsest operator");
+                set_error("coarse inverse: singular coarsest operator");
                 return MG_EINVAL;
             }
         q0 = q1;

@@ -16,7 +16,7 @@
 //                result to the level's SU slot
 //
 // What bounds it: 20 dependent stencil passes per level in one block, each its
-// SM's shared-memory traffic and a barrier.  A thread owns WT_RPT rows of a
+// SM's shared-memory traffic and a barrier.  A thread owns wt_rpt() rows of a
 // column: x, d, g and the diagonal of its nodes stay in registers, north and
 // south neighbours inside its rows too, and the two shared vectors (x, the
 // residual t) have a zero border, so a pass loads 2.5 values per node and
@@ -25,8 +25,16 @@
 // chain followed pointer by pointer the two launches took 29 and 26 us for
 // levels of 63 and 31; now 21 and 19 us (of which ~5 are the launch and the first loads).
 //
-// Slots and per-node arithmetic are those of the multi-launch path
-// (k_cheb_step, k_restrict<MODE_HELM>, k_prolong<PMODE_ADD>); the Chebyshev
+// In FP64 the four rows a thread would need for 64 rows do not fit its
+// registers (a complex value takes four), so a level of more than 32 rows keeps
+// its launches, which also spread the FP64 work over all SMs: with a tail that
+// took levels up to 51 x 51 in shared memory an FGMRES step without ADR
+// corrections ran 702 us at n = 264 (level of 33), 917 at n = 400 (50), 1277 at n =
+// 700 (43), with those levels per launch 592, 695 and 1107 us.
+//
+// Slots are those of the multi-launch path (k_cheb_step, k_restrict<MODE_HELM>,
+// k_prolong<PMODE_ADD>) and in FP64 its per-node arithmetic; in FP32 the
+// Laplacian is a sum of differences (wave_nodes.cuh).  The Chebyshev
 // direction lives in registers only (the first step of a smoothing does not
 // read it).  Only block barriers are used; every thread runs the same level
 // loop.
