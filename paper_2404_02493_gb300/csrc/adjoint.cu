@@ -1390,18 +1390,25 @@ extern "C" int mg_cycle_backward(mg_handle* h, const void* u0, const void* g, in
         rc = step(b);
     }
     for (int b = 0; b < ni && !rc && replay; ++b) {
+        // (an instance whose step cannot be captured goes on emitting it)
         cudaGraph_t gr = nullptr;
-        if (cudaStreamBeginCapture(ss[b], cudaStreamCaptureModeRelaxed) != cudaSuccess) { rc = MG_ECUDA; break; }
-        rc = step(b);
-        if (cudaStreamEndCapture(ss[b], &gr) != cudaSuccess || !gr) { rc = rc ? rc : MG_ECUDA; break; }
-        if (!rc && cudaGraphInstantiate(&gexec[b], gr, 0) != cudaSuccess) rc = MG_ECUDA;
-        cudaGraphDestroy(gr);
+        bool ok = cudaStreamBeginCapture(ss[b], cudaStreamCaptureModeRelaxed) == cudaSuccess;
+        if (ok) {
+            rc = step(b);
+            ok = cudaStreamEndCapture(ss[b], &gr) == cudaSuccess && gr &&
+                 cudaGraphInstantiate(&gexec[b], gr, 0) == cudaSuccess;
+            if (gr) cudaGraphDestroy(gr);
+        }
+        if (!ok) {
+            gexec[b] = nullptr;
+            cudaGetLastError();
+        }
     }
     for (int k = K - 2; k >= 0 && !rc; --k)
         for (int b = 0; b < ni; ++b) {
             const size_t bytes = sizeof(double2) * H.inst[b].lv[0].slot_stride;
             cudaMemcpyAsync(bf[b].uin, ck[b][k], bytes, cudaMemcpyDeviceToDevice, ss[b]);
-            if (!replay) {
+            if (!gexec[b]) {
                 if ((rc = step(b)) != MG_OK) break;
             } else if (cudaGraphLaunch(gexec[b], ss[b]) != cudaSuccess) {
                 rc = MG_ECUDA;

@@ -9,6 +9,7 @@ import numpy as np
 import pytest
 
 import synth
+from fake_runtime import run
 from gpu_util import lib_handle, rel, rnd
 from paper_2404_02493_gb300 import binding as B
 
@@ -37,3 +38,36 @@ def test_gradients_of_many_cycles(sizes, K):
     assert rel(gu, bar) < 1e-12
     assert rel(gphi, rphi) < 1e-12
     assert rel(gw, rw) < 1e-12
+
+
+@pytest.mark.parametrize("which", [1, 2, 3])
+def test_steps_are_emitted_where_the_capture_fails(tmp_path, which):
+    """(a stand-in for the failing call, on the host)"""
+    out = run(tmp_path, """
+        import numpy as np
+        import synth
+        from gpu_util import lib_handle, rnd
+        from paper_2404_02493_gb300 import binding as B
+
+        insts = [synth.config_lognormal(n=n, omega=0.3 * (n + 1), seed=n) for n in (47, 63)]
+        N = sum(I.n * I.n for I in insts)
+        h = lib_handle(insts, "fp64", M=2, n_cmax=7, autotune=0)
+        fake = ctypes.c_int.in_dll(lib, "fake_capture")
+        refused = ctypes.c_int.in_dll(lib, "fake_captures_refused")
+
+        def gradients():
+            gphi, gw, gu = np.zeros(N), np.zeros(2 * B.MG_MAX_LEVELS), np.zeros(N, complex)
+            B.mg_cycle_backward(h, rnd((N,), 3), rnd((N,), 1), 4, rnd((N,), 2), gphi, gw, gu)
+            return gphi, gw, gu
+
+        want = gradients()
+        assert refused.value == 0
+        fake.value = %d
+        got = gradients()
+        fake.value = 0
+        assert refused.value == 2
+        assert all(np.array_equal(a, b) for a, b in zip(want, got))
+        B.mg_destroy(h)
+        print("passed")
+    """ % which)
+    assert "passed" in out
